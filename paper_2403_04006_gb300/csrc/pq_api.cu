@@ -18,6 +18,7 @@
 #include <numeric>
 #include <queue>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include "../../include/pq.h"
@@ -279,14 +280,69 @@ static CutCost forward_cut_cost(const ItemPlan& it)
     return cc;
 }
 
+// Items that any cut treats alike: the same number of summed rows, column
+// multiplicities and radices.  A batch holds few such groups (4096 patterns of
+// 12 photons: about 60; the 65536-permanent ragged batch: about 9000) and
+// searching the sub-multisets of the digits is most of a plan's time, so a
+// plan cuts one item of each group and applies the cut to the others.
+struct Cut {
+    int J = 0;
+    int64_t L = 1;
+    std::vector<int> low_count;  // digits of each radix that go low; empty: a prefix
+};
+
+struct ItemGroups {
+    std::vector<int32_t> of;      // group of each item (-1: trivial)
+    std::vector<ItemPlan> first;  // one item of each group
+    std::vector<int64_t> count;
+    std::vector<Cut> cut;
+    explicit ItemGroups(const std::vector<ItemPlan>& items)
+    {
+        std::unordered_map<std::string, int32_t> known;
+        std::string key;
+        of.assign(items.size(), -1);
+        for (size_t p = 0; p < items.size(); ++p) {
+            const ItemPlan& it = items[p];
+            if (it.trivial)
+                continue;
+            key.clear();
+            key.push_back((char)it.k);
+            for (int c : it.cmul)
+                key.push_back((char)c);
+            key.push_back(0);
+            for (int r : it.drad)  // in ascending order
+                key.push_back((char)r);
+            const auto at = known.emplace(key, (int32_t)first.size());
+            if (at.second) {
+                first.push_back(it);
+                count.push_back(0);
+            }
+            of[p] = at.first->second;
+            ++count[of[p]];
+        }
+        cut.resize(first.size());
+    }
+};
+
+static void finish_cut(ItemPlan& it, int J, int64_t L)
+{
+    it.J = J;
+    it.L = L;
+    it.nchunks = it.T / L;
+    it.weighted = false;
+    for (int d = 0; d < J; ++d)
+        if (it.drad[d] > 2)
+            it.weighted = true;
+}
+
 // Cut the item's code into chunks of the lowest digits: the longest prefix of
 // digits whose radix product stays within the target length.  With reorder
 // (batched plans), the low digits may be any sub-multiset of the digits, not
 // only a prefix of the ascending list; see below.  cc: the kernel's costs
-// (default: the forward's).
+// (default: the forward's).  out: receives the cut, for apply_cut.
 static void choose_chunks(ItemPlan& it, int log2_cap, int jmax = kMaxLowDigits,
                           int64_t min_chunks = kWarp, bool reorder = false,
-                          const CutCost* cc = nullptr)
+                          const CutCost* cc = nullptr, Cut* out = nullptr)
 {
     if (it.trivial) {
         it.J = 0;
@@ -296,6 +352,7 @@ static void choose_chunks(ItemPlan& it, int log2_cap, int jmax = kMaxLowDigits,
     }
     if (reorder)  // start from the ascending order, whatever an earlier cut chose
         order_digits(it, {});
+    std::vector<int> low_count;  // of a cut that is not a prefix
     int64_t target = it.T / min_chunks;  // aim for at least min_chunks chunks
     int64_t cap = int64_t(1) << std::max(0, std::min(log2_cap, 30));
     if (target > cap)
@@ -404,7 +461,7 @@ static void choose_chunks(ItemPlan& it, int log2_cap, int jmax = kMaxLowDigits,
             };
             dfs(0, 0, 1);
             if (!bestc.empty()) {
-                std::vector<int> low_count(kMaxLowRadix + 1, 0);
+                low_count.assign(kMaxLowRadix + 1, 0);
                 J = 0;
                 L = 1;
                 for (size_t i = 0; i < vals.size(); ++i) {
@@ -417,13 +474,16 @@ static void choose_chunks(ItemPlan& it, int log2_cap, int jmax = kMaxLowDigits,
             }
         }
     }
-    it.J = J;
-    it.L = L;
-    it.nchunks = it.T / L;
-    it.weighted = false;
-    for (int d = 0; d < J; ++d)
-        if (it.drad[d] > 2)
-            it.weighted = true;
+    if (out)
+        *out = Cut{J, L, low_count};
+    finish_cut(it, J, L);
+}
+
+// The cut that choose_chunks (with reorder) made for an item of the same group.
+static void apply_cut(ItemPlan& it, const Cut& c)
+{
+    order_digits(it, c.low_count);
+    finish_cut(it, c.J, c.L);
 }
 
 static double fwd_flops_per_term(const ItemPlan& it)
@@ -654,16 +714,21 @@ static int schedule_and_upload(pq_plan* P)
         // task is a quarter of a share).  Chunk lengths that the caller fixed
         // are kept as they are.
         const double warps = (double)P->blocks * P->wpb;
+        for (ItemPlan& it : P->items)  // an earlier cut may have reordered the digits
+            if (!it.trivial && !std::is_sorted(it.drad.begin(), it.drad.end()))
+                order_digits(it, {});
+        ItemGroups groups(P->items);
         auto cut_all = [&](int gcap) {
             double total = 0.0, longest = 0.0;
-            for (ItemPlan& it : P->items) {
+            for (size_t g = 0; g < groups.first.size(); ++g) {
+                ItemPlan& it = groups.first[g];
                 const int e = explicit_log2_for(P, it);
-                choose_chunks(it, e > 0 ? e : std::min(10, gcap), kMaxLowDigits, kWarp, true);
-                if (it.trivial)
-                    continue;
+                choose_chunks(it, e > 0 ? e : std::min(10, gcap), kMaxLowDigits, kWarp, true,
+                              nullptr, &groups.cut[g]);
                 const double cost = (double)it.L * fwd_flops_per_term(it) +
                                     2.0 * (double)((int)it.drow.size() - it.J) * it.l + 2.0 * it.l;
-                total += cost * (double)((it.nchunks + kWarp - 1) / kWarp);
+                total += (double)groups.count[g] * cost *
+                         (double)((it.nchunks + kWarp - 1) / kWarp);
                 longest = std::max(longest, cost);
             }
             return total > 0.0 ? longest / (total / warps) : 0.0;
@@ -675,6 +740,13 @@ static int schedule_and_upload(pq_plan* P)
                 gcap = c;
                 ratio = cut_all(gcap);
             }
+        }
+        for (int64_t p = 0; p < np; ++p) {
+            ItemPlan& it = P->items[p];
+            if (it.trivial)
+                choose_chunks(it, 10);
+            else
+                apply_cut(it, groups.cut[groups.of[p]]);
         }
     }
 
@@ -1474,27 +1546,35 @@ static int ensure_backward(pq_plan* P)
     // short chunks to fill the GPU: it keeps caps of 2^4 terms (the ragged
     // batch's plain backward took 5.9 s with them, 17.7 s with 2^7).
     const int cap0 = P->opts.method == PQ_METHOD_PLAIN ? 4 : kBwdChunkLog2;
-    std::vector<int> cls_cap(ncls, cap0);
-    for (int c = 0; c < ncls && cap0 > 4; ++c) {
+    for (ItemPlan& it : items)
+        if (!it.trivial && !std::is_sorted(it.drad.begin(), it.drad.end()))
+            order_digits(it, {});
+    ItemGroups groups(items);
+    std::vector<std::vector<int32_t>> cls_groups(ncls);
+    for (size_t g = 0; g < groups.first.size(); ++g) {
+        int c = 0;
+        while (c + 1 < ncls && kBwdClassLd[c] < groups.first[g].l)
+            ++c;
+        cls_groups[c].push_back((int32_t)g);
+    }
+    for (int c = 0; c < ncls; ++c) {
         if (!cls_used[c])
             continue;
         const BwdClass& C = cls[c];
         const double warps = (double)C.blocks * C.wpb;
         for (int cap = cap0; cap >= 4; --cap) {
             double total = 0.0, longest = 0.0;
-            for (int64_t p = 0; p < np; ++p) {
-                if (P->bwd_class_of[p] != c || items[p].trivial)
-                    continue;
-                ItemPlan it = items[p];
+            for (int32_t g : cls_groups[c]) {
+                ItemPlan& it = groups.first[g];
                 const CutCost bc = bwd_cut_cost(it, C);
-                choose_chunks(it, cap, std::max(C.jb, 1), kWarp, true, &bc);
+                choose_chunks(it, cap, std::max(C.jb, 1), kWarp, true, &bc, &groups.cut[g]);
                 const double task = (double)it.L * bc.per_term +
                                     ((int)it.drad.size() - it.J) * bc.per_high + bc.per_task +
                                     it.J * bc.per_task_low;
-                total += task * (double)((it.nchunks + kWarp - 1) / kWarp);
+                total += (double)groups.count[g] * task *
+                         (double)((it.nchunks + kWarp - 1) / kWarp);
                 longest = std::max(longest, task);
             }
-            cls_cap[c] = cap;
             if (total <= 0.0 || longest <= 0.5 * total / warps)
                 break;
         }
@@ -1503,8 +1583,7 @@ static int ensure_backward(pq_plan* P)
         ItemPlan& it = items[p];
         const BwdClass& C = cls[P->bwd_class_of[p]];
         if (!it.trivial) {
-            const CutCost bc = bwd_cut_cost(it, C);
-            choose_chunks(it, cls_cap[P->bwd_class_of[p]], std::max(C.jb, 1), kWarp, true, &bc);
+            apply_cut(it, groups.cut[groups.of[p]]);
             const PermDesc& Df = P->desc_h[p];
             const int nd = (int)it.drow.size();
             int32_t* dig = meta_bwd.data() + Df.meta + 2 * Df.k + 2 * Df.l;
