@@ -3,155 +3,311 @@
 // Sampling"; Eq. (per_def) for the permanent, Eq. (BS_prob) for the
 // probabilities written by the final reduction).
 //
-// One thread walks one chunk of the Gray code.  On GB300 the FP64 pipe (1.68
-// lane operations per clock per SM, saturated by four warps whatever their
-// dependency chains) is the only resource the walk loads, so the kernel is
-// written to issue exactly the FP64 instructions the method needs and nothing
-// else into that pipe:
-//   * every lane's column sums S_j = sum_i (r_i - 2 g_i) b_ij live in shared
-//     memory, lane-major (one 16-byte complex per lane per column, so a warp
-//     access is conflict-free); the loops over columns are plain runtime loops,
-//     never unrolled against a bound and never if-converted, so no predicated-
-//     off or speculative FP64 instruction takes a pipe slot;
+// One thread walks one chunk of the Gray code.  The FP64 pipe (2 lane
+// operations per clock and SM) would bound the walk, so its column sums and
+// products are 64-bit block integers (pq_blockint.cuh) on the integer pipes:
+//   * a lane's column sums S_j = sum_i (r_i - 2 g_i) b_ij are scaled integers,
+//     in shared memory, lane-major (one 16-byte pair per lane per column, so a
+//     warp access is conflict-free), or in registers;
 //   * a Gray step changes one row's sign count by +-1 for all lanes at once:
-//     S_j += -+2 b_ij, one DFMA per real component, b read as a broadcast;
+//     S_j += -+2 b_ij, one 64-bit add per component, 2 b read as a broadcast;
+//     the shared-memory walk makes it in the loop that forms the next term;
 //   * product columns are sorted by non-increasing multiplicity, so
 //     prod_j S_j^{c_j} = prod_m P(n_m) with P(q) = S_0 ... S_{q-1}: l - 1
 //     complex products for P(l) plus one per extra prefix, instead of n - 1;
-//     the last product is fused into the running sum (four DFMA);
-//   * the sign (-1)^step alternates, so pairs of terms are unrolled with the
-//     sign folded into the DFMA operands; the binomial weight of the low
-//     digits changes only when a digit of radix > 2 moves, so a run of equally
-//     weighted terms is summed unweighted and weighted once (two DFMA);
+//     without repeated columns they are taken in pairs, p (S_j S_{j+1}),
+//     which halves the dependent chain;
+//   * a term is converted to FP64 and added to a running FP64 sum with its
+//     sign (-1)^step and its power of two in one DFMA per component; the
+//     binomial weight of the low digits changes only when a digit of radix > 2
+//     moves, so a run of equally weighted terms is summed unweighted and
+//     weighted once (two DFMA);
 //   * every 32 terms the FP64 running sum is folded into a double-double
 //     accumulator with TwoSum.
+// A base matrix with a non-finite entry, or a column whose bound overflows, has
+// no such scale: its tasks walk in FP64 (fp64_walk), so that infinities and
+// NaNs propagate as FP64 arithmetic gives them.
 // A warp task is up to 32 chunks of one permanent (one per lane).  The lanes'
 // sums are added exactly, in 128-bit integers (pq_fixsum.cuh), and the tasks
 // of one permanent in task order by the warp that finishes last, so results
 // do not depend on scheduling.
 #include <cuda_runtime.h>
 
+#include "../../include/pq.h"
+#include "pq_blockint.cuh"
 #include "pq_device.cuh"
 #include "pq_fixsum.cuh"
 #include "pq_kernels.h"
 
 namespace pqi {
 
-// Shared memory of one warp: base matrix (kmax x ld complex), base column sums
-// (ld complex), column sums of the 32 lanes (ld x 32 complex), low-digit rows
-// (16 ints), extra-factor counts (ld ints).
+// Shared memory of one warp: base matrix (kmax x ld pairs), base column sums
+// (ld pairs), the column sums of the 32 lanes (ld x 32 pairs; only the
+// shared-memory walk), low-digit rows (16 ints), extra-factor counts and scale
+// exponents (ld ints each).
 __host__ __device__ inline int warp_smem_bytes(int kmax, int ld)
 {
-    int bytes = (kmax * ld + ld + 32 * ld) * 16 + (16 + ld) * 4;
+    int bytes = (kmax * ld + ld + 32 * ld) * 16 + (16 + 2 * ld) * 4;
+    return (bytes + 15) & ~15;
+}
+
+__host__ __device__ inline int reg_warp_smem_bytes(int kmax, int ld)
+{
+    int bytes = (kmax * ld + ld) * 16 + (16 + 2 * ld) * 4;
     return (bytes + 15) & ~15;
 }
 
 struct WarpSmem {
-    double2* M;       // kmax x ld
-    double2* base;    // ld
-    double2* S;       // ld x 32, S[j * 32 + lane]
+    longlong2* M;     // kmax x ld: 2 b_ij scaled (b_ij itself, as doubles, for fp64_walk)
+    longlong2* base;  // ld: column sums at all digits zero (biased; doubles for fp64_walk)
+    longlong2* S;     // ld x 32, S[j * 32 + lane] (shared-memory walk)
     int32_t* lowrow;  // 16
     int32_t* ecnt;    // ld
+    int32_t* cexp;    // ld: scale exponent of each column
     int ld;
-    __device__ WarpSmem(unsigned char* raw, int kmax, int ld_)
+    __device__ WarpSmem(unsigned char* raw, int kmax, int ld_, bool sums)
     {
         ld = ld_;
-        M = reinterpret_cast<double2*>(raw);
+        M = reinterpret_cast<longlong2*>(raw);
         base = M + kmax * ld;
         S = base + ld;
-        lowrow = reinterpret_cast<int32_t*>(S + 32 * ld);
+        lowrow = reinterpret_cast<int32_t*>(S + (sums ? 32 * ld : 0));
         ecnt = lowrow + 16;
+        cexp = ecnt + ld;
     }
 };
 
-// Copy the oriented base matrix of permanent D into shared memory and form
-// base_j = sum_i r_i b_ij (all Gray digits at zero).
-template <class SM>
-__device__ void stage_perm(const ExecArgs& a, const PermDesc& D, const MetaView& mv, SM& sm,
-                           int lane)
+// What a warp keeps about the permanent it has staged.
+struct Staged {
+    int perm = -1;
+    int exp2 = 0;       // the terms' sum times 2^exp2 is the sum of prod_j S_j^{c_j}
+    uint32_t emask = 0; // bit j: column j < 32 has extra prefixes
+    bool fp64 = false;  // staged as doubles, for fp64_walk
+};
+
+__device__ __forceinline__ bool not_finite(double x)
+{
+    return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000;
+}
+
+// Copy the oriented base matrix of permanent D into shared memory as scaled
+// integers and form base_j = sum_i r_i b_ij (all Gray digits at zero).
+__device__ void stage_perm(const ExecArgs& a, const PermDesc& D, const MetaView& mv, WarpSmem& sm,
+                           Staged& st, int lane)
 {
     const int k = D.k, l = D.l;
+    double2* Md = reinterpret_cast<double2*>(sm.M);
+    bool bad = false;
     for (int e = lane; e < k * l; e += kWarp) {
         const int i = e / l, j = e - i * l;
         const int64_t off = D.src_off + (int64_t)mv.ridx[i] * D.si + (int64_t)mv.cidx[j] * D.sj;
-        sm.M[i * sm.ld + j] = a.src[off];
+        const double2 b = a.src[off];
+        bad = bad || not_finite(b.x) || not_finite(b.y);
+        Md[i * sm.ld + j] = b;
     }
     for (int d = lane; d < D.J; d += kWarp)
         sm.lowrow[d] = mv.drow[d];
     for (int j = lane; j < l; j += kWarp)
         sm.ecnt[j] = mv.ecnt[j];
     __syncwarp();
+    int xsum = 0;
     for (int j = lane; j < l; j += kWarp) {
-        double2 s = make_double2(0.0, 0.0);
+        uint32_t hmax = 0, units = 0;
         for (int i = 0; i < k; ++i) {
-            const double r = (double)mv.rmul[i];
-            const double2 b = sm.M[i * sm.ld + j];
-            s.x = __fma_rn(r, b.x, s.x);
-            s.y = __fma_rn(r, b.y, s.y);
+            const double2 b = Md[i * sm.ld + j];
+            hmax = max(hmax, bint_mag(b.x, b.y));
+        }
+        for (int i = 0; i < k; ++i) {
+            const double2 b = Md[i * sm.ld + j];
+            units += (uint32_t)mv.rmul[i] * bint_units(bint_mag(b.x, b.y), hmax);
+        }
+        int e = bint_scale(hmax, units);
+        if (hmax < 0x100000u) {
+            uint64_t sum = 0;
+            for (int i = 0; i < k; ++i) {
+                const double2 b = Md[i * sm.ld + j];
+                sum += (uint64_t)mv.rmul[i] * bint_mag_subnormal(b.x, b.y);
+            }
+            e = bint_scale_subnormal(sum);
+        }
+        bad = bad || e < kSumBits - 1024;  // the sums can overflow FP64
+        sm.cexp[j] = e;
+        xsum += mv.cmul[j] * e;
+    }
+    st.perm = -1;
+    st.fp64 = __any_sync(0xffffffffu, bad);
+    if (st.fp64) {
+        double2* base = reinterpret_cast<double2*>(sm.base);
+        for (int j = lane; j < l; j += kWarp) {
+            double2 s = make_double2(0.0, 0.0);
+            for (int i = 0; i < k; ++i) {
+                const double r = (double)mv.rmul[i];
+                const double2 b = Md[i * sm.ld + j];
+                s.x = __fma_rn(r, b.x, s.x);
+                s.y = __fma_rn(r, b.y, s.y);
+            }
+            base[j] = s;
+        }
+        st.exp2 = 0;
+        __syncwarp();
+        return;
+    }
+    __syncwarp();
+    for (int e = lane; e < k * l; e += kWarp) {
+        const int i = e / l, j = e - i * l;
+        const double2 b = Md[i * sm.ld + j];
+        const int x = sm.cexp[j];
+        sm.M[i * sm.ld + j] = make_longlong2(2 * bint_of(b.x, x), 2 * bint_of(b.y, x));
+    }
+    __syncwarp();
+    uint32_t em = 0;
+    for (int j = lane; j < l; j += kWarp) {
+        longlong2 s = make_longlong2(kSumBias, kSumBias);
+        for (int i = 0; i < k; ++i) {
+            const longlong2 b = sm.M[i * sm.ld + j];
+            s.x += mv.rmul[i] * (b.x >> 1);
+            s.y += mv.rmul[i] * (b.y >> 1);
         }
         sm.base[j] = s;
+        if (j < 32 && sm.ecnt[j] > 0)
+            em |= 1u << j;
     }
+    st.emask = __reduce_or_sync(0xffffffffu, em);
+    // n - 1 products, each shifted down by 64; the terms carry 2^-kSumBits
+    st.exp2 = kSumBits + 64 * (D.n - 1) - __reduce_add_sync(0xffffffffu, xsum);
     __syncwarp();
 }
 
-// One Glynn term: acc +-= prod_j S_j^{c_j} (S = this lane's column sums,
-// stride 32).  unit: every c_j = 1; jf: first column with an extra prefix.
-// The low-digit weight is applied by the caller, once per run of terms that
-// share it.
-template <bool NEG>
-__device__ __forceinline__ void glynn_term(const double2* S, int l, bool unit, int jf,
-                                           const int32_t* ecnt, double2& acc)
-{
-    if (unit) {
-        if (l == 1) {  // n = 1: the product is S_0 itself
-            acc.x = NEG ? __dsub_rn(acc.x, S[0].x) : __dadd_rn(acc.x, S[0].x);
-            acc.y = NEG ? __dsub_rn(acc.y, S[0].y) : __dadd_rn(acc.y, S[0].y);
-            return;
+// The column sums of one term, after its Gray step.  Shared memory: column j is
+// read, moved by the changed row's 2 b_j (STEP 1: the digit went up, 2: down,
+// 0: the chunk's first term) and written back as the term needs it.
+template <int STEP>
+struct SharedCols {
+    longlong2* S;        // this lane's, stride 32
+    const longlong2* b;  // the changed row
+    __device__ __forceinline__ longlong2 operator()(int j) const
+    {
+        longlong2 s = S[j * 32];
+        if (STEP != 0) {
+            const longlong2 d = b[j];
+            s.x = STEP == 1 ? s.x - d.x : s.x + d.x;
+            s.y = STEP == 1 ? s.y - d.y : s.y + d.y;
+            S[j * 32] = s;
         }
-        double2 p = S[0];
-#pragma unroll 1
-        for (int j = 1; j < l - 1; ++j)
-            p = cmul(p, S[j * 32]);
-        cfma_acc<NEG>(acc, p, S[(l - 1) * 32]);
-        return;
+        return s;
     }
-    // P(q) for q = 1 .. l in `pre`, extra prefixes multiplied into `ex`
-    double2 pre = S[0];
+};
+
+template <int NL>
+struct RegCols {
+    const longlong2 (&S)[NL];
+    __device__ __forceinline__ longlong2 operator()(int j) const { return S[j]; }
+};
+
+// prod_j S_j without repeated columns, 2^E times the integers returned: S_0 S_1,
+// then the columns in pairs, p (S_j S_{j+1}).  NL > 0: registers, unrolled,
+// l <= NL; NL = 0: shared memory.
+template <int NL, class Cols>
+__device__ __forceinline__ BInt unit_product(const Cols& col, int l, int& E)
+{
+    const longlong2 s0 = col(0);
+    if (l == 1)
+        return bint_plain(s0);
+    BInt p = bmul(sum_limbs(s0), sum_limbs(col(1)));
+    if constexpr (NL == 0) {
+        int j = 2;
 #pragma unroll 1
-    for (int j = 1; j <= jf; ++j)
-        pre = cmul(pre, S[j * 32]);
-    double2 ex = pre;
-#pragma unroll 1
-    for (int e = 1; e < ecnt[jf]; ++e)
-        ex = cmul(ex, pre);
-#pragma unroll 1
-    for (int j = jf + 1; j < l; ++j) {
-        pre = cmul(pre, S[j * 32]);
-#pragma unroll 1
-        for (int e = 0; e < ecnt[j]; ++e)
-            ex = cmul(ex, pre);
+        for (; j + 1 < l; j += 2) {
+            const BLimbs x = sum_limbs(col(j)), y = sum_limbs(col(j + 1));
+            const BInt q = bmul(x, y);
+            bnorm(p, E);
+            p = bmul(limbs(p), limbs(q));
+        }
+        if (j < l) {
+            bnorm(p, E);
+            p = bmul(limbs(p), sum_limbs(col(j)));
+        }
+    } else {
+#pragma unroll
+        for (int j = 2; j < NL; j += 2) {  // NL is even
+            if (j + 1 < l) {
+                const BInt q = bmul(sum_limbs(col(j)), sum_limbs(col(j + 1)));
+                bnorm(p, E);
+                p = bmul(limbs(p), limbs(q));
+            } else if (j < l) {
+                bnorm(p, E);
+                p = bmul(limbs(p), sum_limbs(col(j)));
+            }
+        }
     }
-    cfma_acc<NEG>(acc, pre, ex);
+    return p;
 }
 
-// One Gray step of the warp-uniform low walk: every lane's S += -+2 b_row.
-// Returns true when the changed digit has radix > 2, i.e. when the low-digit
-// weight prod_d C(top_d, g_d) changes (a radix-2 digit has weight C(1, g) = 1).
-__device__ __forceinline__ bool glynn_step(LowWalk& wk, const WarpSmem& sm, double2* S, int l)
+// Column j of a term with repeated columns: pre, the product of the columns so
+// far, is normalised at odd j and before it is used as an extra factor; at the
+// first column with extras (jf) ex starts as that prefix, and every further
+// extra multiplies it in (n_extra = ecnt[j] of them at column j).
+__device__ __forceinline__ void prefix_column(BInt& pre, int& E, BInt& ex, int& Ex, int j, int jf,
+                                              int n_extra)
 {
-    int up;
-    const int d = low_step(wk, up);
-    const double2* Mr = sm.M + sm.lowrow[d] * sm.ld;
-    const double delta = up > 0 ? -2.0 : 2.0;  // x = r - 2g
-#pragma unroll 1
-    for (int j = 0; j < l; ++j) {
-        const double2 b = Mr[j];
-        double2 s = S[j * 32];
-        s.x = __fma_rn(delta, b.x, s.x);
-        s.y = __fma_rn(delta, b.y, s.y);
-        S[j * 32] = s;
+    if ((j & 1) || n_extra > 0)
+        bnorm(pre, E);
+    if (n_extra == 0)
+        return;
+    const BLimbs lp = limbs(pre);
+    int e = 0;
+    if (j == jf) {
+        ex = pre;
+        Ex = E;
+        e = 1;
     }
-    return ((wk.radm1 >> (4 * d)) & 15u) > 1u;
+#pragma unroll 1
+    for (; e < n_extra; ++e) {
+        ex = bmul(limbs(ex), lp);
+        Ex += E;
+        bnorm(ex, Ex);
+    }
+}
+
+// prod_j S_j^{c_j} from the prefixes; jf < 0: no repeated column.
+template <int NL, class Cols>
+__device__ __forceinline__ BInt term_product(const Cols& col, int l, int jf, uint32_t emask,
+                                             const int32_t* ecnt, int& E)
+{
+    E = 0;
+    if (jf < 0)
+        return unit_product<NL>(col, l, E);
+    BInt pre = bint_plain(col(0)), ex = pre;
+    int Ex = 0;
+    if constexpr (NL == 0) {
+        prefix_column(pre, E, ex, Ex, 0, jf, ecnt[0]);
+#pragma unroll 1
+        for (int j = 1; j < l; ++j) {
+            pre = bmul(limbs(pre), sum_limbs(col(j)));
+            prefix_column(pre, E, ex, Ex, j, jf, ecnt[j]);
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < NL; ++j) {
+            if (j < l) {
+                if (j > 0)
+                    pre = bmul(limbs(pre), sum_limbs(col(j)));
+                prefix_column(pre, E, ex, Ex, j, jf, ((emask >> j) & 1u) ? ecnt[j] : 0);
+            }
+        }
+    }
+    E += Ex;
+    return bmul(limbs(pre), limbs(ex));
+}
+
+// acc +-= 2^(-kSumBits - E) p
+__device__ __forceinline__ void add_term(const BInt& p, int E, bool neg, double2& acc)
+{
+    const double f = bint_factor(E, neg);
+    const long long re = (long long)(((uint64_t)(uint32_t)p.rh << 32) | p.rl);
+    const long long im = (long long)(((uint64_t)(uint32_t)p.ih << 32) | p.il);
+    acc.x = __fma_rn(__ll2double_rn(re), f, acc.x);
+    acc.y = __fma_rn(__ll2double_rn(im), f, acc.y);
 }
 
 // A run of equally weighted terms ends: run += wlow * acc, and the walk's new
@@ -165,9 +321,9 @@ __device__ __forceinline__ void reweight(const LowWalk& wk, int J, double& wlow,
     wlow = (double)low_weight(wk, J);
 }
 
-// Write per = 2^{-(n-1)} * sum, and |per|^2 * norm; a sharded plan writes
-// its unscaled double-double sum instead.
-__device__ __forceinline__ void finalize(const ExecArgs& a, const PermDesc& D, dd2 v)
+// Write per = 2^{-(n-1)} * sum, and |per|^2 * norm, the sum being v 2^exp2; a
+// sharded plan writes its unscaled double-double sum instead.
+__device__ __forceinline__ void finalize(const ExecArgs& a, const PermDesc& D, dd2 v, int exp2)
 {
     if (a.out_partial) {
         double* o = a.out_partial + 4 * (int64_t)D.out;
@@ -175,10 +331,10 @@ __device__ __forceinline__ void finalize(const ExecArgs& a, const PermDesc& D, d
             o[0] = 1.0;
             o[1] = o[2] = o[3] = 0.0;
         } else {
-            o[0] = v.rh;
-            o[1] = v.rl;
-            o[2] = v.ih;
-            o[3] = v.il;
+            o[0] = scalbn(v.rh, exp2);
+            o[1] = scalbn(v.rl, exp2);
+            o[2] = scalbn(v.ih, exp2);
+            o[3] = scalbn(v.il, exp2);
         }
         return;
     }
@@ -189,9 +345,9 @@ __device__ __forceinline__ void finalize(const ExecArgs& a, const PermDesc& D, d
     } else {
         double h, e;
         fast_two_sum(v.rh, v.rl, h, e);
-        re = scalbn(h + e, 1 - D.n);
+        re = scalbn(h + e, exp2 + 1 - D.n);
         fast_two_sum(v.ih, v.il, h, e);
-        im = scalbn(h + e, 1 - D.n);
+        im = scalbn(h + e, exp2 + 1 - D.n);
     }
     if (a.out_amp)
         a.out_amp[D.out] = make_double2(re, im);
@@ -199,7 +355,6 @@ __device__ __forceinline__ void finalize(const ExecArgs& a, const PermDesc& D, d
         a.out_prob[D.out] = (re * re + im * im) * D.norm;
 }
 
-__device__ void combine_task(const ExecArgs& a, const Task& t, const PermDesc& D, dd2 res, int lane);
 
 // The task's sum: every lane's chunk sum (rh + rl, ih + il) times its
 // high-digit weight (-1)^neg whigh_u (zero for a lane without a chunk), added
@@ -232,118 +387,15 @@ __device__ __forceinline__ dd2 task_sum(double rh, double rl, double ih, double 
     return res;
 }
 
-__device__ void process_task(const ExecArgs& a, const Task& t, WarpSmem& sm, int& staged, int lane)
-{
-    const PermDesc D = a.desc[t.perm];
-    const MetaView mv = meta_view(a.meta, D);
-    const int l = D.l, J = D.J, ndig = D.ndig;
-    dd2 res = {0.0, 0.0, 0.0, 0.0};
-
-    if (!D.trivial) {
-        if (staged != t.perm) {
-            __syncwarp();
-            stage_perm(a, D, mv, sm, lane);
-            staged = t.perm;
-        }
-        // ---- this lane's chunk: decode the high digits, start the column sums
-        const int64_t chunk0 = (int64_t)t.part * kWarp;
-        const bool active = chunk0 + lane < D.nchunks;
-        int64_t c = active ? (chunk0 + lane) : 0;
-        double2* S = sm.S + lane;
-#pragma unroll 1
-        for (int j = 0; j < l; ++j)
-            S[j * 32] = sm.base[j];
-        uint64_t whigh_u = 1;
-        int gpar = 0;
-#pragma unroll 1
-        for (int d = J; d < ndig; ++d) {
-            const int rad = mv.drad[d];
-            const int g = (int)(c % rad);
-            c /= rad;
-            if (g == 0)  // no sign flip in this row: nothing to do (for the whole warp, often)
-                continue;
-            const double2* Mr = sm.M + mv.drow[d] * sm.ld;
-            const double coef = (double)(-2 * g);
-#pragma unroll 1
-            for (int j = 0; j < l; ++j) {
-                const double2 b = Mr[j];
-                double2 s = S[j * 32];
-                s.x = __fma_rn(coef, b.x, s.x);
-                s.y = __fma_rn(coef, b.y, s.y);
-                S[j * 32] = s;
-            }
-            whigh_u *= binom_u64(mv.dtop[d], g);
-            gpar += g;
-        }
-
-        // ---- warp-uniform walk over the low digits
-        LowWalk wk;
-        wk.v = 0;
-        wk.g = 0;
-        wk.dir = 0;
-        wk.radm1 = 0;
-        wk.topp = 0;
-        for (int d = 0; d < J; ++d) {
-            wk.radm1 |= uint64_t(mv.drad[d] - 1) << (4 * d);
-            wk.topp |= uint64_t(mv.dtop[d]) << (4 * d);
-        }
-        const bool weighted = D.weighted != 0;
-        const bool unit = D.jf < 0;
-        const int jf = D.jf;
-        // acc: the terms since the weight last changed (unweighted); run: the
-        // weighted sum since the last fold; every 32 terms run (or, for an
-        // unweighted permanent, acc) is folded into the double-double rh/rl,
-        // ih/il.  The weight changes only when a digit of radix > 2 moves, so
-        // it costs 2 DFMA per change instead of 2 DMUL per term.
-        double wlow = 1.0;
-        double2 acc = make_double2(0.0, 0.0), run = make_double2(0.0, 0.0);
-        double rh = 0.0, rl = 0.0, ih = 0.0, il = 0.0;
-        const int64_t L = D.L;
-        int64_t s = 0;
-        int blk = 0;
-#pragma unroll 1
-        while (s < L) {
-            glynn_term<false>(S, l, unit, jf, sm.ecnt, acc);
-            if (++s < L) {
-                if (glynn_step(wk, sm, S, l) && weighted)
-                    reweight(wk, J, wlow, acc, run);
-                glynn_term<true>(S, l, unit, jf, sm.ecnt, acc);
-                if (++s < L && glynn_step(wk, sm, S, l) && weighted)
-                    reweight(wk, J, wlow, acc, run);
-            }
-            if (++blk == 16) {
-                blk = 0;
-                if (weighted) {
-                    run.x = __fma_rn(wlow, acc.x, run.x);
-                    run.y = __fma_rn(wlow, acc.y, run.y);
-                    acc = run;
-                    run = make_double2(0.0, 0.0);
-                }
-                dd_acc(rh, rl, acc.x);
-                dd_acc(ih, il, acc.y);
-                acc = make_double2(0.0, 0.0);
-            }
-        }
-        if (weighted) {
-            run.x = __fma_rn(wlow, acc.x, run.x);
-            run.y = __fma_rn(wlow, acc.y, run.y);
-            acc = run;
-        }
-        dd_acc(rh, rl, acc.x);
-        dd_acc(ih, il, acc.y);
-        res = task_sum(rh, rl, ih, il, whigh_u, (gpar & 1) != 0, active);
-    }
-    combine_task(a, t, D, res, lane);
-}
-
 // The task's sum res (the same on every lane) goes to the permanent's output
 // if the permanent has one task; otherwise to its slot, and the warp that
 // writes the last slot adds the slots in task order.
-__device__ void combine_task(const ExecArgs& a, const Task& t, const PermDesc& D, dd2 res, int lane)
+__device__ void combine_task(const ExecArgs& a, const Task& t, const PermDesc& D, dd2 res, int exp2,
+                             int lane)
 {
     if (D.ntasks <= 1) {
         if (lane == 0)
-            finalize(a, D, res);
+            finalize(a, D, res, exp2);
         return;
     }
     int last = 0;
@@ -370,176 +422,12 @@ __device__ void combine_task(const ExecArgs& a, const Task& t, const PermDesc& D
     warp_fix_sum(tot.rh, tot.rl, tot.rh, tot.rl);
     warp_fix_sum(tot.ih, tot.il, tot.ih, tot.il);
     if (lane == 0)
-        finalize(a, D, tot);
+        finalize(a, D, tot, exp2);
 }
 
-// ---------------------------------------------------------------- register-resident walk
-// For product sides of at most kFwdRegMaxLd columns a lane keeps its column
-// sums in registers, in a walk instantiated for even column bounds NL and
-// launched once per class of permanents (at most NL product columns).
-// Columns 0 .. l-2 live in registers 0 .. l-2 and the last column l-1 in
-// register NL-1; the registers between are padding whose sum stays exactly
-// 1 + 0i (its base-matrix entries are staged as zeros and its extra-prefix
-// count as 0).  So no FP64 instruction of the walk depends on l: every column
-// loop runs over all NL registers without a test, and a padding column costs
-// its products by 1, which are exact (a test per column made the compiler
-// predicate the FP64 work, and predicated-off instructions took 40-55% of
-// the FP64 pipe).  The products are formed in the order of the shared-memory
-// walk, so both give the same bits.  A warp's shared memory holds the base
-// matrix and its column sums in register order and the small integer arrays.
-__host__ __device__ inline int reg_warp_smem_bytes(int kmax, int ld)
+// ---------------------------------------------------------------- the walk
+__device__ __forceinline__ void start_walk(LowWalk& wk, const MetaView& mv, int J)
 {
-    int bytes = (kmax * ld + ld) * 16 + (16 + ld) * 4;
-    return (bytes + 15) & ~15;
-}
-
-struct RegSmem {
-    double2* M;       // kmax x ld, register order
-    double2* base;    // ld, register order
-    int32_t* lowrow;  // 16
-    int32_t* ecnt;    // ld, register order
-    int ld;
-    __device__ RegSmem(unsigned char* raw, int kmax, int ld_)
-    {
-        ld = ld_;
-        M = reinterpret_cast<double2*>(raw);
-        base = M + kmax * ld;
-        lowrow = reinterpret_cast<int32_t*>(base + ld);
-        ecnt = lowrow + 16;
-    }
-};
-
-// Register of product column j of a permanent with l columns.
-template <int NL>
-__device__ __forceinline__ int reg_of(int j, int l)
-{
-    return j == l - 1 ? NL - 1 : j;
-}
-
-// Stage permanent D for the register walk: base matrix and base column sums
-// in register order (padding: entries 0, sum 1 + 0i), extra-prefix counts in
-// register order (padding: 0).  sm.ld = NL.
-template <int NL>
-__device__ void stage_perm_reg(const ExecArgs& a, const PermDesc& D, const MetaView& mv,
-                               RegSmem& sm, int lane)
-{
-    const int k = D.k, l = D.l;
-    for (int e = lane; e < k * NL; e += kWarp) {
-        const int i = e / NL, r = e - i * NL;
-        double2 v = make_double2(0.0, 0.0);
-        const int j = r == NL - 1 ? l - 1 : r;
-        if (r == NL - 1 || r < l - 1) {
-            const int64_t off =
-                D.src_off + (int64_t)mv.ridx[i] * D.si + (int64_t)mv.cidx[j] * D.sj;
-            v = a.src[off];
-        }
-        sm.M[e] = v;
-    }
-    for (int d = lane; d < D.J; d += kWarp)
-        sm.lowrow[d] = mv.drow[d];
-    for (int r = lane; r < NL; r += kWarp)
-        sm.ecnt[r] = r == NL - 1 ? mv.ecnt[l - 1] : (r < l - 1 ? mv.ecnt[r] : 0);
-    __syncwarp();
-    for (int r = lane; r < NL; r += kWarp) {
-        double2 s = make_double2(0.0, 0.0);
-        if (r == NL - 1 || r < l - 1) {
-            for (int i = 0; i < k; ++i) {
-                const double rm = (double)mv.rmul[i];
-                const double2 b = sm.M[i * NL + r];
-                s.x = __fma_rn(rm, b.x, s.x);
-                s.y = __fma_rn(rm, b.y, s.y);
-            }
-        } else {
-            s = make_double2(1.0, 0.0);
-        }
-        sm.base[r] = s;
-    }
-    __syncwarp();
-}
-
-// S += coef * (row Mr), every register (padding entries are zero).
-template <int NL>
-__device__ __forceinline__ void reg_add_row(double2 (&S)[NL], const double2* Mr, double coef)
-{
-#pragma unroll
-    for (int r = 0; r < NL; ++r) {
-        const double2 b = Mr[r];
-        S[r].x = __fma_rn(coef, b.x, S[r].x);
-        S[r].y = __fma_rn(coef, b.y, S[r].y);
-    }
-}
-
-// One term, as glynn_term: acc +-= prod_j S_j^{c_j}.  jr = register of the
-// first column with an extra prefix (-1: every c_j = 1); ec = extra-prefix
-// counts in register order.
-template <int NL, bool NEG>
-__device__ __forceinline__ void reg_term(const double2 (&S)[NL], int jr, const int (&ec)[NL],
-                                         double2& acc)
-{
-    if (jr < 0) {
-        double2 p = S[0];
-#pragma unroll
-        for (int r = 1; r < NL - 1; ++r)
-            p = cmul(p, S[r]);
-        cfma_acc<NEG>(acc, p, S[NL - 1]);
-        return;
-    }
-    // P(q) = S_0 ... S_{q-1} for every column; at the first column with an
-    // extra prefix ex starts as that prefix, and each extra multiplies it in
-    double2 pre = S[0], ex = S[0];
-#pragma unroll
-    for (int r = 0; r < NL; ++r) {
-        if (r > 0)
-            pre = cmul(pre, S[r]);
-        ex = r == jr ? pre : ex;
-        const int e0 = r == jr ? 1 : 0;
-#pragma unroll 1
-        for (int e = e0; e < ec[r]; ++e)
-            ex = cmul(ex, pre);
-    }
-    cfma_acc<NEG>(acc, pre, ex);
-}
-
-// One Gray step, as glynn_step, on the register column sums.
-template <int NL>
-__device__ __forceinline__ bool reg_step(LowWalk& wk, const RegSmem& sm, double2 (&S)[NL])
-{
-    int up;
-    const int d = low_step(wk, up);
-    reg_add_row(S, sm.M + sm.lowrow[d] * NL, up > 0 ? -2.0 : 2.0);
-    return ((wk.radm1 >> (4 * d)) & 15u) > 1u;
-}
-
-// The walk of this lane's chunk c (as in process_task); returns the task's
-// sum over the warp (task_sum).
-template <int NL>
-__device__ __forceinline__ dd2 reg_walk(const PermDesc& D, const MetaView& mv, const RegSmem& sm,
-                                        int64_t c, bool active)
-{
-    const int l = D.l, J = D.J, ndig = D.ndig;
-    double2 S[NL];
-    int ec[NL];
-#pragma unroll
-    for (int r = 0; r < NL; ++r) {
-        S[r] = sm.base[r];
-        ec[r] = sm.ecnt[r];
-    }
-    const int jr = D.jf < 0 ? -1 : reg_of<NL>(D.jf, l);
-    uint64_t whigh_u = 1;
-    int gpar = 0;
-#pragma unroll 1
-    for (int d = J; d < ndig; ++d) {
-        const int rad = mv.drad[d];
-        const int g = (int)(c % rad);
-        c /= rad;
-        if (g == 0)
-            continue;
-        reg_add_row(S, sm.M + mv.drow[d] * NL, (double)(-2 * g));
-        whigh_u *= binom_u64(mv.dtop[d], g);
-        gpar += g;
-    }
-
-    LowWalk wk;
     wk.v = 0;
     wk.g = 0;
     wk.dir = 0;
@@ -549,25 +437,105 @@ __device__ __forceinline__ dd2 reg_walk(const PermDesc& D, const MetaView& mv, c
         wk.radm1 |= uint64_t(mv.drad[d] - 1) << (4 * d);
         wk.topp |= uint64_t(mv.dtop[d]) << (4 * d);
     }
+}
+
+// Digit of radix rad split off the chunk index c.
+__device__ __forceinline__ int next_digit(int64_t& c, int rad, bool narrow)
+{
+    if (narrow) {
+        const uint32_t v = (uint32_t)c, q = v / (uint32_t)rad;
+        c = q;
+        return (int)(v - q * (uint32_t)rad);
+    }
+    const int g = (int)(c % rad);
+    c /= rad;
+    return g;
+}
+
+// C(top, g) for a high digit.
+__device__ __forceinline__ uint64_t high_binom(int top, int g)
+{
+    if (top <= 3)
+        return (g == 0 || g == top) ? 1 : (uint64_t)top;
+    return binom_u64(top, g);
+}
+
+// The walk of this lane's chunk; returns the task's sum over the warp
+// (task_sum).  NL = 0: column sums in shared memory; NL > 0: in registers.
+template <int NL>
+__device__ __forceinline__ dd2 int_walk(const PermDesc& D, const MetaView& mv, const WarpSmem& sm,
+                                        uint32_t emask, int64_t chunk, bool active, int lane)
+{
+    const int l = D.l, J = D.J, ndig = D.ndig, ld = NL > 0 ? NL : sm.ld;
+    constexpr int kRegs = NL > 0 ? NL : 1;
+    longlong2 R[kRegs];
+    longlong2* S = sm.S + lane;
+    if constexpr (NL > 0) {
+#pragma unroll
+        for (int j = 0; j < NL; ++j)
+            R[j] = j < l ? sm.base[j] : make_longlong2(0, 0);
+    } else {
+#pragma unroll 1
+        for (int j = 0; j < l; ++j)
+            S[j * 32] = sm.base[j];
+    }
+    const bool narrow = D.nchunks <= 0x7fffffff;
+    uint64_t whigh_u = 1;
+    int gpar = 0;
+#pragma unroll 1
+    for (int d = J; d < ndig; ++d) {
+        const int g = next_digit(chunk, mv.drad[d], narrow);
+        if (g == 0)  // no sign flip in this row: nothing to do (for the whole warp, often)
+            continue;
+        const longlong2* Mr = sm.M + mv.drow[d] * ld;
+        if constexpr (NL > 0) {
+#pragma unroll
+            for (int j = 0; j < NL; ++j) {
+                if (j < l) {
+                    const longlong2 b = Mr[j];
+                    R[j].x -= g * b.x;
+                    R[j].y -= g * b.y;
+                }
+            }
+        } else {
+#pragma unroll 1
+            for (int j = 0; j < l; ++j) {
+                const longlong2 b = Mr[j];
+                longlong2 s = S[j * 32];
+                s.x -= g * b.x;
+                s.y -= g * b.y;
+                S[j * 32] = s;
+            }
+        }
+        whigh_u *= high_binom(mv.dtop[d], g);
+        gpar += g;
+    }
+
+    LowWalk wk;
+    start_walk(wk, mv, J);
     const bool weighted = D.weighted != 0;
+    const int jf = D.jf;
+    // acc: the terms since the weight last changed (unweighted); run: the
+    // weighted sum since the last fold; every 32 terms run (or, for an
+    // unweighted permanent, acc) is folded into the double-double rh/rl,
+    // ih/il.  The weight changes only when a digit of radix > 2 moves, so
+    // it costs 2 DFMA per change instead of 2 DMUL per term.
     double wlow = 1.0;
     double2 acc = make_double2(0.0, 0.0), run = make_double2(0.0, 0.0);
     double rh = 0.0, rl = 0.0, ih = 0.0, il = 0.0;
     const int64_t L = D.L;
+    int E;
+    BInt p;
+    if constexpr (NL > 0)
+        p = term_product<NL>(RegCols<kRegs>{R}, l, jf, emask, sm.ecnt, E);
+    else
+        p = term_product<0>(SharedCols<0>{S, sm.M}, l, jf, emask, sm.ecnt, E);
     int64_t s = 0;
-    int blk = 0;
 #pragma unroll 1
-    while (s < L) {
-        reg_term<NL, false>(S, jr, ec, acc);
-        if (++s < L) {
-            if (reg_step(wk, sm, S) && weighted)
-                reweight(wk, J, wlow, acc, run);
-            reg_term<NL, true>(S, jr, ec, acc);
-            if (++s < L && reg_step(wk, sm, S) && weighted)
-                reweight(wk, J, wlow, acc, run);
-        }
-        if (++blk == 16) {
-            blk = 0;
+    for (;;) {
+        add_term(p, E, (s & 1) != 0, acc);
+        ++s;
+        if (s == L || (s & 31) == 0) {
             if (weighted) {
                 run.x = __fma_rn(wlow, acc.x, run.x);
                 run.y = __fma_rn(wlow, acc.y, run.y);
@@ -577,36 +545,162 @@ __device__ __forceinline__ dd2 reg_walk(const PermDesc& D, const MetaView& mv, c
             dd_acc(rh, rl, acc.x);
             dd_acc(ih, il, acc.y);
             acc = make_double2(0.0, 0.0);
+            if (s == L)
+                break;
+        }
+        int up;
+        const int d = low_step(wk, up);
+        const longlong2* Mr = sm.M + sm.lowrow[d] * ld;
+        // a digit of radix > 2 moves the weight prod_d C(top_d, g_d)
+        if (weighted && ((wk.radm1 >> (4 * d)) & 15u) > 1u)
+            reweight(wk, J, wlow, acc, run);
+        if constexpr (NL > 0) {
+            if (up > 0) {
+#pragma unroll
+                for (int j = 0; j < NL; ++j) {
+                    const longlong2 b = Mr[j];
+                    R[j].x -= b.x;
+                    R[j].y -= b.y;
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < NL; ++j) {
+                    const longlong2 b = Mr[j];
+                    R[j].x += b.x;
+                    R[j].y += b.y;
+                }
+            }
+            p = term_product<NL>(RegCols<kRegs>{R}, l, jf, emask, sm.ecnt, E);
+        } else if (up > 0) {
+            p = term_product<0>(SharedCols<1>{S, Mr}, l, jf, emask, sm.ecnt, E);
+        } else {
+            p = term_product<0>(SharedCols<2>{S, Mr}, l, jf, emask, sm.ecnt, E);
         }
     }
-    if (weighted) {
-        run.x = __fma_rn(wlow, acc.x, run.x);
-        run.y = __fma_rn(wlow, acc.y, run.y);
-        acc = run;
+    return task_sum(rh, rl, ih, il, whigh_u, (gpar & 1) != 0, active);
+}
+
+// The same walk in FP64, for a base matrix without integer scales (non-finite
+// entries, a column bound beyond FP64): column sums in local memory, products
+// in the same order.  Speed is not the point here: infinities and NaNs are
+// combined as FP64 arithmetic does.
+__device__ void fp64_term(const double2* S, int l, int jf, const int32_t* ecnt, bool neg,
+                          double2& acc)
+{
+    double2 pre = S[0], ex = make_double2(neg ? -1.0 : 1.0, 0.0);
+    if (jf < 0) {
+        if (l == 1) {  // n = 1: the product is S_0 itself
+            acc.x = neg ? __dsub_rn(acc.x, pre.x) : __dadd_rn(acc.x, pre.x);
+            acc.y = neg ? __dsub_rn(acc.y, pre.y) : __dadd_rn(acc.y, pre.y);
+            return;
+        }
+        for (int j = 1; j < l - 1; ++j)
+            pre = cmul(pre, S[j]);
+        ex = S[l - 1];
+    } else {
+        for (int j = 0; j < l; ++j) {
+            if (j > 0)
+                pre = cmul(pre, S[j]);
+            if (j == jf)
+                ex = pre;
+            for (int e = j == jf ? 1 : 0; e < ecnt[j]; ++e)
+                ex = cmul(ex, pre);
+        }
     }
-    dd_acc(rh, rl, acc.x);
-    dd_acc(ih, il, acc.y);
+    if (neg)
+        cfma_acc<true>(acc, pre, ex);
+    else
+        cfma_acc<false>(acc, pre, ex);
+}
+
+__device__ __noinline__ dd2 fp64_walk(const PermDesc& D, const MetaView& mv, const WarpSmem& sm,
+                                      int64_t chunk, bool active)
+{
+    const int l = D.l, J = D.J, ndig = D.ndig;
+    const double2* M = reinterpret_cast<const double2*>(sm.M);
+    const double2* base = reinterpret_cast<const double2*>(sm.base);
+    double2 S[PQ_MAX_PRODUCT_COLS];
+    for (int j = 0; j < l; ++j)
+        S[j] = base[j];
+    auto add_row = [&](int row, double coef) {
+        for (int j = 0; j < l; ++j) {
+            const double2 b = M[row * sm.ld + j];
+            S[j].x = __fma_rn(coef, b.x, S[j].x);
+            S[j].y = __fma_rn(coef, b.y, S[j].y);
+        }
+    };
+    uint64_t whigh_u = 1;
+    int gpar = 0;
+    for (int d = J; d < ndig; ++d) {
+        const int g = next_digit(chunk, mv.drad[d], false);
+        if (g == 0)
+            continue;
+        add_row(mv.drow[d], (double)(-2 * g));
+        whigh_u *= binom_u64(mv.dtop[d], g);
+        gpar += g;
+    }
+    LowWalk wk;
+    start_walk(wk, mv, J);
+    double wlow = 1.0;
+    double2 acc = make_double2(0.0, 0.0), run = make_double2(0.0, 0.0);
+    double rh = 0.0, rl = 0.0, ih = 0.0, il = 0.0;
+    for (int64_t s = 0;;) {
+        fp64_term(S, l, D.jf, sm.ecnt, (s & 1) != 0, acc);
+        ++s;
+        if (s == D.L || (s & 31) == 0) {
+            run.x = __fma_rn(wlow, acc.x, run.x);
+            run.y = __fma_rn(wlow, acc.y, run.y);
+            dd_acc(rh, rl, run.x);
+            dd_acc(ih, il, run.y);
+            acc = run = make_double2(0.0, 0.0);
+            if (s == D.L)
+                break;
+        }
+        int up;
+        const int d = low_step(wk, up);
+        if (((wk.radm1 >> (4 * d)) & 15u) > 1u)
+            reweight(wk, J, wlow, acc, run);
+        add_row(sm.lowrow[d], up > 0 ? -2.0 : 2.0);
+    }
     return task_sum(rh, rl, ih, il, whigh_u, (gpar & 1) != 0, active);
 }
 
 template <int NL>
-__device__ void process_task_reg(const ExecArgs& a, const Task& t, RegSmem& sm, int& staged,
-                                 int lane)
+__device__ __forceinline__ void process_task(const ExecArgs& a, const Task& t, WarpSmem& sm,
+                                             Staged& st, int lane)
 {
     const PermDesc D = a.desc[t.perm];
     const MetaView mv = meta_view(a.meta, D);
     dd2 res = {0.0, 0.0, 0.0, 0.0};
     if (!D.trivial) {
-        if (staged != t.perm) {
+        if (st.perm != t.perm) {
             __syncwarp();
-            stage_perm_reg<NL>(a, D, mv, sm, lane);
-            staged = t.perm;
+            stage_perm(a, D, mv, sm, st, lane);
+            st.perm = t.perm;
         }
         const int64_t chunk0 = (int64_t)t.part * kWarp;
         const bool active = chunk0 + lane < D.nchunks;
-        res = reg_walk<NL>(D, mv, sm, active ? (chunk0 + lane) : 0, active);
+        const int64_t chunk = active ? (chunk0 + lane) : 0;
+        res = st.fp64 ? fp64_walk(D, mv, sm, chunk, active)
+                      : int_walk<NL>(D, mv, sm, st.emask, chunk, active, lane);
     }
-    combine_task(a, t, D, res, lane);
+    combine_task(a, t, D, res, st.exp2, lane);
+}
+
+// Task ti of the list, once its guards pass (a failing task is skipped and
+// recorded in the error record).
+template <int NL>
+__device__ __forceinline__ void run_task(const ExecArgs& a, int64_t ti, WarpSmem& sm, int kmax,
+                                         int ld, Staged& st, int lane)
+{
+    const Task t = a.tasks[ti];
+    const int32_t bad = task_guard(t, a.desc, a.nperm, a.nmeta, a.nslots, kmax, ld, kMaxLowDigits);
+    if (bad) {
+        if (lane == 0)
+            record_error(a.err, bad, ti);
+        return;
+    }
+    process_task<NL>(a, t, sm, st, lane);
 }
 
 // The register-resident kernel of column bound NL: tasks as in
@@ -616,7 +710,7 @@ __device__ void process_task_reg(const ExecArgs& a, const Task& t, RegSmem& sm, 
 // SM run one instantiation of the walk: warps running different ones (a
 // single kernel dispatching on l) ran 1.6 times slower.
 template <int NL>
-__global__ void __launch_bounds__(256, 1) glynn_fwd_reg_kernel(ExecArgs a, int64_t t_begin,
+__global__ void __launch_bounds__(256, NL <= 6 ? 3 : 2) glynn_fwd_reg_kernel(ExecArgs a, int64_t t_begin,
                                                              int64_t t_end, int kmax, int ld,
                                                              int queue)
 {
@@ -627,23 +721,12 @@ __global__ void __launch_bounds__(256, 1) glynn_fwd_reg_kernel(ExecArgs a, int64
             record_error(a.err, kErrDescLayout, t_begin);
         return;
     }
-    RegSmem sm(smem_raw + warp * reg_warp_smem_bytes(kmax, ld), kmax, NL);
-    int staged = -1;
-    auto run = [&](int64_t ti) {
-        const Task t = a.tasks[ti];
-        const int32_t bad = task_guard(t, a.desc, a.nperm, a.nmeta, a.nslots, kmax,
-                                       ld < NL ? ld : NL, kMaxLowDigits);
-        if (bad) {
-            if (lane == 0)
-                record_error(a.err, bad, ti);
-            return;
-        }
-        process_task_reg<NL>(a, t, sm, staged, lane);
-    };
+    WarpSmem sm(smem_raw + warp * reg_warp_smem_bytes(kmax, ld), kmax, NL, false);
+    Staged st;
     if (!queue) {
         const int64_t ti = t_begin + (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
         if (ti < t_end)
-            run(ti);
+            run_task<NL>(a, ti, sm, kmax, NL, st, lane);
         return;
     }
     for (;;) {
@@ -654,41 +737,26 @@ __global__ void __launch_bounds__(256, 1) glynn_fwd_reg_kernel(ExecArgs a, int64
         const int64_t ti = t_begin + q;
         if (ti >= t_end)
             break;
-        run(ti);
+        run_task<NL>(a, ti, sm, kmax, NL, st, lane);
     }
-}
-
-// Task ti of the list, once its guards pass (a failing task is skipped and
-// recorded in the error record).
-__device__ __forceinline__ void run_task(const ExecArgs& a, int64_t ti, WarpSmem& sm, int kmax,
-                                         int ld, int& staged, int lane)
-{
-    const Task t = a.tasks[ti];
-    const int32_t bad = task_guard(t, a.desc, a.nperm, a.nmeta, a.nslots, kmax, ld, kMaxLowDigits);
-    if (bad) {
-        if (lane == 0)
-            record_error(a.err, bad, ti);
-        return;
-    }
-    process_task(a, t, sm, staged, lane);
 }
 
 // Tasks [t_begin, t_end) of the list.  queue != 0: every warp pulls tasks from
 // the global counter until the range is exhausted (persistent launch of a
 // whole batch); queue == 0: warp w of block b takes task t_begin + b * wpb + w
 // (one launch per permanent, the plain method).
-__global__ void __launch_bounds__(256, 2) glynn_fwd_kernel(ExecArgs a, int64_t t_begin,
+__global__ void __launch_bounds__(256, 3) glynn_fwd_kernel(ExecArgs a, int64_t t_begin,
                                                          int64_t t_end, int kmax, int ld,
                                                          int queue)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    WarpSmem sm(smem_raw + warp * warp_smem_bytes(kmax, ld), kmax, ld);
-    int staged = -1;
+    WarpSmem sm(smem_raw + warp * warp_smem_bytes(kmax, ld), kmax, ld, true);
+    Staged st;
     if (!queue) {
         const int64_t ti = t_begin + (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
         if (ti < t_end)
-            run_task(a, ti, sm, kmax, ld, staged, lane);
+            run_task<0>(a, ti, sm, kmax, ld, st, lane);
         return;
     }
     for (;;) {
@@ -699,20 +767,20 @@ __global__ void __launch_bounds__(256, 2) glynn_fwd_kernel(ExecArgs a, int64_t t
         const int64_t ti = t_begin + q;
         if (ti >= t_end)
             break;
-        run_task(a, ti, sm, kmax, ld, staged, lane);
+        run_task<0>(a, ti, sm, kmax, ld, st, lane);
     }
 }
 
 // All column classes in one persistent launch: each task runs the
 // instantiation of its own class.
-__global__ void __launch_bounds__(256, 1) glynn_fwd_reg_mixed_kernel(ExecArgs a, int64_t t_begin,
+__global__ void __launch_bounds__(256, 2) glynn_fwd_reg_mixed_kernel(ExecArgs a, int64_t t_begin,
                                                                      int64_t t_end, int kmax,
                                                                      int ld, int queue)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     unsigned char* raw = smem_raw + warp * reg_warp_smem_bytes(kmax, ld);
-    int staged = -1, staged_nl = 0;
+    Staged st;
     auto run = [&](int64_t ti) {
         const Task t = a.tasks[ti];
         const int32_t bad =
@@ -729,14 +797,11 @@ __global__ void __launch_bounds__(256, 1) glynn_fwd_reg_mixed_kernel(ExecArgs a,
                 record_error(a.err, kErrDescLayout, ti);
             return;
         }
-        if (nl != staged_nl)
-            staged = -1;  // the staged layout depends on the class
-        staged_nl = nl;
         switch (nl) {
 #define PQ_REG_CASE(N)                                   \
     case N: {                                            \
-        RegSmem sm(raw, kmax, N);                        \
-        process_task_reg<N>(a, t, sm, staged, lane);     \
+        WarpSmem sm(raw, kmax, N, false);                \
+        process_task<N>(a, t, sm, st, lane);             \
         break;                                           \
     }
             PQ_REG_CASE(4)

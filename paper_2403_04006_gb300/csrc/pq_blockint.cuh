@@ -1,0 +1,215 @@
+// pq_blockint.cuh -- complex products in 64-bit block integers, the arithmetic
+// of the walks' products.
+//
+// GB300 issues 2 FP64 lane operations per clock and SM, and the integer pipes
+// 64 to 128; a 32 x 32 + 64 bit multiply-add (IMAD.WIDE) runs at 32 lanes per
+// clock and SM.  A complex product in FP64 takes 4 FP64 instructions and the
+// column update of a Gray step 2, 3.3 clocks per lane, column and term at the
+// pipe's measured 1.8; the same work in the integers below takes 0.57.  So a
+// lane's column sums and running products are integers, and FP64 is left
+// with one conversion and one fused add per term and component.
+//
+// Column sums.  Column j of a permanent is scaled by 2^e_j, chosen so that
+// every |Re S_j|, |Im S_j| the code can reach stays below 2^62 (the bound is
+// sum_i r_i max(|Re b_ij|, |Im b_ij|), added up in integers of 21 bits: FP64
+// would take the 16 warps of an SM longer than the rest of the staging), and its entries are rounded to
+// integers once, when the base matrix is staged.  Every update of a column sum
+// is then exact; in FP64 each of them rounded, at 2^-53 of the largest sum on
+// the way against the single rounding at 2^-62 of the bound here.
+//
+// Products.  A complex number is two signed 64-bit integers with one binary
+// exponent.  p s is formed from 32-bit limbs (high signed, low signed after
+// moving its carry up): the four high products in 64 bits and the high words
+// of the eight cross products, low times low left out: (p s) >> 64 with an
+// absolute error of about one unit.  Every second product is normalised
+// (shifted left until the larger component has its top bit at 61, the shift
+// added to the exponent).  A product of two typical column sums has about 2^56,
+// so two products cost an error of about 2^-55 of the product's magnitude, a
+// third of what two FP64 complex products round.
+//
+// The multiply-adds are written as mul.wide plus a 64-bit add: ptxas fuses
+// these, while mad.wide was split into more instructions (0.57 against 0.70
+// clocks per lane, column and term in an isolated loop).
+#pragma once
+#include <cuda_runtime.h>
+#include <stdint.h>
+
+namespace pqi {
+
+constexpr int kSumBits = 62;  // column sums stay below 2^kSumBits in magnitude
+
+// Complex number of two 64-bit integers in 32-bit words.
+struct BInt {
+    int rh, ih;
+    uint32_t rl, il;
+};
+
+// re = a 2^32 + b, im = c 2^32 + d with signed low words.
+struct BLimbs {
+    int a, b, c, d;
+};
+
+__host__ __device__ __forceinline__ uint64_t bint_bits(double x)
+{
+#ifdef __CUDA_ARCH__
+    return (uint64_t)__double_as_longlong(x);
+#else
+    uint64_t u;
+    __builtin_memcpy(&u, &x, sizeof(u));
+    return u;
+#endif
+}
+
+// The bound of a column's sums, in integers.  An entry counts with the high
+// word of the larger of |Re|, |Im| (bint_mag).  With hmax the column's largest
+// it is below bint_units(h, hmax) 2^(hmax's exponent field - 1043), and a
+// column whose units (times multiplicity) add up to u is scaled by
+// 2^bint_scale(hmax, u), which keeps its sums below 2^kSumBits (1 - 2^-21).
+// A column of subnormal entries (hmax < 2^20) is added up exactly, in units of
+// 2^-1074, so that it loses no bits (bint_scale_subnormal).
+__host__ __device__ __forceinline__ uint32_t bint_mag(double re, double im)
+{
+    const uint32_t x = (uint32_t)(bint_bits(re) >> 32) & 0x7fffffffu;
+    const uint32_t y = (uint32_t)(bint_bits(im) >> 32) & 0x7fffffffu;
+    return x > y ? x : y;
+}
+
+__host__ __device__ __forceinline__ uint32_t bint_units(uint32_t h, uint32_t hmax)
+{
+    const int f = (int)(h >> 20), d = (int)(hmax >> 20) - (f == 0 ? 1 : f);
+    const uint32_t m = (h & 0xfffffu) + (f == 0 ? 1u : 0x100001u);  // rounded up
+    return d <= 0 ? m : (d > 31 ? 1u : (m >> d) + 1u);
+}
+
+__host__ __device__ __forceinline__ int bint_width(uint64_t u)  // u < 2^width
+{
+#ifdef __CUDA_ARCH__
+    return 64 - __clzll((long long)u);
+#else
+    int bits = 0;
+    while (bits < 64 && (u >> bits) != 0)
+        ++bits;
+    return bits;
+#endif
+}
+
+__host__ __device__ __forceinline__ int bint_scale(uint32_t hmax, uint32_t units)
+{
+    return kSumBits + 1043 - (int)(hmax >> 20) - bint_width(units);
+}
+
+__host__ __device__ __forceinline__ uint64_t bint_mag_subnormal(double re, double im)
+{
+    const uint64_t x = bint_bits(re) & 0xfffffffffffffull, y = bint_bits(im) & 0xfffffffffffffull;
+    return x > y ? x : y;
+}
+
+__host__ __device__ __forceinline__ int bint_scale_subnormal(uint64_t sum)
+{
+    return kSumBits + 1074 - bint_width(sum);
+}
+
+// round(x 2^e) as an integer, ties away from zero; |x| 2^e < 2^63.
+__host__ __device__ __forceinline__ int64_t bint_of(double x, int e)
+{
+    const uint64_t u = bint_bits(x);
+    const int f = (int)((u >> 52) & 0x7ff);
+    uint64_t m = u & 0xfffffffffffffull;
+    if (f != 0)
+        m |= 0x10000000000000ull;
+    const int s = (f == 0 ? 1 : f) - 1075 + e;
+    if (s >= 0)
+        m <<= s;
+    else if (s > -55)
+        m = (m + (1ull << (-s - 1))) >> (-s);
+    else
+        m = 0;
+    return (u >> 63) ? -(int64_t)m : (int64_t)m;
+}
+
+#ifdef __CUDACC__
+// Column sums are kept with 2^31 added to each component, so that the high
+// word already holds the carry of the signed low word.
+constexpr int64_t kSumBias = int64_t(1) << 31;
+
+__device__ __forceinline__ BLimbs sum_limbs(longlong2 s)
+{
+    BLimbs v;
+    v.a = (int)(s.x >> 32);
+    v.b = (int)((uint32_t)s.x ^ 0x80000000u);
+    v.c = (int)(s.y >> 32);
+    v.d = (int)((uint32_t)s.y ^ 0x80000000u);
+    return v;
+}
+
+__device__ __forceinline__ BLimbs limbs(const BInt& p)
+{
+    BLimbs v;
+    v.a = p.rh + (int)(p.rl >> 31);
+    v.b = (int)p.rl;
+    v.c = p.ih + (int)(p.il >> 31);
+    v.d = (int)p.il;
+    return v;
+}
+
+__device__ __forceinline__ int64_t mulw(int a, int b)
+{
+    int64_t r;
+    asm("mul.wide.s32 %0, %1, %2;" : "=l"(r) : "r"(a), "r"(b));
+    return r;
+}
+
+// (p s) >> 64.  High words within 2^30 in magnitude, low words within 2^31:
+// the cross sums stay within [-2^63, 2^63).  (The differences are taken of
+// the products: negating a low word would overflow at -2^31.)
+__device__ __forceinline__ BInt bmul(const BLimbs& p, const BLimbs& s)
+{
+    const int64_t mr = (mulw(p.a, s.b) + mulw(p.b, s.a)) - (mulw(p.c, s.d) + mulw(p.d, s.c));
+    const int64_t mi = (mulw(p.a, s.d) + mulw(p.b, s.c)) + (mulw(p.c, s.b) + mulw(p.d, s.a));
+    const int64_t hr = mulw(p.a, s.a) - mulw(p.c, s.c) + (int64_t)(int)(mr >> 32);
+    const int64_t hi = mulw(p.a, s.c) + mulw(p.c, s.a) + (int64_t)(int)(mi >> 32);
+    BInt r;
+    r.rh = (int)(hr >> 32);
+    r.rl = (uint32_t)hr;
+    r.ih = (int)(hi >> 32);
+    r.il = (uint32_t)hi;
+    return r;
+}
+
+// Shift left until the larger high word has its top bit at position 29; the
+// shift (at most 30) is added to E.
+__device__ __forceinline__ void bnorm(BInt& p, int& E)
+{
+    const uint32_t t = (uint32_t)abs(p.rh) | (uint32_t)abs(p.ih);
+    int top;
+    asm("bfind.u32 %0, %1;" : "=r"(top) : "r"(t));  // -1 for zero
+    const int s = 29 - top;
+    E += s;
+    p.rh = (int)__funnelshift_l(p.rl, (uint32_t)p.rh, s);
+    p.rl <<= s;
+    p.ih = (int)__funnelshift_l(p.il, (uint32_t)p.ih, s);
+    p.il <<= s;
+}
+
+__device__ __forceinline__ BInt bint_plain(longlong2 s)
+{
+    BInt p;
+    s.x -= kSumBias;
+    s.y -= kSumBias;
+    p.rh = (int)(s.x >> 32);
+    p.rl = (uint32_t)s.x;
+    p.ih = (int)(s.y >> 32);
+    p.il = (uint32_t)s.y;
+    return p;
+}
+
+// +-2^(-kSumBits - E): the factor that takes a product's integers to the
+// range of FP64 (zero below its smallest normal number).
+__device__ __forceinline__ double bint_factor(int E, bool neg)
+{
+    const int f = max(1023 - kSumBits - E, 0);
+    return __hiloint2double((f << 20) | (neg ? (int)0x80000000 : 0), 0);
+}
+#endif
+
+}  // namespace pqi

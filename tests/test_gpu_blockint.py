@@ -1,0 +1,124 @@
+"""The forward walk's block-integer arithmetic where it can go wrong: low
+words at the edge of their range, column scales over the whole exponent range,
+entries that vanish beside their column's largest, exact zeros, and inputs that
+have no scale at all (non-finite, or a column bound beyond FP64).  Expected
+values are exact rational permanents; the bound is that of an FP64 evaluation
+of the Glynn sum, 8 n 2^-53 of the mean absolute term."""
+import numpy as np
+import pytest
+
+from paper_2403_04006_gb300 import api, workloads as W
+from exact import abs_err, exact_perm_grouped
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def dev():
+    return torch.device("cuda:0")
+
+
+def abs_sum(A):
+    """2^-(n-1) sum over sign vectors (first fixed) of prod_j |sum_i d_i a_ij|."""
+    n = A.shape[0]
+    signs = np.array(np.meshgrid(*[[1.0, -1.0]] * (n - 1), indexing="ij")).reshape(n - 1, -1).T
+    d = np.concatenate([np.ones((signs.shape[0], 1)), signs], axis=1)
+    return float(np.prod(np.abs(d @ A), axis=1).sum()) / 2 ** (n - 1)
+
+
+def check(items, dev, method, sums):
+    pb = W.pack_batch(items)
+    plan = api.Plan.for_batch(pb, method=method, column_sums=sums)
+    got = api.permanent_batched(api.DeviceBatch(pb, dev), plan).cpu().numpy()
+    for q, ((B, r, c), g) in enumerate(zip(items, got)):
+        A = np.repeat(np.repeat(np.asarray(B), r, 0), c, 1)
+        err = abs_err(complex(g), exact_perm_grouped(B, r, c))
+        assert err <= 8 * A.shape[0] * 2.0 ** -53 * abs_sum(A), (q, g, err)
+
+
+FORMS = [(m, s) for m in ("batched", "plain") for s in ("shared", "registers")]
+
+
+@pytest.mark.parametrize("method,sums", FORMS)
+def test_low_words_at_the_edge(dev, method, sums):
+    """Column sums whose integers have a low word of exactly 2^31 (with a
+    column bound in (1, 2) the unit is 2^-61, so 2^-30 is 2^31 units), in the
+    real and in the imaginary part, against columns of every size up to 9."""
+    rng = np.random.default_rng(1)
+    items = []
+    for n in range(2, 10):
+        for part in (1.0, 1j):
+            A = rng.integers(-4, 5, (n, n)) / (8.0 * n) + 1j * rng.integers(-4, 5, (n, n)) / (8.0 * n)
+            A[0] += 1.0 + part * 2.0 ** -30
+            items.append((A, [1] * n, [1] * n))
+        items.append((A[:, :2] if n == 2 else A[:, :n - 1], [1] * n,
+                      [1] * 2 if n == 2 else [2] + [1] * (n - 2)))
+    check(items, dev, method, sums)
+
+
+@pytest.mark.parametrize("method,sums", FORMS)
+def test_scales_over_the_exponent_range(dev, method, sums):
+    """Columns times 2^400, 2^-400 and subnormal columns beside large ones,
+    with repeated rows and columns; entries below the unit of their column."""
+    rng = np.random.default_rng(2)
+    items = []
+    for n in (2, 3, 5, 6):
+        A = rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))
+        e = np.where(np.arange(n) % 2 == 0, 400, -400)
+        items.append((np.ldexp(A.real, e) + 1j * np.ldexp(A.imag, e), [1] * n, [1] * n))
+    A = rng.standard_normal((3, 3)) + 1j * rng.standard_normal((3, 3))
+    e = np.array([-1060, 500, 500])
+    items.append((np.ldexp(A.real, e) + 1j * np.ldexp(A.imag, e), [1] * 3, [1] * 3))
+    A = rng.standard_normal((4, 3)) + 1j * rng.standard_normal((4, 3))
+    A[1] *= 1e-17
+    A[2] *= 1e-25
+    items.append((A, [1, 2, 1, 2], [3, 2, 1]))
+    check(items, dev, method, sums)
+
+
+@pytest.mark.parametrize("method,sums", FORMS)
+def test_exact_zeros(dev, method, sums):
+    """A zero row, a zero column, and a block structure without a perfect
+    matching give exactly zero."""
+    rng = np.random.default_rng(3)
+    items = []
+    for n in (2, 4, 7, 11):
+        A = rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))
+        Z = A.copy()
+        Z[n // 2] = 0
+        items.append((Z, [1] * n, [1] * n))
+        Z = A.copy()
+        Z[:, n - 1] = 0
+        items.append((Z, [1] * n, [1] * n))
+    pb = W.pack_batch(items)
+    got = api.permanent_batched(api.DeviceBatch(pb, dev),
+                                api.Plan.for_batch(pb, method=method, column_sums=sums))
+    assert (got.cpu().numpy() == 0).all()
+
+
+@pytest.mark.parametrize("method,sums", FORMS)
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan, 1.7e308])
+def test_inputs_without_a_scale(dev, method, sums, bad):
+    """An infinite or NaN entry, or a column whose sums overflow FP64, gives a
+    result that is not finite; the permanents beside it keep their bits."""
+    rng = np.random.default_rng(4)
+    items = []
+    for n in (1, 3, 6, 10):
+        A = rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))
+        items.append((A, [1] * n, [1] * n))
+    clean = W.pack_batch(items)
+    want = api.permanent_batched(api.DeviceBatch(clean, dev),
+                                 api.Plan.for_batch(clean, method=method, column_sums=sums))
+    dirty = []
+    for A, r, c in items:
+        A = A.copy()
+        A[0, 0] = bad
+        A[-1, 0] = bad
+        dirty.append((A, r, c))
+    pb = W.pack_batch(items[:2] + dirty[1:] + items[2:])
+    got = api.permanent_batched(api.DeviceBatch(pb, dev),
+                                api.Plan.for_batch(pb, method=method, column_sums=sums))
+    got, want = got.cpu().numpy(), want.cpu().numpy()
+    assert np.array_equal(got[[0, 1, 5, 6]].view(np.float64), want.view(np.float64))
+    assert not np.isfinite(got[2:5]).any()
