@@ -18,10 +18,8 @@
 //     without repeated columns they are taken in pairs, p (S_j S_{j+1}),
 //     which halves the dependent chain;
 //   * a term is converted to FP64 and added to a running FP64 sum with its
-//     sign (-1)^step and its power of two in one DFMA per component; the
-//     binomial weight of the low digits changes only when a digit of radix > 2
-//     moves, so a run of equally weighted terms is summed unweighted and
-//     weighted once (two DFMA);
+//     sign (-1)^step, the binomial weight of the low digits and its power of
+//     two in one DFMA per component;
 //   * every 32 terms the FP64 running sum is folded into a double-double
 //     accumulator with TwoSum.
 // A base matrix with a non-finite entry, or a column whose bound overflows, has
@@ -300,10 +298,10 @@ __device__ __forceinline__ BInt term_product(const Cols& col, int l, int jf, uin
     return bmul(limbs(pre), limbs(ex));
 }
 
-// acc +-= 2^(-kSumBits - E) p
-__device__ __forceinline__ void add_term(const BInt& p, int E, bool neg, double2& acc)
+// acc +-= w 2^(-kSumBits - E) p
+__device__ __forceinline__ void add_term(const BInt& p, int E, double w, bool neg, double2& acc)
 {
-    const double f = bint_factor(E, neg);
+    const double f = bint_factor(w, E, neg);
     const long long re = (long long)(((uint64_t)(uint32_t)p.rh << 32) | p.rl);
     const long long im = (long long)(((uint64_t)(uint32_t)p.ih << 32) | p.il);
     acc.x = __fma_rn(__ll2double_rn(re), f, acc.x);
@@ -511,70 +509,77 @@ __device__ __forceinline__ dd2 int_walk(const PermDesc& D, const MetaView& mv, c
         gpar += g;
     }
 
-    LowWalk wk;
-    start_walk(wk, mv, J);
+    LowDigits lo;
+    lo.radm1 = lo.topp = 0;
+    lo.J = J;
+    for (int d = 0; d < J; ++d) {
+        lo.radm1 |= uint64_t(mv.drad[d] - 1) << (4 * d);
+        lo.topp |= uint64_t(mv.dtop[d]) << (4 * d);
+    }
     const bool weighted = D.weighted != 0;
     const int jf = D.jf;
-    // acc: the terms since the weight last changed (unweighted); run: the
-    // weighted sum since the last fold; every 32 terms run (or, for an
-    // unweighted permanent, acc) is folded into the double-double rh/rl,
-    // ih/il.  The weight changes only when a digit of radix > 2 moves, so
-    // it costs 2 DFMA per change instead of 2 DMUL per term.
-    double wlow = 1.0;
-    double2 acc = make_double2(0.0, 0.0), run = make_double2(0.0, 0.0);
+    // The Gray steps are the same for all lanes.  Every 32 steps each lane
+    // works out one of them (the changed row's offset in M, bit 0: down, and
+    // the weight after it) and the walk takes them by shuffle: about a quarter
+    // of the instructions that carrying the digits from step to step takes on
+    // every lane.
+    uint32_t steps = 0;
+    double step_w = 1.0, w = 1.0;
+    // every 32 terms acc is folded into the double-double rh/rl, ih/il
+    double2 acc = make_double2(0.0, 0.0);
     double rh = 0.0, rl = 0.0, ih = 0.0, il = 0.0;
-    const int64_t L = D.L;
+    const uint32_t L = (uint32_t)D.L;  // at most 2^30 (the planner's cap)
     int E;
     BInt p;
     if constexpr (NL > 0)
         p = term_product<NL>(RegCols<kRegs>{R}, l, jf, emask, sm.ecnt, E);
     else
         p = term_product<0>(SharedCols<0>{S, sm.M}, l, jf, emask, sm.ecnt, E);
-    int64_t s = 0;
+    uint32_t s = 0;
 #pragma unroll 1
     for (;;) {
-        add_term(p, E, (s & 1) != 0, acc);
+        add_term(p, E, w, (s & 1u) != 0, acc);
         ++s;
-        if (s == L || (s & 31) == 0) {
-            if (weighted) {
-                run.x = __fma_rn(wlow, acc.x, run.x);
-                run.y = __fma_rn(wlow, acc.y, run.y);
-                acc = run;
-                run = make_double2(0.0, 0.0);
-            }
+        if (s == L || (s & 31u) == 0) {
             dd_acc(rh, rl, acc.x);
             dd_acc(ih, il, acc.y);
             acc = make_double2(0.0, 0.0);
             if (s == L)
                 break;
         }
-        int up;
-        const int d = low_step(wk, up);
-        const longlong2* Mr = sm.M + sm.lowrow[d] * ld;
-        // a digit of radix > 2 moves the weight prod_d C(top_d, g_d)
-        if (weighted && ((wk.radm1 >> (4 * d)) & 15u) > 1u)
-            reweight(wk, J, wlow, acc, run);
+        const int q = (int)((s - 1u) & 31u);
+        if (q == 0) {
+            bool up;
+            uint64_t wu;
+            const int d = gray_step_at(lo, s + (uint32_t)lane, weighted, up, wu);
+            steps = ((uint32_t)(sm.lowrow[d] * ld) << 1) | (up ? 0u : 1u);
+            step_w = (double)wu;
+        }
+        const uint32_t step = __shfl_sync(0xffffffffu, steps, q);
+        if (weighted)
+            w = __shfl_sync(0xffffffffu, step_w, q);
+        const longlong2* Mr = sm.M + (step >> 1);
         if constexpr (NL > 0) {
-            if (up > 0) {
-#pragma unroll
-                for (int j = 0; j < NL; ++j) {
-                    const longlong2 b = Mr[j];
-                    R[j].x -= b.x;
-                    R[j].y -= b.y;
-                }
-            } else {
+            if (step & 1u) {
 #pragma unroll
                 for (int j = 0; j < NL; ++j) {
                     const longlong2 b = Mr[j];
                     R[j].x += b.x;
                     R[j].y += b.y;
                 }
+            } else {
+#pragma unroll
+                for (int j = 0; j < NL; ++j) {
+                    const longlong2 b = Mr[j];
+                    R[j].x -= b.x;
+                    R[j].y -= b.y;
+                }
             }
             p = term_product<NL>(RegCols<kRegs>{R}, l, jf, emask, sm.ecnt, E);
-        } else if (up > 0) {
-            p = term_product<0>(SharedCols<1>{S, Mr}, l, jf, emask, sm.ecnt, E);
-        } else {
+        } else if (step & 1u) {
             p = term_product<0>(SharedCols<2>{S, Mr}, l, jf, emask, sm.ecnt, E);
+        } else {
+            p = term_product<0>(SharedCols<1>{S, Mr}, l, jf, emask, sm.ecnt, E);
         }
     }
     return task_sum(rh, rl, ih, il, whigh_u, (gpar & 1) != 0, active);

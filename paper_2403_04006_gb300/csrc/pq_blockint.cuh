@@ -203,12 +203,14 @@ __device__ __forceinline__ BInt bint_plain(longlong2 s)
     return p;
 }
 
-// +-2^(-kSumBits - E): the factor that takes a product's integers to the
-// range of FP64 (zero below its smallest normal number).
-__device__ __forceinline__ double bint_factor(int E, bool neg)
+// +-w 2^(-kSumBits - E), the factor that takes a product's integers to a term
+// of weight w (a double >= 1) in the range of FP64: integer work on w's
+// exponent (zero below the smallest normal number).
+__device__ __forceinline__ double bint_factor(double w, int E, bool neg)
 {
-    const int f = max(1023 - kSumBits - E, 0);
-    return __hiloint2double((f << 20) | (neg ? (int)0x80000000 : 0), 0);
+    const int h = __double2hiint(w) - ((kSumBits + E) << 20);
+    return h >= 0x100000 ? __hiloint2double(h | (neg ? (int)0x80000000 : 0), __double2loint(w))
+                         : 0.0;
 }
 #endif
 

@@ -253,4 +253,47 @@ __host__ __device__ __forceinline__ uint64_t low_weight(const LowWalk& w, int J)
     return r;
 }
 
+// ---------------------------------------------------------------- Gray steps
+// The low digits of a chunk: radix - 1 and binomial top, 4 bits each.
+struct LowDigits {
+    uint64_t radm1, topp;
+    int J;
+};
+
+// Step s = 1, 2, ... of the reflected mixed-radix Gray code over the low digits
+// (the step that leads to term s), without the steps before it: the digit that
+// moves is the lowest nonzero digit of s in these radices, and it moves up when
+// the number formed by the digits above it is even (a digit sweeps up and
+// down in turn).  weight = prod_d C(top_d, g_d) at term s, if wanted.
+// Returns the digit (0 where s is a multiple of the chunk's length).
+__host__ __device__ __forceinline__ int gray_step_at(const LowDigits& lo, uint32_t s, bool weights,
+                                                    bool& up, uint64_t& weight)
+{
+    uint64_t r1 = lo.radm1, tp = lo.topp;
+    uint32_t x = s;
+    int digit = -1;
+    up = true;
+    weight = 1;
+    for (int d = 0; d < lo.J; ++d) {
+        const uint32_t r = (uint32_t)(r1 & 15u) + 1u;
+        const uint32_t q = r == 2u ? x >> 1 : x / r;
+        const uint32_t v = x - q * r;
+        if (digit < 0 && v != 0) {
+            digit = d;
+            up = (q & 1u) == 0;
+            if (!weights)
+                break;
+        }
+        if (weights) {
+            const int g = (int)((q & 1u) ? r - 1u - v : v), top = (int)(tp & 15u);
+            if (g > 0 && g < top)
+                weight *= top <= 3 ? (uint64_t)top : binom_small(top, g);
+        }
+        x = q;
+        r1 >>= 4;
+        tp >>= 4;
+    }
+    return digit < 0 ? 0 : digit;
+}
+
 }  // namespace pqi
