@@ -31,6 +31,16 @@
 // Sturm-count bisection on the Jacobi matrix of He_N, and the kernel
 // multiplies the factors in pairs: 2 FP64 operations per unit of N instead
 // of Horner's 5.
+//
+// The walk runs in 64-bit block integers (pq_blockint.cuh) on the integer
+// pipes, as the permanent's does: q, y and l are scaled integers (every update
+// is exact), the powers and polynomial factors are products of limbs, and FP64
+// takes one conversion and one fused add per term and component.  All sums are
+// taken modulo 2^64: only q and l themselves have to stay in range.  In FP64
+// the walk was bound by the FP64 pipe (85 to 90% active): (2, ..., 2) at
+// N = 36 took 19.1 ms (hafnian), N = 28 with loops 1.68 ms.  A matrix
+// without a scale (non-finite or subnormal entries, a bound beyond FP64) is
+// walked in FP64.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -40,6 +50,7 @@
 #include <vector>
 
 #include "../../include/pq.h"
+#include "pq_blockint.cuh"
 #include "pq_device.cuh"
 #include "pq_fixsum.cuh"
 #include "pq_kernels.h"
@@ -47,6 +58,11 @@
 namespace pqi {
 
 constexpr int kHafMaxHalf = PQ_MAX_N / 2;  // loop-polynomial factors j = 1 .. N/2
+// integers of a loop polynomial of J = N/2 roots: 3 a pair, 2 for an odd root
+__host__ __device__ constexpr int haf_integers(int J) { return 3 * (J / 2) + 2 * (J % 2); }
+constexpr int kHafMaxInts = 40;
+static_assert(haf_integers(kHafMaxHalf) <= kHafMaxInts && haf_integers(kHafMaxHalf - 1) <= kHafMaxInts,
+              "room for the integers of every loop polynomial");
 
 // Per (loop) hafnian: k kept base indices, digits as for the permanent.
 struct alignas(16) HafDesc {
@@ -66,19 +82,21 @@ struct HafArgs {
     int64_t ntasks;
     const double2* src;
     const double2* gamma;  // loop weights (loop hafnian only)
-    const double* loopc;   // loop-polynomial factors per distinct N (loop hafnian only)
+    const double* loopc;   // loop-polynomial factors per distinct N (loop hafnian only):
+                           // J + 1 doubles, then the integers of loop_integers
     double2* out;
     double* partials;
     int32_t* counters;
 };
 
 // Shared memory of one warp: M (k x k), y0 = B r (k), gamma (k), y (k x 32,
-// lane-major), y at the low rows (J x 32, lane-major), B restricted to the
-// low rows (J x J), Horner coefficients, low-digit rows.
-__host__ __device__ inline int haf_warp_smem_bytes(int kmax, int jmax)
+// lane-major), loop-polynomial factors (doubles and integers).  The planner
+// puts the rows of the low digits first, so the walk's y and B at the low rows
+// are the first J rows of these.
+__host__ __device__ inline int haf_warp_smem_bytes(int kmax)
 {
-    int bytes = (kmax * kmax + 2 * kmax + 32 * kmax + 32 * jmax + jmax * jmax) * 16 +
-                (kHafMaxHalf + 1) * 8 + 16 * 4;
+    const int bytes = (kmax * kmax + 2 * kmax + 32 * kmax) * 16 +
+                      (kHafMaxHalf + 1 + kHafMaxInts) * 8;
     return (bytes + 15) & ~15;
 }
 
@@ -148,235 +166,649 @@ __device__ __forceinline__ double2 loop_poly(double2 q, double2 l, int P, const 
     return h;
 }
 
+// The pieces of a warp's shared memory; doubles for the FP64 walk, scaled
+// integers for the other.
+struct HafSmem {
+    double2* M;    // k x k: b (FP64), 2 b (integers)
+    double2* y0;   // k: B r
+    double2* gam;  // k
+    double2* Y;    // k x 32, lane-major
+    double* cj;    // loop-polynomial factors
+    int64_t* ci;   // and their integers
+    __device__ HafSmem(unsigned char* raw, int kmax)
+    {
+        M = reinterpret_cast<double2*>(raw);
+        y0 = M + kmax * kmax;
+        gam = y0 + kmax;
+        Y = gam + kmax;
+        cj = reinterpret_cast<double*>(Y + 32 * kmax);
+        ci = reinterpret_cast<int64_t*>(cj + kHafMaxHalf + 1);
+    }
+};
+
+// Integer metadata of one item.
+struct HafMeta {
+    const int32_t *ridx, *rmul, *drow, *drad, *dtop;
+    __device__ HafMeta(const HafArgs& a, const HafDesc& D)
+    {
+        ridx = a.meta + D.meta;
+        rmul = ridx + D.k;
+        drow = rmul + D.k;
+        drad = drow + D.ndig;
+        dtop = drad + D.ndig;
+    }
+};
+
+// What a warp keeps about the item it has staged.
+struct HafStaged {
+    int item = -1;
+    bool fp64 = false;  // staged as doubles
+    int exp2 = 0;       // the terms' sum times 2^exp2 is the sum of s(g) times the polynomial
+    int eq = 0, el = 0; // q and l times 2^eq, 2^el are the integers
+    int xref = 0;       // loop hafnian: upper bound of the exponent q and s are aligned to
+};
+
+// The walk of this lane's chunk in FP64; returns the task's sum.
 template <bool LOOP>
-__device__ void haf_task(const HafArgs& a, const Task& t, unsigned char* raw, int kmax, int jmax,
-                         int& staged, int lane)
+__device__ __noinline__ dd2 haf_walk_fp64(const HafDesc& D, const HafMeta& mt, const HafSmem& sm,
+                                  int64_t c, bool active, int lane)
 {
-    const HafDesc D = a.desc[t.perm];
     const int k = D.k, J = D.J, nd = D.ndig;
-    double2* M = reinterpret_cast<double2*>(raw);
-    double2* y0 = M + kmax * kmax;
-    double2* gam = y0 + kmax;
-    double2* Y = gam + kmax;
-    double2* YL = Y + 32 * kmax;
-    double2* Bll = YL + 32 * jmax;
-    double* cj = reinterpret_cast<double*>(Bll + jmax * jmax);
-    int32_t* lowrow = reinterpret_cast<int32_t*>(cj + kHafMaxHalf + 1);
-    const int32_t* ridx = a.meta + D.meta;
-    const int32_t* rmul = ridx + k;
-    const int32_t* drow = rmul + k;
-    const int32_t* drad = drow + nd;
-    const int32_t* dtop = drad + nd;
-    dd2 res = {0.0, 0.0, 0.0, 0.0};
+    const double2 *M = sm.M, *y0 = sm.y0, *gam = sm.gam;
+    const double* cj = sm.cj;
+    const int32_t *rmul = mt.rmul, *drow = mt.drow, *drad = mt.drad, *dtop = mt.dtop;
+    dd2 res;
+    const int64_t c_first = c;
+    double2* y = sm.Y + lane;
+#pragma unroll 1
+    for (int j = 0; j < k; ++j)
+        y[j * 32] = y0[j];
+    // High digits of this lane's chunk: x_row = r_row - 2 g.  y = B x is
+    // finished before x^T y is formed in a second pass over the digits.
+    uint64_t whigh_u = 1;
+    int gpar = 0;
+#pragma unroll 1
+    for (int d = J; d < nd; ++d) {
+        const int rad = drad[d];
+        const int g = (int)(c % rad);
+        c /= rad;
+        if (!g)
+            continue;
+        const int row = drow[d];
+        const double coef = (double)(-2 * g);
+#pragma unroll 1
+        for (int j = 0; j < k; ++j) {
+            const double2 b = M[j * k + row];
+            double2 v = y[j * 32];
+            v.x = __fma_rn(coef, b.x, v.x);
+            v.y = __fma_rn(coef, b.y, v.y);
+            y[j * 32] = v;
+        }
+        whigh_u *= binom_u64(dtop[d], g);
+        gpar += g;
+    }
+    // q = 1/2 (x^T y - sum_i r_i B_ii) and l = gamma^T x, low digits at 0
+    double2 q = make_double2(0.0, 0.0), l = make_double2(0.0, 0.0);
+#pragma unroll 1
+    for (int i = 0; i < k; ++i) {
+        const double2 v = y[i * 32];
+        const double2 bii = M[i * k + i];
+        const double r = (double)rmul[i];
+        q.x = __fma_rn(r, __dsub_rn(v.x, bii.x), q.x);
+        q.y = __fma_rn(r, __dsub_rn(v.y, bii.y), q.y);
+        if (LOOP) {
+            l.x = __fma_rn(r, gam[i].x, l.x);
+            l.y = __fma_rn(r, gam[i].y, l.y);
+        }
+    }
+    c = c_first;
+#pragma unroll 1
+    for (int d = J; d < nd; ++d) {
+        const int rad = drad[d];
+        const int g = (int)(c % rad);
+        c /= rad;
+        if (!g)
+            continue;
+        const int row = drow[d];
+        const double2 v = y[row * 32];
+        const double coef = (double)(-2 * g);
+        q.x = __fma_rn(coef, v.x, q.x);
+        q.y = __fma_rn(coef, v.y, q.y);
+        if (LOOP) {
+            l.x = __fma_rn(coef, gam[row].x, l.x);
+            l.y = __fma_rn(coef, gam[row].y, l.y);
+        }
+    }
+    q.x *= 0.5;
+    q.y *= 0.5;
+    double2* yl = y;  // rows 0 .. J - 1
+    double whigh = active ? (double)whigh_u : 0.0;
+    if (gpar & 1)
+        whigh = -whigh;
 
-    if (!D.trivial) {
-        if (staged != t.perm) {
-            __syncwarp();
-            for (int e = lane; e < k * k; e += kWarp) {
-                const int i = e / k, j = e - i * k;
-                M[e] = a.src[D.src_off + (int64_t)ridx[i] * D.ld + ridx[j]];
-            }
-            for (int d = lane; d < J; d += kWarp)
-                lowrow[d] = drow[d];
-            if (LOOP) {
-                for (int i = lane; i < k; i += kWarp)
-                    gam[i] = a.gamma[D.gam_off + ridx[i]];
-                for (int j = lane; j <= D.N / 2; j += kWarp)
-                    cj[j] = a.loopc[D.coef_off + j];
-            }
-            __syncwarp();
-            for (int e = lane; e < J * J; e += kWarp) {  // B at the low rows
-                const int u = e / J, v = e - u * J;
-                Bll[e] = M[lowrow[u] * k + lowrow[v]];
-            }
-            for (int j = lane; j < k; j += kWarp) {  // y0 = B r
-                double2 s = make_double2(0.0, 0.0);
-                for (int i = 0; i < k; ++i) {
-                    const double r = (double)rmul[i];
-                    s.x = __fma_rn(r, M[j * k + i].x, s.x);
-                    s.y = __fma_rn(r, M[j * k + i].y, s.y);
-                }
-                y0[j] = s;
-            }
-            __syncwarp();
-            staged = t.perm;
-        }
-        const int64_t chunk0 = (int64_t)t.part * kWarp;
-        const bool active = chunk0 + lane < D.nchunks;
-        int64_t c = active ? (chunk0 + lane) : 0;
-        const int64_t c_first = c;
-        double2* y = Y + lane;
-#pragma unroll 1
-        for (int j = 0; j < k; ++j)
-            y[j * 32] = y0[j];
-        // High digits of this lane's chunk: x_row = r_row - 2 g.  y = B x is
-        // finished before x^T y is formed in a second pass over the digits.
-        uint64_t whigh_u = 1;
-        int gpar = 0;
-#pragma unroll 1
-        for (int d = J; d < nd; ++d) {
-            const int rad = drad[d];
-            const int g = (int)(c % rad);
-            c /= rad;
-            if (!g)
-                continue;
-            const int row = drow[d];
-            const double coef = (double)(-2 * g);
-#pragma unroll 1
-            for (int j = 0; j < k; ++j) {
-                const double2 b = M[j * k + row];
-                double2 v = y[j * 32];
-                v.x = __fma_rn(coef, b.x, v.x);
-                v.y = __fma_rn(coef, b.y, v.y);
-                y[j * 32] = v;
-            }
-            whigh_u *= binom_u64(dtop[d], g);
-            gpar += g;
-        }
-        // q = 1/2 (x^T y - sum_i r_i B_ii) and l = gamma^T x, low digits at 0
-        double2 q = make_double2(0.0, 0.0), l = make_double2(0.0, 0.0);
-#pragma unroll 1
-        for (int i = 0; i < k; ++i) {
-            const double2 v = y[i * 32];
-            const double2 bii = M[i * k + i];
-            const double r = (double)rmul[i];
-            q.x = __fma_rn(r, __dsub_rn(v.x, bii.x), q.x);
-            q.y = __fma_rn(r, __dsub_rn(v.y, bii.y), q.y);
-            if (LOOP) {
-                l.x = __fma_rn(r, gam[i].x, l.x);
-                l.y = __fma_rn(r, gam[i].y, l.y);
+    LowWalk wk;
+    wk.v = 0;
+    wk.g = 0;
+    wk.dir = 0;
+    wk.radm1 = 0;
+    wk.topp = 0;
+    for (int d = 0; d < J; ++d) {
+        wk.radm1 |= uint64_t(drad[d] - 1) << (4 * d);
+        wk.topp |= uint64_t(dtop[d]) << (4 * d);
+    }
+    const bool weighted = D.weighted != 0;
+    const int n = D.n, N = D.N;
+    const int form = ((N >> 1) & 1) * 2 + (N & 1), P = N >> 2;
+    double wlow = 1.0;
+    double2 acc = make_double2(0.0, 0.0);
+    double rh = 0.0, rl = 0.0, ih = 0.0, il = 0.0;
+    const int64_t L = D.L;
+    // The term's polynomial value; the uniform switches pick straight-line
+    // code for the exponent or the loop-polynomial shape, so no FP64
+    // instruction is issued under a false predicate.
+    auto value = [&]() -> double2 {
+        if (LOOP) {
+            switch (form) {
+            case 0: return loop_poly<false, false>(q, l, P, cj);
+            case 1: return loop_poly<false, true>(q, l, P, cj);
+            case 2: return loop_poly<true, false>(q, l, P, cj);
+            default: return loop_poly<true, true>(q, l, P, cj);
             }
         }
-        c = c_first;
-#pragma unroll 1
-        for (int d = J; d < nd; ++d) {
-            const int rad = drad[d];
-            const int g = (int)(c % rad);
-            c /= rad;
-            if (!g)
-                continue;
-            const int row = drow[d];
-            const double2 v = y[row * 32];
-            const double coef = (double)(-2 * g);
-            q.x = __fma_rn(coef, v.x, q.x);
-            q.y = __fma_rn(coef, v.y, q.y);
-            if (LOOP) {
-                l.x = __fma_rn(coef, gam[row].x, l.x);
-                l.y = __fma_rn(coef, gam[row].y, l.y);
-            }
+        return cpow_n(q, n);
+    };
+    auto term_pos = [&]() {
+        const double2 p = value();
+        acc.x = __fma_rn(wlow, p.x, acc.x);
+        acc.y = __fma_rn(wlow, p.y, acc.y);
+    };
+    auto term_neg = [&]() {
+        const double2 p = value();
+        acc.x = __fma_rn(-wlow, p.x, acc.x);
+        acc.y = __fma_rn(-wlow, p.y, acc.y);
+    };
+    // One Gray step: x_row moves by -+2.
+    auto step = [&]() {
+        int up;
+        const int d = low_step(wk, up);
+        const double delta = up > 0 ? -2.0 : 2.0;
+        const double2 yr = yl[d * 32];
+        const double2* Bd = M + d * k;
+        const double2 brr = Bd[d];
+        q.x = __fma_rn(delta, yr.x, q.x);
+        q.y = __fma_rn(delta, yr.y, q.y);
+        q.x = __fma_rn(2.0, brr.x, q.x);
+        q.y = __fma_rn(2.0, brr.y, q.y);
+        if (LOOP) {
+            const double2 gr = gam[d];
+            l.x = __fma_rn(delta, gr.x, l.x);
+            l.y = __fma_rn(delta, gr.y, l.y);
         }
-        q.x *= 0.5;
-        q.y *= 0.5;
-        double2* yl = YL + lane;
 #pragma unroll 1
-        for (int e = 0; e < J; ++e)
-            yl[e * 32] = y[lowrow[e] * 32];
-        double whigh = active ? (double)whigh_u : 0.0;
-        if (gpar & 1)
-            whigh = -whigh;
-
-        LowWalk wk;
-        wk.v = 0;
-        wk.g = 0;
-        wk.dir = 0;
-        wk.radm1 = 0;
-        wk.topp = 0;
-        for (int d = 0; d < J; ++d) {
-            wk.radm1 |= uint64_t(drad[d] - 1) << (4 * d);
-            wk.topp |= uint64_t(dtop[d]) << (4 * d);
+        for (int e = 0; e < J; ++e) {
+            const double2 b = Bd[e];
+            double2 v = yl[e * 32];
+            v.x = __fma_rn(delta, b.x, v.x);
+            v.y = __fma_rn(delta, b.y, v.y);
+            yl[e * 32] = v;
         }
-        const bool weighted = D.weighted != 0;
-        const int n = D.n, N = D.N;
-        const int form = ((N >> 1) & 1) * 2 + (N & 1), P = N >> 2;
-        double wlow = 1.0;
-        double2 acc = make_double2(0.0, 0.0);
-        double rh = 0.0, rl = 0.0, ih = 0.0, il = 0.0;
-        const int64_t L = D.L;
-        // The term's polynomial value; the uniform switches pick straight-line
-        // code for the exponent or the loop-polynomial shape, so no FP64
-        // instruction is issued under a false predicate.
-        auto value = [&]() -> double2 {
-            if (LOOP) {
-                switch (form) {
-                case 0: return loop_poly<false, false>(q, l, P, cj);
-                case 1: return loop_poly<false, true>(q, l, P, cj);
-                case 2: return loop_poly<true, false>(q, l, P, cj);
-                default: return loop_poly<true, true>(q, l, P, cj);
-                }
-            }
-            return cpow_n(q, n);
-        };
-        auto term_pos = [&]() {
-            const double2 p = value();
-            acc.x = __fma_rn(wlow, p.x, acc.x);
-            acc.y = __fma_rn(wlow, p.y, acc.y);
-        };
-        auto term_neg = [&]() {
-            const double2 p = value();
-            acc.x = __fma_rn(-wlow, p.x, acc.x);
-            acc.y = __fma_rn(-wlow, p.y, acc.y);
-        };
-        // One Gray step: x_row moves by -+2.
-        auto step = [&]() {
-            int up;
-            const int d = low_step(wk, up);
-            const double delta = up > 0 ? -2.0 : 2.0;
-            const double2 yr = yl[d * 32];
-            const double2* Bd = Bll + d * J;
-            const double2 brr = Bd[d];
-            q.x = __fma_rn(delta, yr.x, q.x);
-            q.y = __fma_rn(delta, yr.y, q.y);
-            q.x = __fma_rn(2.0, brr.x, q.x);
-            q.y = __fma_rn(2.0, brr.y, q.y);
-            if (LOOP) {
-                const double2 gr = gam[lowrow[d]];
-                l.x = __fma_rn(delta, gr.x, l.x);
-                l.y = __fma_rn(delta, gr.y, l.y);
-            }
+        if (weighted && ((wk.radm1 >> (4 * d)) & 15u) > 1u)
+            wlow = (double)low_weight(wk, J);
+    };
+    // Term 0 has sign +; then pairs (odd: -, even: +), folded into the
+    // double-double sums every 16 terms by the outer loop.
+    term_pos();
+    int64_t s = 1;
 #pragma unroll 1
-            for (int e = 0; e < J; ++e) {
-                const double2 b = Bd[e];
-                double2 v = yl[e * 32];
-                v.x = __fma_rn(delta, b.x, v.x);
-                v.y = __fma_rn(delta, b.y, v.y);
-                yl[e * 32] = v;
-            }
-            if (weighted && ((wk.radm1 >> (4 * d)) & 15u) > 1u)
-                wlow = (double)low_weight(wk, J);
-        };
-        // Term 0 has sign +; then pairs (odd: -, even: +), folded into the
-        // double-double sums every 16 terms by the outer loop.
-        term_pos();
-        int64_t s = 1;
+    while (s < L) {
+        const int npairs = (int)min((L - s) >> 1, (int64_t)8);
 #pragma unroll 1
-        while (s < L) {
-            const int npairs = (int)min((L - s) >> 1, (int64_t)8);
-#pragma unroll 1
-            for (int i = 0; i < npairs; ++i) {
-                step();
-                term_neg();
-                step();
-                term_pos();
-            }
-            s += 2 * npairs;
-            if (npairs == 0) {  // one (odd) term left
-                step();
-                term_neg();
-                s += 1;
-            }
-            dd_acc(rh, rl, acc.x);
-            dd_acc(ih, il, acc.y);
-            acc = make_double2(0.0, 0.0);
+        for (int i = 0; i < npairs; ++i) {
+            step();
+            term_neg();
+            step();
+            term_pos();
+        }
+        s += 2 * npairs;
+        if (npairs == 0) {  // one (odd) term left
+            step();
+            term_neg();
+            s += 1;
         }
         dd_acc(rh, rl, acc.x);
         dd_acc(ih, il, acc.y);
-        fast_two_sum(rh, rl, rh, rl);
-        fast_two_sum(ih, il, ih, il);
-        dd_mul_d(rh, rl, whigh);
-        dd_mul_d(ih, il, whigh);
-        // the lanes' sums added exactly in integers (pq_fixsum.cuh)
-        warp_fix_sum(rh, rl, res.rh, res.rl);
-        warp_fix_sum(ih, il, res.ih, res.il);
+        acc = make_double2(0.0, 0.0);
+    }
+    dd_acc(rh, rl, acc.x);
+    dd_acc(ih, il, acc.y);
+    fast_two_sum(rh, rl, rh, rl);
+    fast_two_sum(ih, il, ih, il);
+    dd_mul_d(rh, rl, whigh);
+    dd_mul_d(ih, il, whigh);
+    // the lanes' sums added exactly in integers (pq_fixsum.cuh)
+    warp_fix_sum(rh, rl, res.rh, res.rl);
+    warp_fix_sum(ih, il, res.ih, res.il);
+    return res;
+}
+
+// Stage item D as scaled integers: M = 2 b, y0 = B r, gam.  Returns false (nothing converted) if the item has no scale.
+template <bool LOOP>
+__device__ bool haf_stage_int(const HafDesc& D, const HafMeta& mt, const HafSmem& sm, HafStaged& st,
+                              int lane)
+{
+    const int k = D.k;
+    bool bad = false;
+    uint32_t hmax = 0, gmax = 0;
+    for (int e = lane; e < k * k; e += kWarp)
+        hmax = max(hmax, bint_mag(sm.M[e].x, sm.M[e].y));
+    hmax = __reduce_max_sync(0xffffffffu, hmax);
+    // |q| <= 1/2 (sum_ij r_i r_j |b_ij| + sum_i r_i |b_ii|)
+    uint64_t units = 0;
+    for (int i = lane; i < k; i += kWarp) {
+        uint32_t row = 0;
+        for (int j = 0; j < k; ++j)
+            row += (uint32_t)(mt.rmul[j] + (j == i ? 1 : 0)) *
+                   bint_units(bint_mag(sm.M[i * k + j].x, sm.M[i * k + j].y), hmax);
+        units += (uint64_t)mt.rmul[i] * row;
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1)
+        units += __shfl_xor_sync(0xffffffffu, units, off);
+    units += (units >> 20) + 1;  // the rounding of the entries stays inside the bound
+    const int eq = kSumBits + 1044 - (int)(hmax >> 20) - bint_width(units);
+    bad = hmax < 0x100000u || hmax >= 0x7ff00000u || eq < kSumBits - 1023;
+    int el = 0;
+    if (LOOP) {
+        bool nonzero = false;
+        for (int i = lane; i < k; i += kWarp) {
+            gmax = max(gmax, bint_mag(sm.gam[i].x, sm.gam[i].y));
+            nonzero = nonzero || sm.gam[i].x != 0.0 || sm.gam[i].y != 0.0;
+        }
+        gmax = __reduce_max_sync(0xffffffffu, gmax);
+        uint32_t gu = 0;
+        for (int i = lane; i < k; i += kWarp)
+            gu += (uint32_t)mt.rmul[i] * bint_units(bint_mag(sm.gam[i].x, sm.gam[i].y), gmax);
+        gu = __reduce_add_sync(0xffffffffu, gu);
+        if (__any_sync(0xffffffffu, nonzero)) {
+            el = bint_scale(gmax, gu);
+            bad = bad || gmax < 0x100000u || gmax >= 0x7ff00000u || el < kSumBits - 1023;
+        }
+    }
+    if (bad)
+        return false;
+    longlong2* M = reinterpret_cast<longlong2*>(sm.M);
+    longlong2* y0 = reinterpret_cast<longlong2*>(sm.y0);
+    longlong2* gam = reinterpret_cast<longlong2*>(sm.gam);
+    for (int e = lane; e < k * k; e += kWarp) {
+        const double2 b = sm.M[e];
+        M[e] = make_longlong2(2 * bint_of(b.x, eq), 2 * bint_of(b.y, eq));
+    }
+    if (LOOP) {
+        for (int i = lane; i < k; i += kWarp) {
+            const double2 b = sm.gam[i];
+            gam[i] = make_longlong2(bint_of(b.x, el), bint_of(b.y, el));
+        }
+    }
+    __syncwarp();
+    for (int j = lane; j < k; j += kWarp) {
+        uint64_t x = 0, y = 0;
+        for (int i = 0; i < k; ++i) {
+            const longlong2 b = M[j * k + i];
+            x += (uint64_t)mt.rmul[i] * (uint64_t)(b.x >> 1);
+            y += (uint64_t)mt.rmul[i] * (uint64_t)(b.y >> 1);
+        }
+        y0[j] = make_longlong2((long long)x, (long long)y);
+    }
+    __syncwarp();
+    st.eq = eq;
+    st.el = el;
+    if (LOOP) {
+        // P pairs at 2 X + 64, an odd root at X, an odd N at -el; 64 per product
+        const int P = D.N >> 2, jo = (D.N >> 1) & 1, no = D.N & 1;
+        const int parts = P + jo + no;
+        st.xref = 1 + (P + jo > 0 ? max(-eq, 64 - 2 * el + (int)sm.ci[0]) : 0);
+        st.exp2 = kSumBits + 64 * (P + parts - 1) + (2 * P + jo) * st.xref - no * el;
+    } else {
+        st.exp2 = kSumBits + 64 * (D.n - 1) - D.n * eq;
+    }
+    return true;
+}
+
+__device__ __forceinline__ BInt bint_words(longlong2 s)
+{
+    BInt p;
+    p.rh = (int)(s.x >> 32);
+    p.rl = (uint32_t)s.x;
+    p.ih = (int)(s.y >> 32);
+    p.il = (uint32_t)s.y;
+    return p;
+}
+
+__device__ __forceinline__ longlong2 bint_pair(const BInt& p)
+{
+    return make_longlong2((long long)(((uint64_t)(uint32_t)p.rh << 32) | p.rl),
+                          (long long)(((uint64_t)(uint32_t)p.ih << 32) | p.il));
+}
+
+// q^n, n >= 1 (binary method from the top bit; n is uniform): the integers,
+// normalised except after the last product, and their exponent E.
+__device__ __forceinline__ BInt haf_power(longlong2 q, int n, int& E)
+{
+    BInt x = bint_words(q);
+    int Ex = 0;
+    bnorm(x, Ex);
+    const BLimbs lx = limbs(x);
+    BInt h = x;
+    E = Ex;
+#pragma unroll 1
+    for (int bit = 30 - __clz(n); bit >= 0; --bit) {
+        const BLimbs lh = limbs(h);
+        h = bmul(lh, lh);
+        E *= 2;
+        bnorm(h, E);
+        if ((n >> bit) & 1) {
+            h = bmul(limbs(h), lx);
+            E += Ex;
+            bnorm(h, E);
+        }
+    }
+    return h;
+}
+
+// 2 (c v >> 64) of a real 0 <= c < 2^63, the product of v and c 2^-63.
+__device__ __forceinline__ longlong2 real_scale(int64_t c, const BLimbs& v)
+{
+    const int ch = (int)((c + kSumBias) >> 32), cl = (int)(uint32_t)c;
+    const int64_t mr = mulw(v.a, cl) + mulw(v.b, ch), mi = mulw(v.c, cl) + mulw(v.d, ch);
+    const int64_t hr = mulw(v.a, ch) + (int64_t)(int)(mr >> 32);
+    const int64_t hi = mulw(v.c, ch) + (int64_t)(int)(mi >> 32);
+    return make_longlong2(2 * hr, 2 * hi);
+}
+
+__device__ __forceinline__ longlong2 shift_right(longlong2 v, int n)
+{
+    return make_longlong2(v.x >> n, v.y >> n);
+}
+
+// The loop polynomial of q and l without its leading factor: P pairs of roots
+// q^2 + a q s + b s^2 with s = l^2, an odd root q + c s, an odd N one factor l.
+// The roots spread over two decades, so every pair has its own scale 2^kp of
+// s (ci: kp, a 2^-kp, b 2^-2kp of each pair, kp and c 2^-kp of an odd root, all
+// coefficients at most 1), and its three terms are brought to the larger of
+// the exponents of q^2 and (2^kp s)^2: whichever of q and s is large, a factor
+// keeps its bits.  E counts the exponents against xref, their upper bound.
+__device__ __forceinline__ BInt haf_loop_poly(longlong2 q, longlong2 l, int P, bool jodd, bool nodd,
+                                              const int64_t* ci, const HafStaged& st, int& E)
+{
+    BInt lw = bint_words(l), h;
+    int El = 0;
+    bnorm(lw, El);
+    E = 0;
+    bool first = true;
+    if (P > 0 || jodd) {
+        BInt qw = bint_words(q);
+        int Eq = 0;
+        bnorm(qw, Eq);
+        const BLimbs ll = limbs(lw);
+        BInt sw = bmul(ll, ll);
+        int Es = 0;
+        bnorm(sw, Es);
+        // one bit down, so that a factor stays below 2^62
+        const longlong2 qv = shift_right(bint_pair(qw), 1), sv = shift_right(bint_pair(sw), 1);
+        constexpr int kNone = -(1 << 20);  // exponent of an exact zero
+        const int xq = (qv.x | qv.y) == 0 ? kNone : 1 - st.eq - Eq;
+        const int xs = (sv.x | sv.y) == 0 ? kNone : 65 - 2 * (st.el + El) - Es;
+        const BLimbs lq = limbs(bint_words(qv)), ls = limbs(bint_words(sv));
+        if (P > 0) {
+            const longlong2 q2 = bint_pair(bmul(lq, lq));
+            const BLimbs qs = limbs(bmul(lq, ls)), s2 = limbs(bmul(ls, ls));
+#pragma unroll 1
+            for (int p = 0; p < P; ++p) {
+                const int64_t* c = ci + 3 * p;
+                const int y = xs + (int)c[0], n = min(abs(xq - y), 63), n2 = min(2 * n, 63);
+                const longlong2 t0 = shift_right(q2, xq < y ? n2 : 0);
+                const longlong2 t1 = shift_right(real_scale(c[1], qs), n);
+                const longlong2 t2 = shift_right(real_scale(c[2], s2), xq < y ? 0 : n2);
+                const BInt t = bint_words(make_longlong2(t0.x + t1.x + t2.x, t0.y + t1.y + t2.y));
+                h = first ? t : bmul(limbs(h), limbs(t));
+                first = false;
+                E += 2 * (st.xref - max(max(xq, y), kNone / 2));
+                bnorm(h, E);
+            }
+        }
+        if (jodd) {
+            const int64_t* c = ci + 3 * P;
+            const int y = xs + (int)c[0], n = min(abs(xq - y), 63);
+            const longlong2 t0 = shift_right(qv, xq < y ? n : 0);
+            const longlong2 t1 = shift_right(real_scale(c[1], ls), xq < y ? 0 : n);
+            const BInt t = bint_words(make_longlong2(t0.x + t1.x, t0.y + t1.y));
+            h = first ? t : bmul(limbs(h), limbs(t));
+            first = false;
+            E += st.xref - max(max(xq, y), kNone / 2);
+            bnorm(h, E);
+        }
+    }
+    if (nodd) {
+        h = first ? lw : bmul(limbs(h), limbs(lw));
+        E += El;
+    }
+    return h;
+}
+
+// The walk of this lane's chunk in block integers; returns the task's sum.
+// All sums are taken modulo 2^64 (unsigned): y may leave the range of 64 bits,
+// q and l do not.
+template <bool LOOP>
+__device__ __forceinline__ dd2 haf_walk_int(const HafDesc& D, const HafMeta& mt, const HafSmem& sm,
+                                            const HafStaged& st, int64_t c, bool active, int lane)
+{
+    const int k = D.k, J = D.J, nd = D.ndig;
+    const ulonglong2* M = reinterpret_cast<const ulonglong2*>(sm.M);
+    const ulonglong2* y0 = reinterpret_cast<const ulonglong2*>(sm.y0);
+    const ulonglong2* gam = reinterpret_cast<const ulonglong2*>(sm.gam);
+    ulonglong2* y = reinterpret_cast<ulonglong2*>(sm.Y) + lane;
+    // High digits of this lane's chunk: x_row = r_row - 2 g.  y = B x is
+    // finished before x^T y is formed in a second pass over the digits.
+#pragma unroll 1
+    for (int j = 0; j < k; ++j)
+        y[j * 32] = y0[j];
+    uint64_t whigh_u = 1;
+    int gpar = 0;
+    int64_t cc = c;
+#pragma unroll 1
+    for (int d = J; d < nd; ++d) {
+        const int g = (int)(cc % mt.drad[d]);
+        cc /= mt.drad[d];
+        if (!g)
+            continue;
+        const ulonglong2* Mr = M + mt.drow[d];
+#pragma unroll 1
+        for (int j = 0; j < k; ++j) {
+            const ulonglong2 b = Mr[j * k];
+            ulonglong2 v = y[j * 32];
+            v.x -= (uint64_t)g * b.x;
+            v.y -= (uint64_t)g * b.y;
+            y[j * 32] = v;
+        }
+        whigh_u *= binom_u64(mt.dtop[d], g);
+        gpar += g;
+    }
+    // 2 q = x^T y - sum_i r_i B_ii and l = gamma^T x, low digits at 0
+    ulonglong2 q = make_ulonglong2(0, 0), l = make_ulonglong2(0, 0);
+#pragma unroll 1
+    for (int i = 0; i < k; ++i) {
+        const ulonglong2 v = y[i * 32], bii = M[i * k + i];
+        const uint64_t r = (uint64_t)mt.rmul[i];
+        q.x += r * (v.x - (uint64_t)((int64_t)bii.x >> 1));
+        q.y += r * (v.y - (uint64_t)((int64_t)bii.y >> 1));
+        if (LOOP) {
+            l.x += r * gam[i].x;
+            l.y += r * gam[i].y;
+        }
+    }
+    cc = c;
+#pragma unroll 1
+    for (int d = J; d < nd; ++d) {
+        const int g = (int)(cc % mt.drad[d]);
+        cc /= mt.drad[d];
+        if (!g)
+            continue;
+        const int row = mt.drow[d];
+        const ulonglong2 v = y[row * 32];
+        q.x -= 2 * (uint64_t)g * v.x;
+        q.y -= 2 * (uint64_t)g * v.y;
+        if (LOOP) {
+            l.x -= 2 * (uint64_t)g * gam[row].x;
+            l.y -= 2 * (uint64_t)g * gam[row].y;
+        }
+    }
+    q.x = (uint64_t)((int64_t)q.x >> 1);
+    q.y = (uint64_t)((int64_t)q.y >> 1);
+
+    LowDigits lo;
+    lo.radm1 = lo.topp = 0;
+    lo.J = J;
+    for (int d = 0; d < J; ++d) {
+        lo.radm1 |= uint64_t(mt.drad[d] - 1) << (4 * d);
+        lo.topp |= uint64_t(mt.dtop[d]) << (4 * d);
+    }
+    const bool weighted = D.weighted != 0;
+    const int n = D.n, P = D.N >> 2;
+    const bool jodd = ((D.N >> 1) & 1) != 0, nodd = (D.N & 1) != 0;
+    uint32_t steps = 0;
+    double step_w = 1.0, w = 1.0;
+    double2 acc = make_double2(0.0, 0.0);
+    double rh = 0.0, rl = 0.0, ih = 0.0, il = 0.0;
+    const uint32_t L = (uint32_t)D.L;
+    uint32_t s = 0;
+#pragma unroll 1
+    for (;;) {
+        int E;
+        const longlong2 qs = make_longlong2((long long)q.x, (long long)q.y);
+        const BInt p =
+            LOOP ? haf_loop_poly(qs, make_longlong2((long long)l.x, (long long)l.y), P, jodd, nodd,
+                                 sm.ci, st, E)
+                 : haf_power(qs, n, E);
+        const longlong2 pv = bint_pair(p);
+        const double f = bint_factor(w, E, (s & 1u) != 0);
+        acc.x = __fma_rn(__ll2double_rn(pv.x), f, acc.x);
+        acc.y = __fma_rn(__ll2double_rn(pv.y), f, acc.y);
+        ++s;
+        if (s == L || (s & 15u) == 0) {
+            dd_acc(rh, rl, acc.x);
+            dd_acc(ih, il, acc.y);
+            acc = make_double2(0.0, 0.0);
+            if (s == L)
+                break;
+        }
+        // the Gray steps 32 at a time, one per lane, as in the permanent's walk
+        const int sq = (int)((s - 1u) & 31u);
+        if (sq == 0) {
+            bool up;
+            uint64_t wu;
+            const int d = gray_step_at(lo, s + (uint32_t)lane, weighted, up, wu);
+            steps = ((uint32_t)d << 1) | (up ? 0u : 1u);
+            step_w = (double)wu;
+        }
+        const uint32_t step = __shfl_sync(0xffffffffu, steps, sq);
+        if (weighted)
+            w = __shfl_sync(0xffffffffu, step_w, sq);
+        // x_d moves by -+2: q += -+2 y_d + 2 B_dd, then y moves by -+2 B
+        const int d = (int)(step >> 1);
+        const ulonglong2 yd = y[d * 32];
+        const ulonglong2* Bd = M + d * k;
+        const ulonglong2 bdd = Bd[d];
+        if (step & 1u) {
+            q.x += 2 * yd.x + bdd.x;
+            q.y += 2 * yd.y + bdd.y;
+#pragma unroll 1
+            for (int e = 0; e < J; ++e) {
+                const ulonglong2 b = Bd[e];
+                ulonglong2 v = y[e * 32];
+                v.x += b.x;
+                v.y += b.y;
+                y[e * 32] = v;
+            }
+            if (LOOP) {
+                l.x += 2 * gam[d].x;
+                l.y += 2 * gam[d].y;
+            }
+        } else {
+            q.x += bdd.x - 2 * yd.x;
+            q.y += bdd.y - 2 * yd.y;
+#pragma unroll 1
+            for (int e = 0; e < J; ++e) {
+                const ulonglong2 b = Bd[e];
+                ulonglong2 v = y[e * 32];
+                v.x -= b.x;
+                v.y -= b.y;
+                y[e * 32] = v;
+            }
+            if (LOOP) {
+                l.x -= 2 * gam[d].x;
+                l.y -= 2 * gam[d].y;
+            }
+        }
+    }
+    double whigh = active ? (double)whigh_u : 0.0;
+    if (gpar & 1)
+        whigh = -whigh;
+    fast_two_sum(rh, rl, rh, rl);
+    fast_two_sum(ih, il, ih, il);
+    dd_mul_d(rh, rl, whigh);
+    dd_mul_d(ih, il, whigh);
+    // the lanes' sums added exactly in integers (pq_fixsum.cuh)
+    dd2 res;
+    warp_fix_sum(rh, rl, res.rh, res.rl);
+    warp_fix_sum(ih, il, res.ih, res.il);
+    return res;
+}
+
+template <bool LOOP>
+__device__ void haf_task(const HafArgs& a, const Task& t, const HafSmem& sm, HafStaged& st, int lane)
+{
+    const HafDesc D = a.desc[t.perm];
+    const int k = D.k;
+    dd2 res = {0.0, 0.0, 0.0, 0.0};
+
+    if (!D.trivial) {
+        const HafMeta mt(a, D);
+        if (st.item != t.perm) {
+            __syncwarp();
+            for (int e = lane; e < k * k; e += kWarp) {
+                const int i = e / k, j = e - i * k;
+                sm.M[e] = a.src[D.src_off + (int64_t)mt.ridx[i] * D.ld + mt.ridx[j]];
+            }
+            if (LOOP) {
+                const int nf = D.N / 2 + 1;
+                for (int i = lane; i < k; i += kWarp)
+                    sm.gam[i] = a.gamma[D.gam_off + mt.ridx[i]];
+                for (int j = lane; j < nf; j += kWarp)
+                    sm.cj[j] = a.loopc[D.coef_off + j];
+                for (int j = lane; j < haf_integers(D.N / 2); j += kWarp)
+                    sm.ci[j] = __double_as_longlong(a.loopc[D.coef_off + nf + j]);
+            }
+            __syncwarp();
+            st.fp64 = !haf_stage_int<LOOP>(D, mt, sm, st, lane);
+            if (st.fp64) {
+                for (int j = lane; j < k; j += kWarp) {  // y0 = B r
+                    double2 s = make_double2(0.0, 0.0);
+                    for (int i = 0; i < k; ++i) {
+                        const double r = (double)mt.rmul[i];
+                        s.x = __fma_rn(r, sm.M[j * k + i].x, s.x);
+                        s.y = __fma_rn(r, sm.M[j * k + i].y, s.y);
+                    }
+                    sm.y0[j] = s;
+                }
+                __syncwarp();
+            }
+            st.item = t.perm;
+        }
+        const int64_t chunk0 = (int64_t)t.part * kWarp;
+        const bool active = chunk0 + lane < D.nchunks;
+        const int64_t c = active ? (chunk0 + lane) : 0;
+        res = st.fp64 ? haf_walk_fp64<LOOP>(D, mt, sm, c, active, lane)
+                      : haf_walk_int<LOOP>(D, mt, sm, st, c, active, lane);
     }
 
     auto finish = [&](dd2 v) {
@@ -384,11 +816,14 @@ __device__ void haf_task(const HafArgs& a, const Task& t, unsigned char* raw, in
         if (D.trivial) {
             o = make_double2(D.value, 0.0);
         } else {
+            // the FP64 walk's terms hold the loop polynomial's leading factor
+            const double f = LOOP && !st.fp64 ? D.value * sm.cj[0] : D.value;
+            const int x = (st.fp64 ? 0 : st.exp2) + 1 - D.N;
             double h, e;
             fast_two_sum(v.rh, v.rl, h, e);
-            o.x = scalbn(h + e, 1 - D.N) * D.value;
+            o.x = scalbn((h + e) * f, x);
             fast_two_sum(v.ih, v.il, h, e);
-            o.y = scalbn(h + e, 1 - D.N) * D.value;
+            o.y = scalbn((h + e) * f, x);
         }
         a.out[t.perm] = o;
     };
@@ -427,12 +862,12 @@ __device__ void haf_task(const HafArgs& a, const Task& t, unsigned char* raw, in
 
 // Persistent: every warp takes tasks from a global queue (counters[0]).
 template <bool LOOP>
-__global__ void __launch_bounds__(256, 1) hafnian_kernel(HafArgs a, int kmax, int jmax)
+__global__ void __launch_bounds__(256, 2) hafnian_kernel(HafArgs a, int kmax)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    unsigned char* raw = smem_raw + warp * haf_warp_smem_bytes(kmax, jmax);
-    int staged = -1;
+    const HafSmem sm(smem_raw + warp * haf_warp_smem_bytes(kmax), kmax);
+    HafStaged st;
     for (;;) {
         int q = 0;
         if (lane == 0)
@@ -440,7 +875,7 @@ __global__ void __launch_bounds__(256, 1) hafnian_kernel(HafArgs a, int kmax, in
         q = __shfl_sync(0xffffffffu, q, 0);
         if (q >= a.ntasks)
             break;
-        haf_task<LOOP>(a, a.tasks[q], raw, kmax, jmax, staged, lane);
+        haf_task<LOOP>(a, a.tasks[q], sm, st, lane);
     }
 }
 
@@ -516,6 +951,35 @@ static std::vector<double> loop_factors(int N)
     return cf;
 }
 
+// The factors after the first as integers for haf_loop_poly: for each pair kp,
+// the exponent with 2 max|z| <= 2^kp over the pair's roots, and (times 2^63) a
+// 2^-kp and b 2^-2kp; for an odd root kp and -z 2^-kp.  The roots' sizes
+// descend, so the first kp is the largest.
+static std::vector<int64_t> loop_integers(const std::vector<double>& cf)
+{
+    const int J = (int)cf.size() - 1, P = J / 2;
+    std::vector<int64_t> ci;
+    auto scale_of = [](double z) {
+        int e = 0;
+        std::frexp(2.0 * z * (1.0 + 0x1p-40), &e);
+        return e;
+    };
+    auto fixed = [](double v) { return (int64_t)std::llround(std::min(v, 0x1.ffp62)); };
+    for (int p = 0; p < P; ++p) {
+        const double a = cf[1 + 2 * p], b = cf[2 + 2 * p];
+        const int kp = scale_of(0.5 * (a + std::sqrt(std::max(0.0, a * a - 4.0 * b))));
+        ci.push_back(kp);
+        ci.push_back(fixed(std::ldexp(a, 63 - kp)));
+        ci.push_back(fixed(std::ldexp(b, 63 - 2 * kp)));
+    }
+    if (J % 2) {
+        const double c = -cf[1 + 2 * P];
+        ci.push_back(scale_of(c));
+        ci.push_back(fixed(std::ldexp(c, 63 - scale_of(c))));
+    }
+    return ci;
+}
+
 static double factorial_h(int n)
 {
     double r = 1.0;
@@ -532,7 +996,7 @@ static double factorial_h(int n)
 struct pq_haf_plan {
     int loop = 0;
     int64_t batch = 0, ntasks = 0;
-    int kmax = 1, jmax = 1, wpb = 1, blocks = 1, per_warp = 0;
+    int kmax = 1, wpb = 1, blocks = 1, per_warp = 0;
     pqi::HafDesc* desc_d = nullptr;
     int32_t* meta_d = nullptr;
     pqi::Task* tasks_d = nullptr;
@@ -646,7 +1110,7 @@ static int haf_plan_build(const int64_t* mat_off, const int32_t* k, const int32_
     std::vector<double> cost;
     std::vector<double> loopc;
     std::vector<int32_t> coef_at(PQ_MAX_N + 1, -1);
-    int kmax = 1, jmax = 1;
+    int kmax = 1;
     int32_t slot = 0;
     for (int64_t b = 0; b < batch; ++b) {
         HafDesc& D = desc[b];
@@ -667,6 +1131,11 @@ static int haf_plan_build(const int64_t* mat_off, const int32_t* k, const int32_
                 coef_at[N] = (int32_t)loopc.size();
                 const std::vector<double> cf = loop_factors(N);
                 loopc.insert(loopc.end(), cf.begin(), cf.end());
+                for (int64_t v : loop_integers(cf)) {
+                    double bits;
+                    std::memcpy(&bits, &v, sizeof(bits));
+                    loopc.push_back(bits);
+                }
             }
             D.coef_off = coef_at[N];
         }
@@ -695,7 +1164,6 @@ static int haf_plan_build(const int64_t* mat_off, const int32_t* k, const int32_
                 Lc *= it.dg[j].rad;
             }
         }
-        jmax = std::max(jmax, J);
         D.J = J;
         D.L = L;
         D.nchunks = T / L;
@@ -707,6 +1175,24 @@ static int haf_plan_build(const int64_t* mat_off, const int32_t* k, const int32_
             return report(PQ_ERR_UNSUPPORTED, "too many tasks");
         D.ntasks = (int32_t)nt;
         D.meta = (int32_t)meta.size();
+        // rows of the low digits first, in digit order
+        {
+            std::vector<int32_t> at(kk, -1), idx(kk), rm(kk);
+            int next = 0;
+            for (int d = 0; d < J; ++d)
+                at[it.dg[d].row] = next++;
+            for (int i = 0; i < kk; ++i)
+                if (at[i] < 0)
+                    at[i] = next++;
+            for (int i = 0; i < kk; ++i) {
+                idx[at[i]] = it.ridx[i];
+                rm[at[i]] = it.rm[i];
+            }
+            it.ridx = idx;
+            it.rm = rm;
+            for (Dg& d : it.dg)
+                d.row = at[d.row];
+        }
         meta.insert(meta.end(), it.ridx.begin(), it.ridx.end());
         meta.insert(meta.end(), it.rm.begin(), it.rm.end());
         for (const Dg& d : it.dg)
@@ -745,7 +1231,6 @@ static int haf_plan_build(const int64_t* mat_off, const int32_t* k, const int32_
         sorted[q] = tasks[order[q]];
     P->ntasks = (int64_t)sorted.size();
     P->kmax = kmax;
-    P->jmax = jmax;
     int rc = PQ_OK;
     if (dev_alloc((void**)&P->loopc_d, sizeof(double) * std::max<size_t>(loopc.size(), 1)) !=
             cudaSuccess ||
@@ -768,14 +1253,16 @@ static int haf_plan_build(const int64_t* mat_off, const int32_t* k, const int32_
                                        cudaMemcpyHostToDevice) != cudaSuccess)))
         rc = report(PQ_ERR_CUDA, "hafnian upload failed");
     if (rc == PQ_OK) {
-        P->per_warp = haf_warp_smem_bytes(kmax, jmax);
-        int wpb = 8;
-        while (wpb > 1 && wpb * P->per_warp > 227 * 1024)
-            --wpb;
-        const int bps = std::max(1, std::min(2, (227 * 1024) / (wpb * P->per_warp)));
+        P->per_warp = haf_warp_smem_bytes(kmax);
+        cudaFuncAttributes fa{};
+        const cudaError_t ea = loop ? cudaFuncGetAttributes(&fa, hafnian_kernel<true>)
+                                    : cudaFuncGetAttributes(&fa, hafnian_kernel<false>);
+        // as many resident warps as fit: a product waits on its own chain
+        int wpb = 1, bps = 1;
+        launch_geometry_max(ea == cudaSuccess ? fa.numRegs : 128, P->per_warp, 8, wpb, bps);
         P->wpb = wpb;
         const int64_t want_blocks = (P->ntasks + wpb - 1) / wpb;
-        P->blocks = (int)std::max<int64_t>(1, std::min<int64_t>(sms * bps, want_blocks));
+        P->blocks = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)sms * bps, want_blocks));
         // raise (never lower) the dynamic shared-memory limit of the kernel
         cudaFuncAttributes at{};
         cudaError_t e = loop ? cudaFuncGetAttributes(&at, hafnian_kernel<true>)
@@ -818,9 +1305,9 @@ static int haf_plan_launch(pq_haf_plan* P, const pq_c128* mats, const pq_c128* g
     a.counters = P->cnt_d;
     const int smem = P->wpb * P->per_warp;
     if (P->loop)
-        hafnian_kernel<true><<<P->blocks, 32 * P->wpb, smem, st>>>(a, P->kmax, P->jmax);
+        hafnian_kernel<true><<<P->blocks, 32 * P->wpb, smem, st>>>(a, P->kmax);
     else
-        hafnian_kernel<false><<<P->blocks, 32 * P->wpb, smem, st>>>(a, P->kmax, P->jmax);
+        hafnian_kernel<false><<<P->blocks, 32 * P->wpb, smem, st>>>(a, P->kmax);
     if (cudaGetLastError() != cudaSuccess)
         return report(PQ_ERR_CUDA, "hafnian kernel launch failed");
     return PQ_OK;

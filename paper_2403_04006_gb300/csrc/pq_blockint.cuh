@@ -208,7 +208,7 @@ __device__ __forceinline__ BInt bint_plain(longlong2 s)
 // exponent (zero below the smallest normal number).
 __device__ __forceinline__ double bint_factor(double w, int E, bool neg)
 {
-    const int h = __double2hiint(w) - ((kSumBits + E) << 20);
+    const int h = __double2hiint(w) - ((kSumBits + min(E, 1900)) << 20);
     return h >= 0x100000 ? __hiloint2double(h | (neg ? (int)0x80000000 : 0), __double2loint(w))
                          : 0.0;
 }

@@ -1,12 +1,13 @@
-"""The forward walk's block-integer arithmetic where it can go wrong: low
-words at the edge of their range, column scales over the whole exponent range,
-entries that vanish beside their column's largest, exact zeros, and inputs that
-have no scale at all (non-finite, or a column bound beyond FP64).  Expected
-values are exact rational permanents; the bound is that of an FP64 evaluation
-of the Glynn sum, 8 n 2^-53 of the mean absolute term."""
+"""The walks' block-integer arithmetic (permanents and hafnians) where it can go
+wrong: low words at the edge of their range, scales over the whole exponent
+range, entries that vanish beside the largest, exact zeros, and inputs that have
+no scale at all (non-finite, or a bound beyond FP64).  Permanents are compared
+with exact rational values; the bound is that of an FP64 evaluation of the Glynn
+sum, 8 n 2^-53 of the mean absolute term."""
 import numpy as np
 import pytest
 
+import oracle as O
 from paper_2403_04006_gb300 import api, workloads as W
 from exact import abs_err, exact_perm_grouped
 
@@ -122,3 +123,71 @@ def test_inputs_without_a_scale(dev, method, sums, bad):
     got, want = got.cpu().numpy(), want.cpu().numpy()
     assert np.array_equal(got[[0, 1, 5, 6]].view(np.float64), want.view(np.float64))
     assert not np.isfinite(got[2:5]).any()
+
+
+# ------------------------------------------------------------------ hafnians
+def haf_items(rng):
+    """(B, repetitions, loop weights): sizes from one index up, entries scaled
+    by powers of two, one entry far above the others, loop weights far above
+    and far below the square root of the entries, and none."""
+    out = []
+    for k in (1, 2, 3, 4, 5):
+        for e, ge in ((0, 0), (200, 100), (-200, -100), (0, 60), (0, -60)):
+            B = rng.standard_normal((k, k)) + 1j * rng.standard_normal((k, k))
+            B = (B + B.T) / 2
+            if k > 1 and e == 0:
+                B[0, 1] *= 1e9
+                B[1, 0] = B[0, 1]
+            gam = rng.standard_normal(k) + 1j * rng.standard_normal(k)
+            r = rng.integers(1, 4, k)
+            out.append((np.ldexp(B.real, e) + 1j * np.ldexp(B.imag, e), r,
+                        np.ldexp(gam.real, ge) + 1j * np.ldexp(gam.imag, ge)))
+        out.append((B, r, np.zeros(k, dtype=complex)))
+    return out
+
+
+def run_hafnians(items, dev, loop):
+    ks = np.array([B.shape[0] for B, _, _ in items], dtype=np.int32)
+    mo = np.concatenate([[0], np.cumsum(ks.astype(np.int64) ** 2)[:-1]])
+    ro = np.concatenate([[0], np.cumsum(ks, dtype=np.int64)[:-1]])
+    mats = torch.from_numpy(np.concatenate([B.reshape(-1) for B, _, _ in items])).to(dev)
+    gam = torch.from_numpy(np.concatenate([g for _, _, g in items])).to(dev)
+    rep = np.concatenate([r for _, r, _ in items]).astype(np.int32)
+    return api.hafnian_repeated(mats, mo, ks, rep, ro, gamma=gam if loop else None).cpu().numpy()
+
+
+@pytest.mark.parametrize("loop", [False, True])
+def test_hafnian_scales(dev, loop):
+    """Against the oracle's double-double sum, within 32 N 2^-53 of the sum of
+    the terms' magnitudes (an FP64 evaluation's own bound: N products, the
+    updates of q and l, and the accumulation)."""
+    items = haf_items(np.random.default_rng(5))
+    got = run_hafnians(items, dev, loop)
+    for q, ((B, r, g), v) in enumerate(zip(items, got)):
+        want, scale = (O.lhaf_grouped(B, g, r, info=True) if loop
+                       else O.haf_grouped(B, r, info=True))
+        if not np.isfinite(want):  # beyond FP64
+            assert not np.isfinite(v)
+            continue
+        assert abs(v - want) <= 32 * int(sum(r)) * 2.0 ** -53 * max(scale, abs(want)), (q, v, want)
+
+
+@pytest.mark.parametrize("loop", [False, True])
+@pytest.mark.parametrize("bad", [np.inf, np.nan, 1.2e308])
+def test_hafnians_without_a_scale(dev, loop, bad):
+    """Non-finite entries and sums beyond FP64 give results that are not
+    finite; the items beside them keep their bits, a zero matrix gives zero."""
+    rng = np.random.default_rng(6)
+    items = [x for x in haf_items(rng) if x[0].shape[0] > 1][:6]
+    items = [(B, 2 * np.ones_like(r), g) for B, r, g in items]
+    want = run_hafnians(items, dev, loop)
+    dirty = []
+    for B, r, g in items[:2]:
+        B = B.copy()
+        B[0, 1] = B[1, 0] = bad
+        dirty.append((B, r, g))
+    zero = (np.zeros((3, 3), dtype=complex), np.array([2, 1, 1]), np.zeros(3, dtype=complex))
+    got = run_hafnians(items[:3] + dirty + [zero] + items[3:], dev, loop)
+    assert np.array_equal(got[[0, 1, 2, 6, 7, 8]].view(np.float64), want.view(np.float64))
+    assert not np.isfinite(got[3:5]).any()
+    assert got[5] == 0
