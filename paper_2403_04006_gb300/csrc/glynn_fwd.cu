@@ -386,41 +386,16 @@ __device__ __forceinline__ dd2 task_sum(double rh, double rl, double ih, double 
 }
 
 // The task's sum res (the same on every lane) goes to the permanent's output
-// if the permanent has one task; otherwise to its slot, and the warp that
-// writes the last slot adds the slots in task order.
+// if the permanent has one task; otherwise to its slot, and the warps that
+// finish last add the slots (gather_partials).
 __device__ void combine_task(const ExecArgs& a, const Task& t, const PermDesc& D, dd2 res, int exp2,
                              int lane)
 {
-    if (D.ntasks <= 1) {
-        if (lane == 0)
-            finalize(a, D, res, exp2);
-        return;
-    }
-    int last = 0;
-    if (lane == 0) {
-        double* pp = a.partials + 4 * (int64_t)(D.slot0 + t.part - D.part0);
-        pp[0] = res.rh;
-        pp[1] = res.rl;
-        pp[2] = res.ih;
-        pp[3] = res.il;
-        __threadfence();
-        const int old = atomicAdd(a.counters + 1 + t.perm, 1);
-        last = (old == D.ntasks - 1);
-    }
-    last = __shfl_sync(0xffffffffu, last, 0);
-    if (!last)
-        return;
-    __threadfence();
-    dd2 tot = {0.0, 0.0, 0.0, 0.0};
-    for (int q = lane; q < D.ntasks; q += kWarp) {
-        const double* pp = a.partials + 4 * (int64_t)(D.slot0 + q);
-        dd_add(tot.rh, tot.rl, __ldcg(pp + 0), __ldcg(pp + 1));
-        dd_add(tot.ih, tot.il, __ldcg(pp + 2), __ldcg(pp + 3));
-    }
-    warp_fix_sum(tot.rh, tot.rl, tot.rh, tot.rl);
-    warp_fix_sum(tot.ih, tot.il, tot.ih, tot.il);
-    if (lane == 0)
-        finalize(a, D, tot, exp2);
+    if (gather_partials(a.partials + 4 * (int64_t)D.slot0, a.counters + 1 + t.perm,
+                        a.groups + D.gslot0, t.part - D.part0, D.ntasks, res.rh, res.rl, res.ih,
+                        res.il, lane) &&
+        lane == 0)
+        finalize(a, D, res, exp2);
 }
 
 // ---------------------------------------------------------------- the walk
@@ -435,27 +410,6 @@ __device__ __forceinline__ void start_walk(LowWalk& wk, const MetaView& mv, int 
         wk.radm1 |= uint64_t(mv.drad[d] - 1) << (4 * d);
         wk.topp |= uint64_t(mv.dtop[d]) << (4 * d);
     }
-}
-
-// Digit of radix rad split off the chunk index c.
-__device__ __forceinline__ int next_digit(int64_t& c, int rad, bool narrow)
-{
-    if (narrow) {
-        const uint32_t v = (uint32_t)c, q = v / (uint32_t)rad;
-        c = q;
-        return (int)(v - q * (uint32_t)rad);
-    }
-    const int g = (int)(c % rad);
-    c /= rad;
-    return g;
-}
-
-// C(top, g) for a high digit.
-__device__ __forceinline__ uint64_t high_binom(int top, int g)
-{
-    if (top <= 3)
-        return (g == 0 || g == top) ? 1 : (uint64_t)top;
-    return binom_u64(top, g);
 }
 
 // The walk of this lane's chunk; returns the task's sum over the warp
@@ -699,7 +653,8 @@ __device__ __forceinline__ void run_task(const ExecArgs& a, int64_t ti, WarpSmem
                                          int ld, Staged& st, int lane)
 {
     const Task t = a.tasks[ti];
-    const int32_t bad = task_guard(t, a.desc, a.nperm, a.nmeta, a.nslots, kmax, ld, kMaxLowDigits);
+    const int32_t bad = task_guard(t, a.desc, a.nperm, a.nmeta, a.nslots, kmax, ld, kMaxLowDigits,
+                                   a.ngroups);
     if (bad) {
         if (lane == 0)
             record_error(a.err, bad, ti);
@@ -789,7 +744,8 @@ __global__ void __launch_bounds__(256, 2) glynn_fwd_reg_mixed_kernel(ExecArgs a,
     auto run = [&](int64_t ti) {
         const Task t = a.tasks[ti];
         const int32_t bad =
-            task_guard(t, a.desc, a.nperm, a.nmeta, a.nslots, kmax, ld, kMaxLowDigits);
+            task_guard(t, a.desc, a.nperm, a.nmeta, a.nslots, kmax, ld, kMaxLowDigits,
+                       a.ngroups);
         if (bad) {
             if (lane == 0)
                 record_error(a.err, bad, ti);

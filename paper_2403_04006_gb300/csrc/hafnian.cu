@@ -70,6 +70,7 @@ struct alignas(16) HafDesc {
     int32_t k, n, N, ld;   // kept indices, N/2, expanded size, source row stride
     int32_t meta;          // ridx[k], rmul[k], drow[nd], drad[nd], dtop[nd]
     int32_t ndig, J, ntasks, slot0;
+    int32_t gslot0;        // first counter of its task groups (more than 32 tasks)
     int32_t weighted, trivial;  // trivial: result = value (0 for odd N, 1 for N = 0)
     int32_t coef_off;           // loop hafnian: factors of its loop polynomial in loopc
     double value;               // final multiplier (or the trivial result)
@@ -86,7 +87,8 @@ struct HafArgs {
                            // J + 1 doubles, then the integers of loop_integers
     double2* out;
     double* partials;
-    int32_t* counters;
+    int32_t* counters;  // [0] task queue head, [1 + b] finished tasks (or groups) of item b
+    int32_t* groups;    // finished tasks of each group of 32
 };
 
 // Shared memory of one warp: M (k x k), y0 = B r (k), gamma (k), y (k x 32,
@@ -614,11 +616,11 @@ __device__ __forceinline__ dd2 haf_walk_int(const HafDesc& D, const HafMeta& mt,
         y[j * 32] = y0[j];
     uint64_t whigh_u = 1;
     int gpar = 0;
+    const bool narrow = D.nchunks <= 0x7fffffff;
     int64_t cc = c;
 #pragma unroll 1
     for (int d = J; d < nd; ++d) {
-        const int g = (int)(cc % mt.drad[d]);
-        cc /= mt.drad[d];
+        const int g = next_digit(cc, mt.drad[d], narrow);
         if (!g)
             continue;
         const ulonglong2* Mr = M + mt.drow[d];
@@ -630,7 +632,7 @@ __device__ __forceinline__ dd2 haf_walk_int(const HafDesc& D, const HafMeta& mt,
             v.y -= (uint64_t)g * b.y;
             y[j * 32] = v;
         }
-        whigh_u *= binom_u64(mt.dtop[d], g);
+        whigh_u *= high_binom(mt.dtop[d], g);
         gpar += g;
     }
     // 2 q = x^T y - sum_i r_i B_ii and l = gamma^T x, low digits at 0
@@ -649,8 +651,7 @@ __device__ __forceinline__ dd2 haf_walk_int(const HafDesc& D, const HafMeta& mt,
     cc = c;
 #pragma unroll 1
     for (int d = J; d < nd; ++d) {
-        const int g = (int)(cc % mt.drad[d]);
-        cc /= mt.drad[d];
+        const int g = next_digit(cc, mt.drad[d], narrow);
         if (!g)
             continue;
         const int row = mt.drow[d];
@@ -827,37 +828,11 @@ __device__ void haf_task(const HafArgs& a, const Task& t, const HafSmem& sm, Haf
         }
         a.out[t.perm] = o;
     };
-    if (D.ntasks <= 1) {
-        if (lane == 0)
-            finish(res);
-        return;
-    }
-    // Several tasks: partials in task order; the last warp to finish sums them
-    // in a fixed order (no waiting on other warps).
-    int last = 0;
-    if (lane == 0) {
-        double* pp = a.partials + 4 * (int64_t)(D.slot0 + t.part);
-        pp[0] = res.rh;
-        pp[1] = res.rl;
-        pp[2] = res.ih;
-        pp[3] = res.il;
-        __threadfence();
-        last = (atomicAdd(a.counters + 1 + t.perm, 1) == D.ntasks - 1);
-    }
-    last = __shfl_sync(0xffffffffu, last, 0);
-    if (!last)
-        return;
-    __threadfence();
-    dd2 tot = {0.0, 0.0, 0.0, 0.0};
-    for (int p = lane; p < D.ntasks; p += kWarp) {
-        const double* pp = a.partials + 4 * (int64_t)(D.slot0 + p);
-        dd_add(tot.rh, tot.rl, __ldcg(pp + 0), __ldcg(pp + 1));
-        dd_add(tot.ih, tot.il, __ldcg(pp + 2), __ldcg(pp + 3));
-    }
-    warp_fix_sum(tot.rh, tot.rl, tot.rh, tot.rl);
-    warp_fix_sum(tot.ih, tot.il, tot.ih, tot.il);
-    if (lane == 0)
-        finish(tot);
+    if (gather_partials(a.partials + 4 * (int64_t)D.slot0, a.counters + 1 + t.perm,
+                        a.groups + D.gslot0, t.part, D.ntasks, res.rh, res.rl, res.ih, res.il,
+                        lane) &&
+        lane == 0)
+        finish(res);
 }
 
 // Persistent: every warp takes tasks from a global queue (counters[0]).
@@ -995,7 +970,7 @@ static double factorial_h(int n)
 // workspace owned by the plan.
 struct pq_haf_plan {
     int loop = 0;
-    int64_t batch = 0, ntasks = 0;
+    int64_t batch = 0, ntasks = 0, ngroups = 0;
     int kmax = 1, wpb = 1, blocks = 1, per_warp = 0;
     pqi::HafDesc* desc_d = nullptr;
     int32_t* meta_d = nullptr;
@@ -1112,10 +1087,12 @@ static int haf_plan_build(const int64_t* mat_off, const int32_t* k, const int32_
     std::vector<int32_t> coef_at(PQ_MAX_N + 1, -1);
     int kmax = 1;
     int32_t slot = 0;
+    int64_t ngroups = 0;
     for (int64_t b = 0; b < batch; ++b) {
         HafDesc& D = desc[b];
         Item& it = items[b];
         D.slot0 = slot;
+        D.gslot0 = (int32_t)ngroups;
         if (D.trivial) {
             D.ntasks = 1;
             tasks.push_back(Task{(int32_t)b, 0});
@@ -1174,6 +1151,8 @@ static int haf_plan_build(const int64_t* mat_off, const int32_t* k, const int32_
         if (nt + slot > (int64_t(1) << 30))
             return report(PQ_ERR_UNSUPPORTED, "too many tasks");
         D.ntasks = (int32_t)nt;
+        if (nt > 32)
+            ngroups += (nt + 31) / 32;
         D.meta = (int32_t)meta.size();
         // rows of the low digits first, in digit order
         {
@@ -1230,6 +1209,7 @@ static int haf_plan_build(const int64_t* mat_off, const int32_t* k, const int32_
     for (size_t q = 0; q < order.size(); ++q)
         sorted[q] = tasks[order[q]];
     P->ntasks = (int64_t)sorted.size();
+    P->ngroups = ngroups;
     P->kmax = kmax;
     int rc = PQ_OK;
     if (dev_alloc((void**)&P->loopc_d, sizeof(double) * std::max<size_t>(loopc.size(), 1)) !=
@@ -1240,7 +1220,7 @@ static int haf_plan_build(const int64_t* mat_off, const int32_t* k, const int32_
         dev_alloc((void**)&P->tasks_d, sizeof(Task) * sorted.size()) != cudaSuccess ||
         dev_alloc((void**)&P->part_d, sizeof(double) * 4 * std::max<int32_t>(slot, 1)) !=
             cudaSuccess ||
-        dev_alloc((void**)&P->cnt_d, sizeof(int32_t) * (batch + 1)) != cudaSuccess)
+        dev_alloc((void**)&P->cnt_d, sizeof(int32_t) * (batch + 1 + ngroups)) != cudaSuccess)
         rc = report(PQ_ERR_NOMEM, "hafnian workspace allocation failed");
     if (rc == PQ_OK &&
         (cudaMemcpy(P->desc_d, desc.data(), sizeof(HafDesc) * batch, cudaMemcpyHostToDevice) !=
@@ -1290,7 +1270,7 @@ static int haf_plan_launch(pq_haf_plan* P, const pq_c128* mats, const pq_c128* g
 {
     if (P->batch == 0)
         return PQ_OK;
-    if (cudaMemsetAsync(P->cnt_d, 0, sizeof(int32_t) * (P->batch + 1), st) != cudaSuccess)
+    if (cudaMemsetAsync(P->cnt_d, 0, sizeof(int32_t) * (P->batch + 1 + P->ngroups), st) != cudaSuccess)
         return report(PQ_ERR_CUDA, "hafnian counter reset failed");
     HafArgs a;
     a.desc = P->desc_d;
@@ -1303,6 +1283,7 @@ static int haf_plan_launch(pq_haf_plan* P, const pq_c128* mats, const pq_c128* g
     a.out = reinterpret_cast<double2*>(out);
     a.partials = P->part_d;
     a.counters = P->cnt_d;
+    a.groups = P->cnt_d + P->batch + 1;
     const int smem = P->wpb * P->per_warp;
     if (P->loop)
         hafnian_kernel<true><<<P->blocks, 32 * P->wpb, smem, st>>>(a, P->kmax);

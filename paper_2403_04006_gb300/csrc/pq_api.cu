@@ -756,6 +756,7 @@ static int schedule_and_upload(pq_plan* P)
     P->plain_first.assign(np + 1, 0);
     std::vector<double> task_cost;
     int32_t slot = 0;
+    P->ngroups = 0;
     double flops_f = 0.0, flops_b = 0.0, instr_f = 0.0, instr_fx = 0.0;
     int64_t terms = 0;
     for (int64_t p = 0; p < np; ++p) {
@@ -809,6 +810,9 @@ static int schedule_and_upload(pq_plan* P)
         D.part0 = (int32_t)q0;
         D.slot0 = slot;
         slot += (int32_t)nt;
+        D.gslot0 = (int32_t)P->ngroups;
+        if (nt > 32)
+            P->ngroups += (nt + 31) / 32;
         P->plain_first[p] = (int64_t)P->tasks_plain_h.size();
         const double fpt = it.trivial ? 0.0 : fwd_flops_per_term(it);
         const double init = 2.0 * (it.drow.size() - it.J) * it.l + 2.0 * it.l;
@@ -883,7 +887,7 @@ static int schedule_and_upload(pq_plan* P)
     PQ_ALLOC(&P->partials_d, std::max<size_t>(slot, 1) * 4 * sizeof(double));
     dev_free(P->counters_d);
     P->counters_d = nullptr;
-    PQ_ALLOC(&P->counters_d, (size_t)(np + 1) * sizeof(int32_t));
+    PQ_ALLOC(&P->counters_d, (size_t)(np + 1 + P->ngroups) * sizeof(int32_t));
     if (!P->err_d) {
         PQ_ALLOC(&P->err_d, 2 * sizeof(int32_t));
         PQ_CUDA(cudaMemset(P->err_d, 0, 2 * sizeof(int32_t)));
@@ -1123,10 +1127,12 @@ static ExecArgs exec_args(pq_plan* P, const void* src, void* amps, double* probs
     a.out_prob = probs;
     a.partials = P->partials_d;
     a.counters = P->counters_d;
+    a.groups = P->counters_d + P->nperm + 1;
     a.err = P->err_d;
     a.nperm = P->nperm;
     a.nmeta = (int64_t)P->meta_h.size();
     a.nslots = P->nslots;
+    a.ngroups = P->ngroups;
     return a;
 }
 
@@ -1135,7 +1141,8 @@ static int run_forward_raw(pq_plan* P, const void* src, void* amps, double* prob
 {
     if (!P->uploaded)
         return fail(PQ_ERR_STATE, "the plan lost its device data in a failed re-planning");
-    PQ_CUDA(cudaMemsetAsync(P->counters_d, 0, (size_t)(P->nperm + 1) * sizeof(int32_t), st));
+    PQ_CUDA(cudaMemsetAsync(P->counters_d, 0,
+                            (size_t)(P->nperm + 1 + P->ngroups) * sizeof(int32_t), st));
     if (P->nperm == 0)
         return PQ_OK;
     if (P->opts.method == PQ_METHOD_PLAIN) {

@@ -137,6 +137,27 @@ __host__ __device__ __forceinline__ uint64_t binom_small(int top, int g)
 #endif
 }
 
+// Digit of radix rad split off the chunk index c.
+__device__ __forceinline__ int next_digit(int64_t& c, int rad, bool narrow)
+{
+    if (narrow) {
+        const uint32_t v = (uint32_t)c, q = v / (uint32_t)rad;
+        c = q;
+        return (int)(v - q * (uint32_t)rad);
+    }
+    const int g = (int)(c % rad);
+    c /= rad;
+    return g;
+}
+
+// C(top, g) for a high digit.
+__device__ __forceinline__ uint64_t high_binom(int top, int g)
+{
+    if (top <= 3)
+        return (g == 0 || g == top) ? 1 : (uint64_t)top;
+    return binom_u64(top, g);
+}
+
 // C(top, g) in double (exact while it stays below 2^53).
 __device__ __forceinline__ double binom_f64(int top, int g)
 {
@@ -178,13 +199,13 @@ __device__ __forceinline__ MetaView meta_view(const int32_t* pool, const PermDes
 // against the launch's shared-memory layout (kmax rows, ld columns, jmax low
 // digits), the digit counts against the walk's limits, and the descriptor's
 // indices into the metadata pool, the partial slots and the outputs.
-// nslots < 0: the caller indexes its own slots (no slot check).  Returns 0 or
+// nslots < 0: the caller indexes its own slots (no slot or group check).  Returns 0 or
 // the error code.  The guard reads the descriptor through the L2 path into a
 // copy of its own, so the task's code loads what it needs afterwards and no
 // descriptor stays live in registers across the task.
 __device__ __forceinline__ int32_t task_guard(const Task& t, const PermDesc* desc, int64_t nperm,
                                            int64_t nmeta, int64_t nslots, int kmax, int ld,
-                                           int jmax)
+                                           int jmax, int64_t ngroups = 0)
 {
     if (t.perm < 0 || (int64_t)t.perm >= nperm)
         return kErrTaskPerm;
@@ -197,6 +218,9 @@ __device__ __forceinline__ int32_t task_guard(const Task& t, const PermDesc* des
         (int64_t)D.out >= nperm || D.ntasks < 1)
         return kErrDescIndex;
     if (nslots >= 0 && (D.slot0 < 0 || (int64_t)D.slot0 + D.ntasks > nslots))
+        return kErrDescIndex;
+    if (nslots >= 0 && D.ntasks > 32 &&
+        (D.gslot0 < 0 || (int64_t)D.gslot0 + (D.ntasks + 31) / 32 > ngroups))
         return kErrDescIndex;
     const int64_t q = (int64_t)t.part - D.part0;
     if (q < 0 || q >= D.ntasks)

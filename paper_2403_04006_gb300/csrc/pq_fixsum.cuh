@@ -21,6 +21,8 @@
 
 #include <cstring>
 
+#include "pq_device.cuh"
+
 namespace pqi {
 
 constexpr int kFixFrac = 64;  // fraction bits below the largest value's last significand bit
@@ -179,6 +181,73 @@ __device__ __forceinline__ void warp_fix_sum(double hi, double lo, double& shi, 
         limb[q] = __reduce_add_sync(0xffffffffu, limb[q]);
     top = __reduce_add_sync(0xffffffffu, top);
     fix_to_dd(fix_from_limbs(limb, top), emax, shi, slo);
+}
+
+// The partial sums of a permanent's (or hafnian's) tasks, re hi, re lo, im hi,
+// im lo per slot, added by the warps that finish last.  One warp adding
+// thousands of slots in double-double is a serial tail of its own (16384 tasks:
+// 512 slots per lane at 28 dependent FP64 operations each, 0.55 ms; 11072 tasks
+// of a hafnian: 0.75 of 1.08 ms), so the slots are added in two levels: the last
+// warp of every 32 consecutive tasks adds theirs, exactly in integers, into the
+// group's first slot, and the last warp of all adds the groups.  Which warp does
+// it does not change the sum.
+// slots: the first task's; q of ntasks: this task; groups: one zeroed counter
+// per 32 tasks; done: the counter of a permanent of at most 32 tasks, else of
+// its groups.  Returns true on the warp that holds the total in (rh, rl, ih, il).
+__device__ __forceinline__ bool gather_partials(double* slots, int32_t* done, int32_t* groups,
+                                                int q, int ntasks, double& rh, double& rl,
+                                                double& ih, double& il, int lane)
+{
+    if (ntasks <= 1)
+        return true;
+    const int ng = (ntasks + 31) >> 5, g = q >> 5;
+    const int count = min(32, ntasks - 32 * g);
+    auto store = [&](int at) {
+        double* pp = slots + 4 * (int64_t)at;
+        pp[0] = rh;
+        pp[1] = rl;
+        pp[2] = ih;
+        pp[3] = il;
+        __threadfence();
+    };
+    int last = 0;
+    if (lane == 0) {
+        store(q);
+        last = atomicAdd(ng == 1 ? done : groups + g, 1) == count - 1;
+    }
+    last = __shfl_sync(0xffffffffu, last, 0);
+    if (!last)
+        return false;
+    __threadfence();
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    if (lane < count) {
+        const double* pp = slots + 4 * (int64_t)(32 * g + lane);
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            v[e] = __ldcg(pp + e);
+    }
+    warp_fix_sum(v[0], v[1], rh, rl);
+    warp_fix_sum(v[2], v[3], ih, il);
+    if (ng == 1)
+        return true;
+    __syncwarp();  // every lane has read the group's slots
+    if (lane == 0) {
+        store(32 * g);
+        last = atomicAdd(done, 1) == ng - 1;
+    }
+    last = __shfl_sync(0xffffffffu, last, 0);
+    if (!last)
+        return false;
+    __threadfence();
+    rh = rl = ih = il = 0.0;
+    for (int h = lane; h < ng; h += 32) {
+        const double* pp = slots + 4 * (int64_t)(32 * h);
+        dd_add(rh, rl, __ldcg(pp + 0), __ldcg(pp + 1));
+        dd_add(ih, il, __ldcg(pp + 2), __ldcg(pp + 3));
+    }
+    warp_fix_sum(rh, rl, rh, rl);
+    warp_fix_sum(ih, il, ih, il);
+    return true;
 }
 #endif
 

@@ -50,7 +50,7 @@ struct alignas(16) PermDesc {
     int64_t L;        // chunk length
     double norm;      // 1 / (prod t! prod s!) for boson sampling, else 1
     int32_t part0;    // first task part of this plan's shard (0 unless sharded)
-    int32_t pad2;
+    int32_t gslot0;   // first counter of its task groups (more than 32 tasks)
 };
 
 // Integer metadata of one permanent, at pool + PermDesc::meta:
@@ -86,11 +86,13 @@ struct ExecArgs {
     double* out_partial;  // sharded plans: unscaled double-double sum, 4 doubles per
                           // permanent (re hi, re lo, im hi, im lo); nullable
     double* partials;     // 4 doubles per task slot
-    int32_t* counters;    // [0] task queue head, [1 + p] finished tasks of p
+    int32_t* counters;    // [0] task queue head, [1 + p] finished tasks (or groups) of p
+    int32_t* groups;      // finished tasks of each group of 32, permanents of more than 32
     int32_t* err;         // device error record, see below
     int64_t nperm;        // permanents of the plan (bound of Task::perm and PermDesc::out)
     int64_t nmeta;        // entries of the metadata pool
     int64_t nslots;       // task slots of `partials`
+    int64_t ngroups;      // counters of `groups`
 };
 
 // Device error record (two int32 words, zero = no error): the kernels check

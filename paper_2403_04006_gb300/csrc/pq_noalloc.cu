@@ -35,6 +35,10 @@ namespace pqi {
 constexpr size_t kNoAllocBytes = size_t(PQ_NOALLOC_SCRATCH_BYTES);
 constexpr size_t kNoAllocHead = 8192;
 constexpr int64_t kNoAllocMaxTasks = (int64_t)((kNoAllocBytes - kNoAllocHead) / 40);
+// the head's end: the counters of the task groups, then 16 counters
+constexpr int kNoAllocGroups = 1024;
+constexpr size_t kNoAllocGroupsAt = kNoAllocHead - 64 - 4 * kNoAllocGroups;
+static_assert(kNoAllocMaxTasks <= 32 * kNoAllocGroups, "a counter for every task group");
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
@@ -44,7 +48,7 @@ struct NoAllocHead {
     PermDesc desc;
     int32_t meta[2 * PQ_MAX_DIM + 3 * PQ_MAX_DIM + 3 * PQ_MAX_DIM];
 };
-static_assert(sizeof(NoAllocHead) + 64 <= kNoAllocHead, "workspace head too small");
+static_assert(sizeof(NoAllocHead) <= kNoAllocGroupsAt, "workspace head too small");
 static_assert(sizeof(NoAllocHead) % 4 == 0, "head copied as 32-bit words");
 static_assert(sizeof(NoAllocHead) <= 4000, "head must fit the kernel-parameter space");
 
@@ -61,6 +65,9 @@ __global__ void noalloc_setup(const NoAllocHead h, unsigned char* base, int32_t*
             dst[w] = src[w];
         if (threadIdx.x < 16)
             counters[threadIdx.x] = 0;
+        int32_t* groups = reinterpret_cast<int32_t*>(base + kNoAllocGroupsAt);
+        for (int w = threadIdx.x; w < kNoAllocGroups; w += blockDim.x)
+            groups[w] = 0;
     }
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < ntasks;
          q += (int64_t)gridDim.x * blockDim.x) {
@@ -216,6 +223,7 @@ static int noalloc_plan(int k0, int l0, const int32_t* r, const int32_t* c, NoAl
                             "permanent needs more warp tasks than the static workspace holds");
     D.ntasks = (int32_t)ntasks;
     D.slot0 = 0;
+    D.gslot0 = 0;
     D.weighted = 0;
     for (int d = 0; d < J; ++d)
         if (drad[d] > 2)
@@ -311,6 +319,8 @@ extern "C" int pq_permanent_noalloc(const pq_c128* B, int32_t k, int32_t l,
     a.out_partial = nullptr;
     a.partials = partials_d;
     a.counters = counters_d;
+    a.groups = reinterpret_cast<int32_t*>(base + kNoAllocGroupsAt);
+    a.ngroups = kNoAllocGroups;
     a.err = counters_d + 8;
     a.nperm = 1;
     a.nmeta = (int64_t)(sizeof(h.meta) / sizeof(h.meta[0]));
