@@ -58,9 +58,9 @@
 namespace pqi {
 
 constexpr int kHafMaxHalf = PQ_MAX_N / 2;  // loop-polynomial factors j = 1 .. N/2
-// integers of a loop polynomial of J = N/2 roots: 3 a pair, 2 for an odd root
-__host__ __device__ constexpr int haf_integers(int J) { return 3 * (J / 2) + 2 * (J % 2); }
-constexpr int kHafMaxInts = 40;
+// integers of a loop polynomial of J = N/2 roots: 4 a pair, 2 for an odd root
+__host__ __device__ constexpr int haf_integers(int J) { return 4 * (J / 2) + 2 * (J % 2); }
+constexpr int kHafMaxInts = 48;
 static_assert(haf_integers(kHafMaxHalf) <= kHafMaxInts && haf_integers(kHafMaxHalf - 1) <= kHafMaxInts,
               "room for the integers of every loop polynomial");
 
@@ -207,7 +207,7 @@ struct HafStaged {
     bool fp64 = false;  // staged as doubles
     int exp2 = 0;       // the terms' sum times 2^exp2 is the sum of s(g) times the polynomial
     int eq = 0, el = 0; // q and l times 2^eq, 2^el are the integers
-    int xref = 0;       // loop hafnian: upper bound of the exponent q and s are aligned to
+    int ref2 = 0, ref1 = 0;  // loop hafnian: upper bounds of a factor's exponent (pair, odd root)
 };
 
 // The walk of this lane's chunk in FP64; returns the task's sum.
@@ -465,11 +465,12 @@ __device__ bool haf_stage_int(const HafDesc& D, const HafMeta& mt, const HafSmem
     st.eq = eq;
     st.el = el;
     if (LOOP) {
-        // P pairs at 2 X + 64, an odd root at X, an odd N at -el; 64 per product
         const int P = D.N >> 2, jo = (D.N >> 1) & 1, no = D.N & 1;
-        const int parts = P + jo + no;
-        st.xref = 1 + (P + jo > 0 ? max(-eq, 64 - 2 * el + (int)sm.ci[0]) : 0);
-        st.exp2 = kSumBits + 64 * (P + parts - 1) + (2 * P + jo) * st.xref - no * el;
+        const int xq = -eq, xs = 64 - 2 * el;  // upper bounds; the largest root comes first
+        st.ref2 = P == 0 ? 0
+                         : 2 + max(64 + 2 * xq, 66 + xs + max(xq + (int)sm.ci[0], xs + (int)sm.ci[2]));
+        st.ref1 = jo == 0 ? 0 : 2 + max(xq, xs + (int)sm.ci[4 * P] + 2);
+        st.exp2 = kSumBits + 64 * (P + jo + no - 1) + P * st.ref2 + jo * st.ref1 - no * el;
     } else {
         st.exp2 = kSumBits + 64 * (D.n - 1) - D.n * eq;
     }
@@ -517,28 +518,30 @@ __device__ __forceinline__ BInt haf_power(longlong2 q, int n, int& E)
     return h;
 }
 
-// 2 (c v >> 64) of a real 0 <= c < 2^63, the product of v and c 2^-63.
+// c v >> 64 for a real 0 <= c < 2^62 (the limbs of a larger c overflow).
 __device__ __forceinline__ longlong2 real_scale(int64_t c, const BLimbs& v)
 {
     const int ch = (int)((c + kSumBias) >> 32), cl = (int)(uint32_t)c;
     const int64_t mr = mulw(v.a, cl) + mulw(v.b, ch), mi = mulw(v.c, cl) + mulw(v.d, ch);
     const int64_t hr = mulw(v.a, ch) + (int64_t)(int)(mr >> 32);
     const int64_t hi = mulw(v.c, ch) + (int64_t)(int)(mi >> 32);
-    return make_longlong2(2 * hr, 2 * hi);
+    return make_longlong2(hr, hi);
 }
 
 __device__ __forceinline__ longlong2 shift_right(longlong2 v, int n)
 {
+    n = min(n, 63);
     return make_longlong2(v.x >> n, v.y >> n);
 }
 
 // The loop polynomial of q and l without its leading factor: P pairs of roots
 // q^2 + a q s + b s^2 with s = l^2, an odd root q + c s, an odd N one factor l.
-// The roots spread over two decades, so every pair has its own scale 2^kp of
-// s (ci: kp, a 2^-kp, b 2^-2kp of each pair, kp and c 2^-kp of an odd root, all
-// coefficients at most 1), and its three terms are brought to the larger of
-// the exponents of q^2 and (2^kp s)^2: whichever of q and s is large, a factor
-// keeps its bits.  E counts the exponents against xref, their upper bound.
+// q^2, q s and s^2 are normalised once, and the coefficients are integers of 62
+// bits with an exponent each (ci: ea, a, eb, b of each pair, ec and c of an odd
+// root), so every product has its full bits whatever the ratio of q and s; the
+// three terms of a factor are brought to the largest of their exponents and one
+// more, which keeps the factor below 2^62.  E counts the factors' exponents
+// against their upper bounds ref2 and ref1.
 __device__ __forceinline__ BInt haf_loop_poly(longlong2 q, longlong2 l, int P, bool jodd, bool nodd,
                                               const int64_t* ci, const HafStaged& st, int& E)
 {
@@ -555,38 +558,43 @@ __device__ __forceinline__ BInt haf_loop_poly(longlong2 q, longlong2 l, int P, b
         BInt sw = bmul(ll, ll);
         int Es = 0;
         bnorm(sw, Es);
-        // one bit down, so that a factor stays below 2^62
-        const longlong2 qv = shift_right(bint_pair(qw), 1), sv = shift_right(bint_pair(sw), 1);
-        constexpr int kNone = -(1 << 20);  // exponent of an exact zero
-        const int xq = (qv.x | qv.y) == 0 ? kNone : 1 - st.eq - Eq;
-        const int xs = (sv.x | sv.y) == 0 ? kNone : 65 - 2 * (st.el + El) - Es;
-        const BLimbs lq = limbs(bint_words(qv)), ls = limbs(bint_words(sv));
+        constexpr int kNone = -(1 << 18), kLeast = -(1 << 17);  // exponent of an exact zero
+        const int xq = (qw.rh | qw.ih | qw.rl | qw.il) == 0 ? kNone : -st.eq - Eq;
+        const int xs = (sw.rh | sw.ih | sw.rl | sw.il) == 0 ? kNone : 64 - 2 * (st.el + El) - Es;
+        const BLimbs lq = limbs(qw), ls = limbs(sw);
         if (P > 0) {
-            const longlong2 q2 = bint_pair(bmul(lq, lq));
-            const BLimbs qs = limbs(bmul(lq, ls)), s2 = limbs(bmul(ls, ls));
+            int n0 = 0, n1 = 0, n2 = 0;
+            BInt v0 = bmul(lq, lq), v1 = bmul(lq, ls), v2 = bmul(ls, ls);
+            bnorm(v0, n0);
+            bnorm(v1, n1);
+            bnorm(v2, n2);
+            const int x0 = 2 * xq + 64 - n0, x1 = xq + xs + 66 - n1, x2 = 2 * xs + 66 - n2;
+            const longlong2 q2 = bint_pair(v0);
+            const BLimbs qs = limbs(v1), s2 = limbs(v2);
 #pragma unroll 1
             for (int p = 0; p < P; ++p) {
-                const int64_t* c = ci + 3 * p;
-                const int y = xs + (int)c[0], n = min(abs(xq - y), 63), n2 = min(2 * n, 63);
-                const longlong2 t0 = shift_right(q2, xq < y ? n2 : 0);
-                const longlong2 t1 = shift_right(real_scale(c[1], qs), n);
-                const longlong2 t2 = shift_right(real_scale(c[2], s2), xq < y ? 0 : n2);
+                const int64_t* c = ci + 4 * p;
+                const int f1 = x1 + (int)c[0], f2 = x2 + (int)c[2];
+                const int f = max(max(x0 + 1, max(f1, f2)) + 1, kLeast);
+                const longlong2 t0 = shift_right(q2, f - x0);
+                const longlong2 t1 = shift_right(real_scale(c[1], qs), f - f1);
+                const longlong2 t2 = shift_right(real_scale(c[3], s2), f - f2);
                 const BInt t = bint_words(make_longlong2(t0.x + t1.x + t2.x, t0.y + t1.y + t2.y));
                 h = first ? t : bmul(limbs(h), limbs(t));
                 first = false;
-                E += 2 * (st.xref - max(max(xq, y), kNone / 2));
+                E += st.ref2 - f;
                 bnorm(h, E);
             }
         }
         if (jodd) {
-            const int64_t* c = ci + 3 * P;
-            const int y = xs + (int)c[0], n = min(abs(xq - y), 63);
-            const longlong2 t0 = shift_right(qv, xq < y ? n : 0);
-            const longlong2 t1 = shift_right(real_scale(c[1], ls), xq < y ? 0 : n);
+            const int64_t* c = ci + 4 * P;
+            const int f1 = xs + (int)c[0] + 2, f = max(max(xq + 1, f1) + 1, kLeast);
+            const longlong2 t0 = shift_right(bint_pair(qw), f - xq);
+            const longlong2 t1 = shift_right(real_scale(c[1], ls), f - f1);
             const BInt t = bint_words(make_longlong2(t0.x + t1.x, t0.y + t1.y));
             h = first ? t : bmul(limbs(h), limbs(t));
             first = false;
-            E += st.xref - max(max(xq, y), kNone / 2);
+            E += st.ref1 - f;
             bnorm(h, E);
         }
     }
@@ -926,32 +934,24 @@ static std::vector<double> loop_factors(int N)
     return cf;
 }
 
-// The factors after the first as integers for haf_loop_poly: for each pair kp,
-// the exponent with 2 max|z| <= 2^kp over the pair's roots, and (times 2^63) a
-// 2^-kp and b 2^-2kp; for an odd root kp and -z 2^-kp.  The roots' sizes
-// descend, so the first kp is the largest.
+// The factors after the first as integers for haf_loop_poly: the exponent e
+// and v 2^(62 - e) in [2^61, 2^62) of a and b of each pair, and of -z of an odd
+// root.  The roots' sizes descend, so the first pair's exponents are the
+// largest.
 static std::vector<int64_t> loop_integers(const std::vector<double>& cf)
 {
     const int J = (int)cf.size() - 1, P = J / 2;
     std::vector<int64_t> ci;
-    auto scale_of = [](double z) {
+    auto add = [&](double v) {
         int e = 0;
-        std::frexp(2.0 * z * (1.0 + 0x1p-40), &e);
-        return e;
+        const double m = std::frexp(v, &e);
+        ci.push_back(e);
+        ci.push_back((int64_t)std::ldexp(m, 62));  // m < 1 has 53 bits: exact
     };
-    auto fixed = [](double v) { return (int64_t)std::llround(std::min(v, 0x1.ffp62)); };
-    for (int p = 0; p < P; ++p) {
-        const double a = cf[1 + 2 * p], b = cf[2 + 2 * p];
-        const int kp = scale_of(0.5 * (a + std::sqrt(std::max(0.0, a * a - 4.0 * b))));
-        ci.push_back(kp);
-        ci.push_back(fixed(std::ldexp(a, 63 - kp)));
-        ci.push_back(fixed(std::ldexp(b, 63 - 2 * kp)));
-    }
-    if (J % 2) {
-        const double c = -cf[1 + 2 * P];
-        ci.push_back(scale_of(c));
-        ci.push_back(fixed(std::ldexp(c, 63 - scale_of(c))));
-    }
+    for (int j = 1; j <= 2 * P; ++j)
+        add(cf[j]);
+    if (J % 2)
+        add(-cf[1 + 2 * P]);
     return ci;
 }
 
