@@ -22,11 +22,14 @@
 // the result is multiplied by the upstream gradient (PyTorch convention:
 // grad_b = grad_per * conj(G)).
 //
-// As in the forward kernel, every per-lane array lives in shared memory,
-// lane-major, and every loop over columns is a runtime loop, so the FP64 pipe
-// (the only loaded resource on GB300) sees no predicated or speculative work.
+// Product sides of at most kBwdRegMaxLd columns form their products in block
+// integers with the column sums in registers (below).  Wider ones use the
+// kernel that follows: all in FP64, every per-lane array in shared memory,
+// lane-major, and every loop over columns a runtime loop, so that the FP64 pipe
+// sees no predicated or speculative work.
 #include <cuda_runtime.h>
 
+#include "pq_blockint.cuh"
 #include "pq_device.cuh"
 #include "pq_kernels.h"
 
@@ -564,13 +567,16 @@ __global__ void __launch_bounds__(256, 2) glynn_bwd_kernel(BwdArgs a, int64_t t_
 }
 
 // ---------------------------------------------------------------- register-resident walk
-// For product-column bounds NL <= 14 a lane keeps its column sums S, its
-// accumulators A and the term's prefixes P in registers: every column loop is
-// unrolled over NL and columns j >= l are skipped by warp-uniform tests.  Only
-// the correction rows C stay in shared memory, so a warp needs about a third
-// of the shared memory of the kernel above and more warps fit on an SM (the
-// FP64 pipe of an SM sub-partition with a single warp idles whenever that
-// warp waits on a dependent result).
+// For product-column bounds NL <= kBwdRegMaxLd the column sums and the prefix
+// and suffix products are 64-bit block integers (pq_blockint.cuh) in registers,
+// as in the forward walk, and FP64 keeps the accumulations: per term and column
+// two conversions and two fused adds, and two DFMA for the corrections of a
+// step.  With the products in FP64 as well a column took 16 FP64 operations a
+// term, and the FP64 pipe (90% active) bound the walk.
+//
+// Every column loop is unrolled over NL, which is l or l + 1, and a column
+// j >= l is skipped by a warp-uniform test.  Only the correction rows C (and,
+// above kBwdRegAccLd columns, the accumulators A) are in shared memory.
 //
 // The factor c_j of the repeated columns is applied once, when the task's
 // gradient is written: the lanes accumulate A'_j = sum_t w_t Q_j(t) / c_j,
@@ -579,35 +585,43 @@ __global__ void __launch_bounds__(256, 2) glynn_bwd_kernel(BwdArgs a, int64_t t_
 // complex products in the prefix pass and (c_j - 1) in the suffix pass:
 // t = sw S_j^{c_j - 1}, A'_j += P_j t, sw = t S_j.
 //
+// A column's A' holds products of n - 1 sums: in the scaled integers it lacks
+// column j's factor 2^e_j, so column j of the gradient has its own exponent.
+//
 // Per-warp shared memory: base matrix M (kmax x ld), base column sums (ld),
 // a region that holds the correction rows C (jb x ld x kLS) during the walk
-// and, at the end of a task, the accumulators A' (ld x kLS) and the row
-// multipliers X (kmax x kLS doubles), then the correction sums V (jb x ld),
-// the weights wh (32) and small integer arrays.
+// and, at the end of a task, the accumulators A' (ld x kLS; above kBwdRegAccLd
+// columns they have a place of their own) and the row multipliers X (kmax x kLS
+// doubles), then the correction sums V (jb x ld), the weights wh (32) and small
+// integer arrays.
+constexpr int kBwdRegAccLd = 10;
+
 __host__ __device__ inline long bwdr_region_bytes(int kmax, int ld, int jb)
 {
-    const long walk = 16L * kLS * jb * ld;
-    const long end = 16L * kLS * ld + ((8L * kLS * kmax + 15) & ~15L);
+    const long acc = 16L * kLS * ld;
+    const long walk = 16L * kLS * jb * ld + (ld > kBwdRegAccLd ? acc : 0);
+    const long end = acc + ((8L * kLS * kmax + 15) & ~15L);
     return walk > end ? walk : end;
 }
 
 __host__ __device__ inline int bwdr_warp_smem_bytes(int kmax, int ld, int jb)
 {
     const long bytes = 16L * (kmax * ld + ld) + bwdr_region_bytes(kmax, ld, jb) + 16L * jb * ld +
-                       8L * 32 + 4L * (16 + ld + kmax);
+                       8L * 32 + 4L * (16 + 2 * ld + kmax);
     return (int)((bytes + 15) & ~15L);
 }
 
 struct BwdRegSmem {
-    double2* M;       // kmax x ld
+    double2* M;       // kmax x ld (scaled integers 2 b, or doubles for the FP64 walk)
     double2* base;    // ld
-    double2* C;       // jb x ld x kLS    -- region, during the walk
-    double2* A;       // ld x kLS         -- region, at the end of a task
-    double* X;        // kmax x kLS       -- region, at the end of a task
+    double2* A;       // ld x kLS         -- region: at the end of a task (or always)
+    double2* C;       // jb x ld x kLS    -- region: during the walk
+    double* X;        // kmax x kLS       -- region: at the end of a task
     double2* V;       // jb x ld
     double* wh;       // 32
     int32_t* lowrow;  // 16
     int32_t* cm;      // ld
+    int32_t* cexp;    // ld
     int32_t* rowdig;  // kmax
     int ld;
     __device__ BwdRegSmem(unsigned char* raw, int kmax, int ld_, int jb)
@@ -615,75 +629,311 @@ struct BwdRegSmem {
         ld = ld_;
         M = reinterpret_cast<double2*>(raw);
         base = M + kmax * ld;
-        C = base + ld;
-        A = C;
-        X = reinterpret_cast<double*>(reinterpret_cast<unsigned char*>(C) + 16L * kLS * ld);
-        V = reinterpret_cast<double2*>(reinterpret_cast<unsigned char*>(C) +
+        A = base + ld;
+        C = ld > kBwdRegAccLd ? A + kLS * ld : A;
+        X = reinterpret_cast<double*>(A + kLS * ld);
+        V = reinterpret_cast<double2*>(reinterpret_cast<unsigned char*>(A) +
                                        bwdr_region_bytes(kmax, ld, jb));
         wh = reinterpret_cast<double*>(V + jb * ld);
         lowrow = reinterpret_cast<int32_t*>(wh + 32);
         cm = lowrow + 16;
-        rowdig = cm + ld;
+        cexp = cm + ld;
+        rowdig = cexp + ld;
     }
 };
 
-// One term: A'_j += ws Q_j / c_j for j < l.  n2 = number of leading columns
-// with c_j >= 2 (their multiplicities in cm).
-template <int NL>
-__device__ __forceinline__ void bwdr_term(const double2 (&S)[NL], double2 (&A)[NL],
-                                          const int (&cm)[NL], int l, int n2, double ws)
+// What a warp keeps about the permanent it has staged.
+struct BwdStaged {
+    int perm = -1;
+    bool fp64 = false;  // staged as doubles
+    int exp2 = 0;       // column j of A' times 2^(exp2 + cexp[j])
+};
+
+__device__ void bwdr_stage(const BwdArgs& a, const PermDesc& D, const MetaView& mv, BwdRegSmem& sm,
+                           BwdStaged& st, int lane)
 {
-    // prefixes P_j = prod_{j' < j} S_{j'}^{c_{j'}}, j = 1 .. l-1
-    double2 P[NL];
-    double2 run = S[0];
-    if (n2 > 0) {
-#pragma unroll 1
-        for (int e = 1; e < cm[0]; ++e)
-            run = cmul(run, S[0]);
+    const int k = D.k, l = D.l;
+    bwd_stage(a, D, mv, sm, lane);  // doubles, and their base sums
+    bool bad = false;
+    for (int e = lane; e < k * l; e += kWarp) {
+        const int i = e / l;
+        const double2 b = sm.M[i * sm.ld + e - i * l];
+        bad = bad || not_finite(b.x) || not_finite(b.y);
     }
-    P[NL > 1 ? 1 : 0] = run;
-#pragma unroll
-    for (int j = 1; j < NL - 1; ++j) {
-        if (j < l - 1) {
-            run = cmul(run, S[j]);
-            if (j < n2) {
+    int esum = 0;
+    st.fp64 = !bint_stage(sm.M, sm.ld, k, l, mv.rmul, mv.cmul, sm.cexp, bad, lane, esum);
+    st.exp2 = 0;
+    if (st.fp64) {
+        for (int j = lane; j < l; j += kWarp)
+            sm.cexp[j] = 0;
+    } else {
+        const longlong2* M = reinterpret_cast<const longlong2*>(sm.M);
+        longlong2* base = reinterpret_cast<longlong2*>(sm.base);
+        for (int j = lane; j < l; j += kWarp)
+            base[j] = bint_base(M + j, sm.ld, k, mv.rmul);
+        // n - 1 factors, n - 2 products, each shifted down by 64
+        st.exp2 = kSumBits + 64 * (D.n - 2) - esum;
+    }
+    __syncwarp();
+}
+
+// A +-= w 2^(-kSumBits - E) p
+__device__ __forceinline__ void bwd_add(double2& A, const BInt& p, int E, double w, bool neg)
+{
+    const double f = bint_factor(w, E, neg);
+    A.x = __fma_rn(__ll2double_rn((long long)(((uint64_t)(uint32_t)p.rh << 32) | p.rl)), f, A.x);
+    A.y = __fma_rn(__ll2double_rn((long long)(((uint64_t)(uint32_t)p.ih << 32) | p.il)), f, A.y);
+}
+
+// One term: A'_j +-= w Q_j / c_j for j < l.  n2 = number of leading columns
+// with c_j >= 2 (their multiplicities in cm).  ACC(j) is column j's accumulator.
+template <int NL, class Acc>
+__device__ __forceinline__ void bwdr_term(const longlong2 (&S)[NL], const int32_t* cm, int l, int n2,
+                                          double w, bool neg, const Acc& acc)
+{
+    // prefixes P_j = prod_{j' < j} S_{j'}^{c_{j'}}, j = 1 .. l-1, normalised
+    BLimbs P[NL];
+    int EP[NL];
+    {
+        BInt run = bint_plain(S[0]);
+        int E = 0;
+        bnorm(run, E);
+        if (n2 > 0) {
+            const BLimbs s = sum_limbs(S[0]);
 #pragma unroll 1
-                for (int e = 1; e < cm[j]; ++e)
-                    run = cmul(run, S[j]);
+            for (int e = 1; e < cm[0]; ++e) {
+                run = bmul(limbs(run), s);
+                bnorm(run, E);
             }
-            P[j + 1] = run;
+        }
+        P[NL > 1 ? 1 : 0] = limbs(run);
+        EP[NL > 1 ? 1 : 0] = E;
+#pragma unroll
+        for (int j = 1; j < NL - 1; ++j) {
+            if (j < l - 1) {
+                const BLimbs s = sum_limbs(S[j]);
+                run = bmul(P[j], s);
+                bnorm(run, E);
+                if (j < n2) {
+#pragma unroll 1
+                    for (int e = 1; e < cm[j]; ++e) {
+                        run = bmul(limbs(run), s);
+                        bnorm(run, E);
+                    }
+                }
+                P[j + 1] = limbs(run);
+                EP[j + 1] = E;
+            }
         }
     }
-    // suffix pass, last column first; sw = ws prod_{j' > j} S_{j'}^{c_{j'}}
-    // (a separate branch for the last column, whose suffix is real, made the
-    // compiler keep S, A and P in local memory)
-    double2 sw = make_double2(ws, 0.0);
+    // suffix pass, last column first: t = prod_{j' > j} S_{j'}^{c_{j'}}, starting
+    // from 2^61 (which stands for 1: a product with it is shifted down by 3)
+    BInt t;
+    t.rh = 1 << 29;
+    t.rl = t.il = 0;
+    t.ih = 0;
+    int Et = -3;
 #pragma unroll
     for (int j = NL - 1; j >= 1; --j) {
         if (j < l) {
-            double2 t = sw;
+            const BLimbs s = sum_limbs(S[j]);
+            BLimbs lt = limbs(t);
             if (j < n2) {
 #pragma unroll 1
-                for (int e = 1; e < cm[j]; ++e)
-                    t = cmul(t, S[j]);
+                for (int e = 1; e < cm[j]; ++e) {
+                    t = bmul(lt, s);
+                    bnorm(t, Et);
+                    lt = limbs(t);
+                }
             }
-            cfma_acc<false>(A[j], P[j], t);
-            sw = cmul(t, S[j]);
+            const BInt q = bmul(P[j], lt);
+            t = bmul(lt, s);
+            const int E = EP[j] + Et;
+            bnorm(t, Et);
+            acc(j, q, E, w, neg);
         }
     }
     // column 0: S_0^{c_0 - 1} times the suffix (for l = 1 the weight alone)
-    double2 t = sw;
     if (n2 > 0) {
+        const BLimbs s = sum_limbs(S[0]);
 #pragma unroll 1
-        for (int e = 1; e < cm[0]; ++e)
-            t = cmul(t, S[0]);
+        for (int e = 1; e < cm[0]; ++e) {
+            t = bmul(limbs(t), s);
+            bnorm(t, Et);
+        }
     }
-    A[0].x = __dadd_rn(A[0].x, t.x);
-    A[0].y = __dadd_rn(A[0].y, t.y);
+    acc(0, t, Et, w, neg);
+}
+
+// The walk of this lane's chunk: the accumulators A' go to the region and the
+// corrections to C; returns the digits' Gray values at the chunk's end.
+template <int NL>
+__device__ __forceinline__ void bwdr_walk_int(const PermDesc& D, const MetaView& mv,
+                                              const BwdRegSmem& sm, const LowDigits& lo,
+                                              int64_t chunk, int n2, double2 (&A)[NL],
+                                              uint64_t& whigh_u, int& gpar, int lane)
+{
+    constexpr bool kRegAcc = NL <= kBwdRegAccLd;
+    const int l = D.l, J = D.J, ndig = D.ndig;
+    const longlong2* M = reinterpret_cast<const longlong2*>(sm.M);
+    const longlong2* base = reinterpret_cast<const longlong2*>(sm.base);
+    longlong2 S[NL];
+    double2* As = sm.A + lane;
+#pragma unroll
+    for (int j = 0; j < NL; ++j) {
+        S[j] = j < l ? base[j] : make_longlong2(0, 0);
+        if (kRegAcc)
+            A[j] = make_double2(0.0, 0.0);
+        else if (j < l)
+            As[j * kLS] = make_double2(0.0, 0.0);
+    }
+    // the high digits of this lane's chunk: column sums and weight
+    const bool narrow = D.nchunks <= 0x7fffffff;
+#pragma unroll 1
+    for (int d = J; d < ndig; ++d) {
+        const int g = next_digit(chunk, mv.drad[d], narrow);
+        if (g == 0)
+            continue;
+        const longlong2* Mr = M + mv.drow[d] * NL;
+#pragma unroll
+        for (int j = 0; j < NL; ++j) {
+            if (j < l) {
+                const longlong2 b = Mr[j];
+                S[j].x -= g * b.x;
+                S[j].y -= g * b.y;
+            }
+        }
+        whigh_u *= high_binom(mv.dtop[d], g);
+        gpar += g;
+    }
+#pragma unroll 1
+    for (int d = 0; d < J; ++d)
+#pragma unroll 1
+        for (int j = 0; j < l; ++j)
+            sm.C[(d * NL + j) * kLS + lane] = make_double2(0.0, 0.0);
+    auto acc = [&](int j, const BInt& q, int E, double w, bool neg) {
+        if (kRegAcc) {
+            bwd_add(A[j], q, E, w, neg);
+        } else {
+            double2 v = As[j * kLS];
+            bwd_add(v, q, E, w, neg);
+            As[j * kLS] = v;
+        }
+    };
+    const bool weighted = D.weighted != 0;
+    const uint32_t L = (uint32_t)D.L;
+    uint32_t steps = 0;
+    double step_w = 1.0, w = 1.0;
+    uint32_t s = 0;
+#pragma unroll 1
+    for (;;) {
+        bwdr_term<NL>(S, sm.cm, l, n2, w, (s & 1u) != 0, acc);
+        if (++s == L)
+            break;
+        // the Gray steps 32 at a time, one per lane, as in the forward walk
+        const int q = (int)((s - 1u) & 31u);
+        if (q == 0) {
+            bool up;
+            uint64_t wu;
+            const int d = gray_step_at(lo, s + (uint32_t)lane, weighted, up, wu);
+            steps = ((uint32_t)d << 1) | (up ? 0u : 1u);
+            step_w = (double)wu;
+        }
+        const uint32_t step = __shfl_sync(0xffffffffu, steps, q);
+        if (weighted)
+            w = __shfl_sync(0xffffffffu, step_w, q);
+        const int d = (int)(step >> 1);
+        const bool down = (step & 1u) != 0;
+        const longlong2* Mr = M + sm.lowrow[d] * NL;
+        double2* Cd = sm.C + d * NL * kLS + lane;
+        const double delta = down ? 2.0 : -2.0;
+#pragma unroll
+        for (int j = 0; j < NL; ++j) {
+            if (j < l) {
+                const longlong2 b = Mr[j];
+                S[j].x = down ? S[j].x + b.x : S[j].x - b.x;
+                S[j].y = down ? S[j].y + b.y : S[j].y - b.y;
+                const double2 av = kRegAcc ? A[j] : As[j * kLS];
+                double2 cv = Cd[j * kLS];
+                cv.x = __fma_rn(delta, av.x, cv.x);
+                cv.y = __fma_rn(delta, av.y, cv.y);
+                Cd[j * kLS] = cv;
+            }
+        }
+    }
+}
+
+// The same walk in FP64, for a base matrix without integer scales (non-finite
+// entries, a column bound beyond FP64), with the lane's arrays in local memory.
+__device__ __noinline__ void bwdr_walk_fp64(const PermDesc& D, const MetaView& mv,
+                                            const BwdRegSmem& sm, const LowDigits& lo,
+                                            int64_t chunk, int n2, double2* A, uint64_t& whigh_u,
+                                            int& gpar, int lane)
+{
+    const int l = D.l, ld = sm.ld;
+    double2 S[kBwdRegMaxLd], P[kBwdRegMaxLd];
+    for (int j = 0; j < l; ++j) {
+        S[j] = sm.base[j];
+        A[j] = make_double2(0.0, 0.0);
+    }
+    auto add_row = [&](int row, double coef) {
+        for (int j = 0; j < l; ++j) {
+            const double2 b = sm.M[row * ld + j];
+            S[j].x = __fma_rn(coef, b.x, S[j].x);
+            S[j].y = __fma_rn(coef, b.y, S[j].y);
+        }
+    };
+    for (int d = D.J; d < D.ndig; ++d) {
+        const int g = next_digit(chunk, mv.drad[d], false);
+        if (g == 0)
+            continue;
+        add_row(mv.drow[d], (double)(-2 * g));
+        whigh_u *= high_binom(mv.dtop[d], g);
+        gpar += g;
+    }
+    for (int d = 0; d < D.J; ++d)
+        for (int j = 0; j < l; ++j)
+            sm.C[(d * ld + j) * kLS + lane] = make_double2(0.0, 0.0);
+    double w = 1.0;
+    for (uint32_t s = 0;;) {
+        double2 run = S[0];
+        for (int e = 1; e < sm.cm[0]; ++e)
+            run = cmul(run, S[0]);
+        for (int j = 1; j < l; ++j) {
+            P[j] = run;
+            for (int e = 0; e < sm.cm[j]; ++e)
+                run = cmul(run, S[j]);
+        }
+        double2 t = make_double2((s & 1u) ? -w : w, 0.0);
+        for (int j = l - 1; j >= 0; --j) {
+            for (int e = 1; e < sm.cm[j]; ++e)
+                t = cmul(t, S[j]);
+            if (j > 0) {
+                cfma_acc<false>(A[j], P[j], t);
+                t = cmul(t, S[j]);
+            } else {
+                A[0].x = __dadd_rn(A[0].x, t.x);
+                A[0].y = __dadd_rn(A[0].y, t.y);
+            }
+        }
+        if (++s == (uint32_t)D.L)
+            break;
+        bool up;
+        uint64_t wu;
+        const int d = gray_step_at(lo, s, true, up, wu);
+        w = (double)wu;
+        const double delta = up ? -2.0 : 2.0;
+        add_row(sm.lowrow[d], delta);
+        for (int j = 0; j < l; ++j) {
+            double2* cv = sm.C + (d * ld + j) * kLS + lane;
+            cv->x = __fma_rn(delta, A[j].x, cv->x);
+            cv->y = __fma_rn(delta, A[j].y, cv->y);
+        }
+    }
 }
 
 template <int NL>
-__device__ void bwdr_task(const BwdArgs& a, const Task& t, BwdRegSmem& sm, int& staged, int lane)
+__device__ void bwdr_task(const BwdArgs& a, const Task& t, BwdRegSmem& sm, BwdStaged& st, int lane)
 {
     const PermDesc D = a.desc[t.perm];
     const MetaView mv = meta_view(a.meta, D);
@@ -693,98 +943,35 @@ __device__ void bwdr_task(const BwdArgs& a, const Task& t, BwdRegSmem& sm, int& 
 
     if (!D.trivial) {
         __syncwarp();  // the previous task's contraction read the region that C reuses
-        if (staged != t.perm) {
-            bwd_stage(a, D, mv, sm, lane);
-            staged = t.perm;
+        if (st.perm != t.perm) {
+            bwdr_stage(a, D, mv, sm, st, lane);
+            st.perm = t.perm;
         }
         const int64_t chunk0 = (int64_t)t.part * kWarp;
         const bool active = chunk0 + lane < D.nchunks;
         const int64_t chunk = active ? (chunk0 + lane) : 0;
-        double2 S[NL], A[NL];
-        int cm[NL];
-#pragma unroll
-        for (int j = 0; j < NL; ++j) {
-            S[j] = j < l ? sm.base[j] : make_double2(0.0, 0.0);
-            A[j] = make_double2(0.0, 0.0);
-            cm[j] = j < l ? sm.cm[j] : 1;
-        }
-        // the high digits of this lane's chunk: column sums and weight
+        const LowDigits lo = low_digits(mv, J);
+        int n2 = 0;
+        while (n2 < l && sm.cm[n2] >= 2)
+            ++n2;
+        double2 A[NL];
         uint64_t whigh_u = 1;
         int gpar = 0;
-        int64_t c = chunk;
-#pragma unroll 1
-        for (int d = J; d < ndig; ++d) {
-            const int rad = mv.drad[d];
-            const int g = (int)(c % rad);
-            c /= rad;
-            if (g == 0)
-                continue;
-            const double2* Mr = sm.M + mv.drow[d] * NL;
-            const double coef = (double)(-2 * g);
+        bool in_regs = NL <= kBwdRegAccLd;
+        if (st.fp64) {
+            double2 Af[kBwdRegMaxLd];
+            bwdr_walk_fp64(D, mv, sm, lo, chunk, n2, Af, whigh_u, gpar, lane);
 #pragma unroll
-            for (int j = 0; j < NL; ++j) {
-                if (j < l) {
-                    const double2 b = Mr[j];
-                    S[j].x = __fma_rn(coef, b.x, S[j].x);
-                    S[j].y = __fma_rn(coef, b.y, S[j].y);
-                }
-            }
-            whigh_u *= binom_u64(mv.dtop[d], g);
-            gpar += g;
+            for (int j = 0; j < NL; ++j)
+                A[j] = j < l ? Af[j] : make_double2(0.0, 0.0);
+            in_regs = true;
+        } else {
+            bwdr_walk_int<NL>(D, mv, sm, lo, chunk, n2, A, whigh_u, gpar, lane);
         }
         double whigh = active ? (double)whigh_u : 0.0;
         if (gpar & 1)
             whigh = -whigh;
         sm.wh[lane] = whigh;
-        for (int e = 0; e < J * l; ++e) {
-            const int d = e / l, j = e - d * l;
-            sm.C[(d * NL + j) * kLS + lane] = make_double2(0.0, 0.0);
-        }
-        int n2 = 0;
-        while (n2 < l && sm.cm[n2] >= 2)
-            ++n2;
-        uint32_t lowrows = 0;  // row of low digit d in bits [6d, 6d + 6): rows < 64
-        for (int d = 0; d < J; ++d)
-            lowrows |= (uint32_t)sm.lowrow[d] << (6 * d);
-
-        LowWalk wk;
-        wk.v = 0;
-        wk.g = 0;
-        wk.dir = 0;
-        wk.radm1 = 0;
-        wk.topp = 0;
-        for (int d = 0; d < J; ++d) {
-            wk.radm1 |= uint64_t(mv.drad[d] - 1) << (4 * d);
-            wk.topp |= uint64_t(mv.dtop[d]) << (4 * d);
-        }
-        double wlow = 1.0;
-        const int64_t L = D.L;
-#pragma unroll 1
-        for (int64_t s = 0; s < L; ++s) {
-            bwdr_term<NL>(S, A, cm, l, n2, (s & 1) ? -wlow : wlow);
-            if (s + 1 < L) {
-                int up;
-                const int d = low_step(wk, up);
-                const int row = (int)((lowrows >> (6 * d)) & 63u);
-                const double delta = up > 0 ? -2.0 : 2.0;
-                const double2* Mr = sm.M + row * NL;
-                double2* Cd = sm.C + d * NL * kLS + lane;
-#pragma unroll
-                for (int j = 0; j < NL; ++j) {
-                    if (j < l) {
-                        const double2 b = Mr[j];
-                        double2 cv = Cd[j * kLS];
-                        S[j].x = __fma_rn(delta, b.x, S[j].x);
-                        S[j].y = __fma_rn(delta, b.y, S[j].y);
-                        cv.x = __fma_rn(delta, A[j].x, cv.x);
-                        cv.y = __fma_rn(delta, A[j].y, cv.y);
-                        Cd[j * kLS] = cv;
-                    }
-                }
-                if (((wk.radm1 >> (4 * d)) & 15u) > 1u)
-                    wlow = (double)low_weight(wk, J);
-            }
-        }
         // Contraction, as in the kernel above: V from the corrections first,
         // then the accumulators and row multipliers go to the region that
         // held the corrections.
@@ -801,25 +988,27 @@ __device__ void bwdr_task(const BwdArgs& a, const Task& t, BwdRegSmem& sm, int& 
             sm.V[d * NL + j] = make_double2(vx, vy);
         }
         __syncwarp();
+        if (in_regs) {
 #pragma unroll
-        for (int j = 0; j < NL; ++j)
-            if (j < l)
-                sm.A[j * kLS + lane] = A[j];
+            for (int j = 0; j < NL; ++j)
+                if (j < l)
+                    sm.A[j * kLS + lane] = A[j];
+        }
         {
             const double whl = sm.wh[lane];
             double* X = sm.X + lane;
             for (int i = 0; i < k; ++i)
                 X[i * kLS] = whl * (double)mv.rmul[i];
             int64_t cc = chunk;
+            const bool narrow = D.nchunks <= 0x7fffffff;
             for (int d = J; d < ndig; ++d) {
-                const int rad = mv.drad[d];
-                const int g = (int)(cc % rad);
-                cc /= rad;
+                const int g = next_digit(cc, mv.drad[d], narrow);
                 const int row = mv.drow[d];
                 X[row * kLS] = whl * (double)(mv.rmul[row] - 2 * g);
             }
+            const uint64_t gv = gray_value_at(lo, (uint32_t)D.L - 1u);
             for (int d = 0; d < J; ++d) {
-                const int g = (int)((wk.g >> (4 * d)) & 15u);
+                const int g = (int)((gv >> (4 * d)) & 15u);
                 const int row = sm.lowrow[d];
                 X[row * kLS] = whl * (double)(mv.rmul[row] - 2 * g);
             }
@@ -842,8 +1031,9 @@ __device__ void bwdr_task(const BwdArgs& a, const Task& t, BwdRegSmem& sm, int& 
                 gy = __dsub_rn(gy, v.y);
             }
             const double cj = (double)sm.cm[j];
-            slot[2 * e] = cj * gx;
-            slot[2 * e + 1] = cj * gy;
+            const int x = st.exp2 + sm.cexp[j];
+            slot[2 * e] = scalbn(cj * gx, x);
+            slot[2 * e + 1] = scalbn(cj * gy, x);
         }
     }
     bwd_combine(a, t, D, kl, lane);
@@ -853,14 +1043,14 @@ __device__ void bwdr_task(const BwdArgs& a, const Task& t, BwdRegSmem& sm, int& 
 // class bound); the guards are those of the kernel above, without a bound on
 // the repeated columns.
 template <int NL>
-__global__ void __launch_bounds__(256, 1) glynn_bwd_reg_kernel(BwdArgs a, int64_t t_begin,
+__global__ void __launch_bounds__(256, NL <= 4 ? 2 : 1) glynn_bwd_reg_kernel(BwdArgs a, int64_t t_begin,
                                                             int64_t t_end, int kmax, int jb,
                                                             int queue)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     BwdRegSmem sm(smem_raw + warp * bwdr_warp_smem_bytes(kmax, NL, jb), kmax, NL, jb);
-    int staged = -1;
+    BwdStaged st;
     if (!queue) {
         const int64_t ti = t_begin + (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
         if (ti >= t_end)
@@ -871,7 +1061,7 @@ __global__ void __launch_bounds__(256, 1) glynn_bwd_reg_kernel(BwdArgs a, int64_
                 record_error(a.err, bad, ti);
             return;
         }
-        bwdr_task<NL>(a, a.tasks[ti], sm, staged, lane);
+        bwdr_task<NL>(a, a.tasks[ti], sm, st, lane);
         return;
     }
     for (;;) {
@@ -888,7 +1078,7 @@ __global__ void __launch_bounds__(256, 1) glynn_bwd_reg_kernel(BwdArgs a, int64_
                 record_error(a.err, bad, ti);
             continue;
         }
-        bwdr_task<NL>(a, a.tasks[ti], sm, staged, lane);
+        bwdr_task<NL>(a, a.tasks[ti], sm, st, lane);
     }
 }
 
@@ -1032,6 +1222,7 @@ static const void* bwdr_kernel_for(int ld)
     case 10: return (const void*)glynn_bwd_reg_kernel<10>;
     case 12: return (const void*)glynn_bwd_reg_kernel<12>;
     case 14: return (const void*)glynn_bwd_reg_kernel<14>;
+    case 16: return (const void*)glynn_bwd_reg_kernel<16>;
     default: return nullptr;
     }
 }
@@ -1077,6 +1268,7 @@ static cudaError_t bwdr_launch(int ld, const BwdArgs& a, int64_t t_begin, int64_
     case 10: bwdr_launch_nl<10>(a, t_begin, t_end, kmax, jb, grid, wpb, queue, st); break;
     case 12: bwdr_launch_nl<12>(a, t_begin, t_end, kmax, jb, grid, wpb, queue, st); break;
     case 14: bwdr_launch_nl<14>(a, t_begin, t_end, kmax, jb, grid, wpb, queue, st); break;
+    case 16: bwdr_launch_nl<16>(a, t_begin, t_end, kmax, jb, grid, wpb, queue, st); break;
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();

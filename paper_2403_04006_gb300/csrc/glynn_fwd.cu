@@ -83,11 +83,6 @@ struct Staged {
     bool fp64 = false;  // staged as doubles, for fp64_walk
 };
 
-__device__ __forceinline__ bool not_finite(double x)
-{
-    return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000;
-}
-
 // Copy the oriented base matrix of permanent D into shared memory as scaled
 // integers and form base_j = sum_i r_i b_ij (all Gray digits at zero).
 __device__ void stage_perm(const ExecArgs& a, const PermDesc& D, const MetaView& mv, WarpSmem& sm,
@@ -108,32 +103,9 @@ __device__ void stage_perm(const ExecArgs& a, const PermDesc& D, const MetaView&
     for (int j = lane; j < l; j += kWarp)
         sm.ecnt[j] = mv.ecnt[j];
     __syncwarp();
-    int xsum = 0;
-    for (int j = lane; j < l; j += kWarp) {
-        uint32_t hmax = 0, units = 0;
-        for (int i = 0; i < k; ++i) {
-            const double2 b = Md[i * sm.ld + j];
-            hmax = max(hmax, bint_mag(b.x, b.y));
-        }
-        for (int i = 0; i < k; ++i) {
-            const double2 b = Md[i * sm.ld + j];
-            units += (uint32_t)mv.rmul[i] * bint_units(bint_mag(b.x, b.y), hmax);
-        }
-        int e = bint_scale(hmax, units);
-        if (hmax < 0x100000u) {
-            uint64_t sum = 0;
-            for (int i = 0; i < k; ++i) {
-                const double2 b = Md[i * sm.ld + j];
-                sum += (uint64_t)mv.rmul[i] * bint_mag_subnormal(b.x, b.y);
-            }
-            e = bint_scale_subnormal(sum);
-        }
-        bad = bad || e < kSumBits - 1024;  // the sums can overflow FP64
-        sm.cexp[j] = e;
-        xsum += mv.cmul[j] * e;
-    }
+    int esum = 0;
     st.perm = -1;
-    st.fp64 = __any_sync(0xffffffffu, bad);
+    st.fp64 = !bint_stage(Md, sm.ld, k, l, mv.rmul, mv.cmul, sm.cexp, bad, lane, esum);
     if (st.fp64) {
         double2* base = reinterpret_cast<double2*>(sm.base);
         for (int j = lane; j < l; j += kWarp) {
@@ -150,29 +122,15 @@ __device__ void stage_perm(const ExecArgs& a, const PermDesc& D, const MetaView&
         __syncwarp();
         return;
     }
-    __syncwarp();
-    for (int e = lane; e < k * l; e += kWarp) {
-        const int i = e / l, j = e - i * l;
-        const double2 b = Md[i * sm.ld + j];
-        const int x = sm.cexp[j];
-        sm.M[i * sm.ld + j] = make_longlong2(2 * bint_of(b.x, x), 2 * bint_of(b.y, x));
-    }
-    __syncwarp();
     uint32_t em = 0;
     for (int j = lane; j < l; j += kWarp) {
-        longlong2 s = make_longlong2(kSumBias, kSumBias);
-        for (int i = 0; i < k; ++i) {
-            const longlong2 b = sm.M[i * sm.ld + j];
-            s.x += mv.rmul[i] * (b.x >> 1);
-            s.y += mv.rmul[i] * (b.y >> 1);
-        }
-        sm.base[j] = s;
+        sm.base[j] = bint_base(sm.M + j, sm.ld, k, mv.rmul);
         if (j < 32 && sm.ecnt[j] > 0)
             em |= 1u << j;
     }
     st.emask = __reduce_or_sync(0xffffffffu, em);
     // n - 1 products, each shifted down by 64; the terms carry 2^-kSumBits
-    st.exp2 = kSumBits + 64 * (D.n - 1) - __reduce_add_sync(0xffffffffu, xsum);
+    st.exp2 = kSumBits + 64 * (D.n - 1) - esum;
     __syncwarp();
 }
 
@@ -463,13 +421,7 @@ __device__ __forceinline__ dd2 int_walk(const PermDesc& D, const MetaView& mv, c
         gpar += g;
     }
 
-    LowDigits lo;
-    lo.radm1 = lo.topp = 0;
-    lo.J = J;
-    for (int d = 0; d < J; ++d) {
-        lo.radm1 |= uint64_t(mv.drad[d] - 1) << (4 * d);
-        lo.topp |= uint64_t(mv.dtop[d]) << (4 * d);
-    }
+    const LowDigits lo = low_digits(mv, J);
     const bool weighted = D.weighted != 0;
     const int jf = D.jf;
     // The Gray steps are the same for all lanes.  Every 32 steps each lane

@@ -522,19 +522,8 @@ static double bwd_instr_per_term(const ItemPlan& it, bool reg)
     if (it.n == 1)
         return 2.0;
     const int l = it.l;
-    if (reg) {
-        // register-resident walk: the step 4l, column 0's add 2; prefix
-        // products c_j for columns 1 .. l-2 and c_0 - 1 for column 0; per
-        // suffix column j >= 1 its c_j - 1 powers, the accumulation and the
-        // suffix update, 4(c_j - 1) + 8; column 0's c_0 - 1 powers
-        const std::vector<int32_t>& c = it.cmul;
-        double v = 4.0 * l + 2.0 + 8.0 * (c[0] - 1);
-        for (int j = 1; j < l - 1; ++j)
-            v += 4.0 * c[j];
-        for (int j = 1; j < l; ++j)
-            v += 4.0 * (c[j] - 1) + 8.0;
-        return v;
-    }
+    if (reg)  // products in integers: the accumulations 4l, the corrections 2l
+        return 6.0 * l;
     double rep = 0.0;
     for (int c : it.cmul)
         if (c >= 2)
@@ -1510,8 +1499,9 @@ static int ensure_backward(pq_plan* P)
             int wpb = 0, bps = 0;
             launch_geometry_max(regs, per_warp, 8, wpb, bps);
             const double warps = std::min(8.0, (double)(wpb * bps)) / 8.0;
-            const double per_term = 16.0 * C.ld - 10.0;
-            const double start = std::max(0.0, nbar - J) * 2.0 * C.ld / (double)(1 << J);
+            const double per_term = C.reg ? 6.0 * C.ld : 16.0 * C.ld - 10.0;
+            const double start = std::max(0.0, nbar - J) * (C.reg ? 0.5 : 2.0) * C.ld /
+                                 (double)(1 << J);
             const double score = warps * per_term / (per_term + start);
             if (score > best) {
                 best = score;
@@ -1538,7 +1528,8 @@ static int ensure_backward(pq_plan* P)
     auto bwd_cut_cost = [&](const ItemPlan& it, const BwdClass& C) {
         CutCost bc;
         bc.per_term = bwd_instr_per_term(it, C.reg != 0);
-        bc.per_high = 2.0 * it.l;
+        // (in the register walk a high digit is integer work, about a quarter)
+        bc.per_high = C.reg ? 0.5 * it.l + 1.0 : 2.0 * it.l;
         bc.per_task = it.k + 66.0 * it.k * it.l / 32.0;
         bc.per_task_low = 2.0 * it.l;
         return bc;
@@ -1629,7 +1620,8 @@ static int ensure_backward(pq_plan* P)
             // every lane of a task walks L terms and starts its chunk from the
             // high digits; the task ends with the lane contraction
             const double lane = (double)it.L * bwd_instr_per_term(it, C.reg != 0) +
-                                2.0 * it.l * (double)((int)it.drad.size() - it.J);
+                                (C.reg ? 0.0 : 2.0 * it.l) *
+                                    (double)((int)it.drad.size() - it.J);
             instr_b += (double)nt * (32.0 * lane + 32.0 * it.k + 64.0 * it.J * it.l + 66.0 * kl);
         }
     }

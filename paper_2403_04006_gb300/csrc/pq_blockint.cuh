@@ -212,6 +212,72 @@ __device__ __forceinline__ double bint_factor(double w, int E, bool neg)
     return h >= 0x100000 ? __hiloint2double(h | (neg ? (int)0x80000000 : 0), __double2loint(w))
                          : 0.0;
 }
+
+__device__ __forceinline__ bool not_finite(double x)
+{
+    return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000;
+}
+
+// Turn a staged base matrix (k x l doubles in shared memory, row stride ld,
+// row multiplicities rmul, column multiplicities cmul; one warp) into scaled
+// integers 2 b_ij in place: cexp[j] receives column j's exponent and esum the
+// sum of c_j cexp[j].  Returns false, with the doubles left as they are, if a
+// lane passes bad (a non-finite entry) or a column's sums can overflow FP64.
+__device__ __forceinline__ bool bint_stage(double2* Md, int ld, int k, int l, const int32_t* rmul,
+                                           const int32_t* cmul, int32_t* cexp, bool bad, int lane,
+                                           int& esum)
+{
+    int x = 0;
+    for (int j = lane; j < l; j += 32) {
+        uint32_t hmax = 0, units = 0;
+        for (int i = 0; i < k; ++i) {
+            const double2 b = Md[i * ld + j];
+            hmax = max(hmax, bint_mag(b.x, b.y));
+        }
+        for (int i = 0; i < k; ++i) {
+            const double2 b = Md[i * ld + j];
+            units += (uint32_t)rmul[i] * bint_units(bint_mag(b.x, b.y), hmax);
+        }
+        int e = bint_scale(hmax, units);
+        if (hmax < 0x100000u) {
+            uint64_t sum = 0;
+            for (int i = 0; i < k; ++i) {
+                const double2 b = Md[i * ld + j];
+                sum += (uint64_t)rmul[i] * bint_mag_subnormal(b.x, b.y);
+            }
+            e = bint_scale_subnormal(sum);
+        }
+        bad = bad || e < kSumBits - 1024;  // the sums can overflow FP64
+        cexp[j] = e;
+        x += cmul[j] * e;
+    }
+    if (__any_sync(0xffffffffu, bad))
+        return false;
+    esum = __reduce_add_sync(0xffffffffu, x);
+    __syncwarp();
+    longlong2* M = reinterpret_cast<longlong2*>(Md);
+    for (int e = lane; e < k * l; e += 32) {
+        const int i = e / l, j = e - i * l;
+        const double2 b = Md[i * ld + j];
+        const int c = cexp[j];
+        M[i * ld + j] = make_longlong2(2 * bint_of(b.x, c), 2 * bint_of(b.y, c));
+    }
+    __syncwarp();
+    return true;
+}
+
+// sum_i r_i b_ij of a staged column (all Gray digits at zero), biased.
+__device__ __forceinline__ longlong2 bint_base(const longlong2* Mj, int ld, int k,
+                                               const int32_t* rmul)
+{
+    longlong2 s = make_longlong2(kSumBias, kSumBias);
+    for (int i = 0; i < k; ++i) {
+        const longlong2 b = Mj[i * ld];
+        s.x += rmul[i] * (b.x >> 1);
+        s.y += rmul[i] * (b.y >> 1);
+    }
+    return s;
+}
 #endif
 
 }  // namespace pqi

@@ -320,4 +320,31 @@ __host__ __device__ __forceinline__ int gray_step_at(const LowDigits& lo, uint32
     return digit < 0 ? 0 : digit;
 }
 
+// Gray value of every low digit at term s, 4 bits each.
+__host__ __device__ __forceinline__ uint64_t gray_value_at(const LowDigits& lo, uint32_t s)
+{
+    uint64_t r1 = lo.radm1, g = 0;
+    uint32_t x = s;
+    for (int d = 0; d < lo.J; ++d) {
+        const uint32_t r = (uint32_t)(r1 & 15u) + 1u;
+        const uint32_t q = x / r, v = x - q * r;
+        g |= (uint64_t)((q & 1u) ? r - 1u - v : v) << (4 * d);
+        x = q;
+        r1 >>= 4;
+    }
+    return g;
+}
+
+__device__ __forceinline__ LowDigits low_digits(const MetaView& mv, int J)
+{
+    LowDigits lo;
+    lo.radm1 = lo.topp = 0;
+    lo.J = J;
+    for (int d = 0; d < J; ++d) {
+        lo.radm1 |= uint64_t(mv.drad[d] - 1) << (4 * d);
+        lo.topp |= uint64_t(mv.dtop[d]) << (4 * d);
+    }
+    return lo;
+}
+
 }  // namespace pqi

@@ -105,9 +105,9 @@ cudaError_t bwd_launch_persistent(int ld, const BwdArgs& a, int64_t t_begin, int
                                   int kmax, int jb, int n2, int blocks, int wpb, cudaStream_t st);
 cudaError_t bwd_launch_plain(int lmax, const BwdArgs& a, int64_t t_begin, int64_t t_end,
                              int kmax, int jb, int n2, int wpb, cudaStream_t st);
-// The register-resident walk (column sums, accumulators and prefixes in
-// registers) for even product-column bounds up to kBwdRegMaxLd.
-constexpr int kBwdRegMaxLd = 14;
+// The register-resident walk (column sums and prefixes in registers) for even
+// product-column bounds up to kBwdRegMaxLd.
+constexpr int kBwdRegMaxLd = 16;
 bool bwdr_supported(int ld);
 int bwdr_smem_bytes_for(int kmax, int ld, int jb);
 int bwdr_regs_per_thread(int ld);

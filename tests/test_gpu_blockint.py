@@ -4,6 +4,9 @@ range, entries that vanish beside the largest, exact zeros, and inputs that have
 no scale at all (non-finite, or a bound beyond FP64).  Permanents are compared
 with exact rational values; the bound is that of an FP64 evaluation of the Glynn
 sum, 8 n 2^-53 of the mean absolute term."""
+import itertools
+import math
+
 import numpy as np
 import pytest
 
@@ -191,3 +194,90 @@ def test_hafnians_without_a_scale(dev, loop, bad):
     assert np.array_equal(got[[0, 1, 2, 6, 7, 8]].view(np.float64), want.view(np.float64))
     assert not np.isfinite(got[3:5]).any()
     assert got[5] == 0
+
+
+# ------------------------------------------------------------------ gradients
+def gray_terms(m):
+    """Terms when this side is summed: one copy of its least repeated line fixed."""
+    return math.prod(int(x) + 1 for x in m) // (min(m) + 1) * min(m)
+
+
+def grad_abs(B, r, c):
+    """c_j times the mean over the sign vectors of |x_i| |prod of the column sums
+    without one factor S_j|, rows summed: the size of the gradient's terms."""
+    g = np.array(list(itertools.product(*[range(int(x) + 1) for x in r])))
+    w = np.prod([[math.comb(int(ri), int(q)) for ri, q in zip(r, row)] for row in g], axis=1)
+    x = np.asarray(r) - 2 * g
+    S = np.abs(x @ B)
+    out = np.zeros(B.shape)
+    for j in range(B.shape[1]):
+        e = np.asarray(c) - (np.arange(B.shape[1]) == j)
+        q = w * np.prod(S ** e, axis=1)
+        out[:, j] = c[j] * (np.abs(x) * q[:, None]).sum(axis=0) / 2.0 ** int(sum(r))
+    return out
+
+
+@pytest.mark.parametrize("method", ["batched", "plain"])
+def test_gradient_scales(dev, method):
+    """dper/db of every product width up to 18, the product side's columns scaled
+    by powers of two (scaling the summed side would cancel in any arithmetic of
+    53 or 64 bits), repeated rows and columns and zero entries, against the
+    oracle's minors, within 16 n 2^-53 of the terms' size (n - 1 products, the
+    sums' updates and the accumulation in FP64)."""
+    rng = np.random.default_rng(7)
+    items, flip = [], []
+    for l in list(range(1, 11)) + [12, 13, 14, 15, 16, 17, 18]:
+        k = min(l, 5)
+        B = rng.standard_normal((k, l)) + 1j * rng.standard_normal((k, l))
+        c = [1] * l if l > 8 else list(rng.integers(1, 4, l))
+        n = int(sum(c))
+        r = [n // k + (i < n % k) for i in range(k)]
+        flip.append(gray_terms(c) < gray_terms(r))  # the columns are summed
+        e = rng.integers(-60, 61, (k, 1) if flip[-1] else (1, l))
+        B = np.ldexp(B.real, e) + 1j * np.ldexp(B.imag, e)
+        if l == 7:
+            B[1, 2:4] = 0
+        items.append((B, r, c))
+    pb = W.pack_batch(items)
+    go = torch.ones(pb.batch, dtype=torch.complex128, device=dev)
+    db = api.DeviceBatch(pb, dev)
+    plan = api.Plan.for_batch(pb, method=method)
+    got = api.permanent_backward(db, go, plan).cpu().numpy()
+    for b, (B, r, c) in enumerate(items):
+        if flip[b]:  # the oracle, too, has to sum the side that is not scaled
+            want, size = O.perm_grad(B.T, c, r, gold=True).T, grad_abs(B.T, c, r).T
+        else:
+            want, size = O.perm_grad(B, r, c, gold=True), grad_abs(B, r, c)
+        want = np.conj(want)
+        g = got[pb.mat_off[b]:pb.mat_off[b] + B.size].reshape(B.shape)
+        assert (abs(g - want) <= 16 * sum(r) * 2.0 ** -53 * size).all(), b
+
+
+@pytest.mark.parametrize("method", ["batched", "plain"])
+@pytest.mark.parametrize("bad", [np.inf, np.nan, 1.7e308])
+def test_gradients_without_a_scale(dev, method, bad):
+    """A non-finite entry makes its permanent's gradient not finite somewhere;
+    the gradients beside it keep their bits."""
+    rng = np.random.default_rng(8)
+    clean = []
+    for n in (2, 3, 6, 10, 13):
+        clean.append((rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n)),
+                      [1] * n, [1] * n))
+    dirty = []
+    for A, r, c in clean:
+        A = A.copy()
+        A[0, 0] = A[1, 0] = bad
+        dirty.append((A, r, c))
+
+    def grads(items):
+        pb = W.pack_batch(items)
+        go = torch.ones(pb.batch, dtype=torch.complex128, device=dev)
+        g = api.permanent_backward(api.DeviceBatch(pb, dev), go, api.Plan.for_batch(pb, method=method))
+        g = g.cpu().numpy()
+        return [g[o:o + B.size] for o, (B, _, _) in zip(pb.mat_off, items)]
+
+    want = grads(clean)
+    got = grads([x for pair in zip(clean, dirty) for x in pair])
+    for q in range(len(clean)):
+        assert np.array_equal(got[2 * q].view(np.float64), want[q].view(np.float64))
+        assert not np.isfinite(got[2 * q + 1]).all()
