@@ -65,16 +65,26 @@ __global__ void sampler_gather_kernel(const double2* U, int m, int n, int k, int
 // and the draw: the first mode whose running weight sum exceeds u * total,
 // else the last mode with a positive weight; a sample whose weights are all
 // zero records an error and draws mode 0 so that later steps stay in bounds.
-__global__ void sampler_step_kernel(const double2* U, int m, int n, int k, int64_t nsamples,
-                                    const int32_t* cols, const double2* per, const double* uniforms,
-                                    double* w, int32_t* drawn, int32_t* err)
+// One warp per sample, lane i holding the weights of modes i and i + 32; the
+// two sums run over the modes in order on every lane, so a draw is the same
+// whatever the lanes.  (One thread per sample left all but 16 blocks' worth of
+// the chip idle: 18 to 37 us a step for 2000 samples of 16 modes.)
+static_assert(PQ_MAX_DIM <= 64, "two modes a lane");
+
+__global__ void __launch_bounds__(128) sampler_step_kernel(const double2* U, int m, int n, int k,
+                                                           int64_t nsamples, const int32_t* cols,
+                                                           const double2* per,
+                                                           const double* uniforms, int32_t* drawn,
+                                                           int32_t* err)
 {
-    for (int64_t b = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; b < nsamples;
-         b += (int64_t)gridDim.x * blockDim.x) {
-        double* wb = w + b * m;
-        double tot = 0.0;
-        for (int i = 0; i < m; ++i) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; b < nsamples;
+         b += warps) {
+        auto weight = [&](int i) {
             double2 z = make_double2(0.0, 0.0);
+            if (i >= m)
+                return 0.0;
             for (int j = 0; j < k; ++j) {
                 const double2 a = U[(int64_t)i * m + cols[b * n + j]];
                 const double2 pj = (k == 1) ? make_double2(1.0, 0.0) : per[b * k + j];
@@ -83,27 +93,34 @@ __global__ void sampler_step_kernel(const double2* U, int m, int n, int k, int64
                 z.y = __fma_rn(a.x, pj.y, z.y);
                 z.y = __fma_rn(a.y, pj.x, z.y);
             }
-            const double wi = z.x * z.x + z.y * z.y;
-            wb[i] = wi;
-            tot += wi;
-        }
+            return z.x * z.x + z.y * z.y;
+        };
+        const double w0 = weight(lane), w1 = m > 32 ? weight(lane + 32) : 0.0;
+        double tot = 0.0;
+        for (int i = 0; i < m; ++i)
+            tot += __shfl_sync(0xffffffffu, i < 32 ? w0 : w1, i & 31);
         const double thr = uniforms[b * n + (k - 1)] * tot;
         double run = 0.0;
         int pick = -1, last = -1;
         for (int i = 0; i < m; ++i) {
-            if (wb[i] > 0.0)
+            const double wi = __shfl_sync(0xffffffffu, i < 32 ? w0 : w1, i & 31);
+            if (wi > 0.0)
                 last = i;
-            run += wb[i];
-            if (pick < 0 && run > thr)
+            run += wi;
+            if (run > thr) {
                 pick = i;
+                break;
+            }
         }
-        if (pick < 0)
-            pick = last;
-        if (pick < 0) {
-            atomicExch(err, 1);
-            pick = 0;
+        if (lane == 0) {
+            if (pick < 0)
+                pick = last;
+            if (pick < 0) {
+                atomicExch(err, 1);
+                pick = 0;
+            }
+            drawn[b * n + (k - 1)] = pick;
         }
-        drawn[b * n + (k - 1)] = pick;
     }
 }
 
@@ -118,7 +135,7 @@ struct pq_sampler_plan {
     std::vector<int32_t> modes;   // input mode of each photon column
     std::vector<pq_plan*> plans;  // index k = 2 .. n
     double2 *mats_d = nullptr, *per_d = nullptr;
-    double *w_d = nullptr, *u_d = nullptr;
+    double* u_d = nullptr;
     int32_t *cols_d = nullptr, *drawn_d = nullptr, *err_d = nullptr;
     std::vector<int32_t> cols_h, drawn_h;  // host staging of one run
 };
@@ -134,7 +151,6 @@ static void sampler_plan_free(pq_sampler_plan* S)
             pq_plan_destroy(P);
     dev_free(S->mats_d);
     dev_free(S->per_d);
-    dev_free(S->w_d);
     dev_free(S->u_d);
     dev_free(S->cols_d);
     dev_free(S->drawn_d);
@@ -238,7 +254,6 @@ static int sampler_plan_build(int32_t m, const int32_t* input_occ, int64_t nsamp
     if (rc == PQ_OK &&
         (dev_alloc((void**)&S->mats_d, mat_elems * sizeof(double2)) != cudaSuccess ||
          dev_alloc((void**)&S->per_d, Bmax * sizeof(double2)) != cudaSuccess ||
-         dev_alloc((void**)&S->w_d, nsamples * m * sizeof(double)) != cudaSuccess ||
          dev_alloc((void**)&S->u_d, nsamples * n * sizeof(double)) != cudaSuccess ||
          dev_alloc((void**)&S->cols_d, nsamples * n * sizeof(int32_t)) != cudaSuccess ||
          dev_alloc((void**)&S->drawn_d, nsamples * n * sizeof(int32_t)) != cudaSuccess ||
@@ -288,7 +303,7 @@ static int sampler_plan_launch(pq_sampler_plan* S, const pq_c128* U, const int32
         cudaMemsetAsync(S->drawn_d, 0, nsamples * n * sizeof(int32_t), st) != cudaSuccess ||
         cudaMemsetAsync(S->err_d, 0, sizeof(int32_t), st) != cudaSuccess)
         rc = report(PQ_ERR_CUDA, "sampler upload failed");
-    const unsigned sblocks = (unsigned)std::min<int64_t>((nsamples + 127) / 128, 4096);
+    const unsigned sblocks = (unsigned)std::min<int64_t>((nsamples + 3) / 4, 16384);
     for (int k = 1; k <= n && rc == PQ_OK; ++k) {
         if (k >= 2) {
             const int64_t total = nsamples * k * (int64_t)(k - 1) * (k - 1);
@@ -305,7 +320,7 @@ static int sampler_plan_launch(pq_sampler_plan* S, const pq_c128* U, const int32
                 break;
         }
         sampler_step_kernel<<<sblocks, 128, 0, st>>>(reinterpret_cast<const double2*>(U), m, n, k,
-                                                     nsamples, S->cols_d, S->per_d, S->u_d, S->w_d,
+                                                     nsamples, S->cols_d, S->per_d, S->u_d,
                                                      S->drawn_d, S->err_d);
         if (cudaGetLastError() != cudaSuccess)
             rc = report(PQ_ERR_CUDA, "sampling step failed");
