@@ -277,6 +277,15 @@ __device__ __forceinline__ void reweight(const LowWalk& wk, int J, double& wlow,
     wlow = (double)low_weight(wk, J);
 }
 
+// x 2^e: integer work on the exponent where both are normal numbers.
+__device__ __forceinline__ double scale_exp2(double x, int e)
+{
+    const int h = __double2hiint(x), f = (h >> 20) & 0x7ff;
+    if (f == 0 || f == 0x7ff || f + e <= 0 || f + e >= 0x7ff)
+        return scalbn(x, e);
+    return __hiloint2double(h + (int)((uint32_t)e << 20), __double2loint(x));
+}
+
 // Write per = 2^{-(n-1)} * sum, and |per|^2 * norm, the sum being v 2^exp2; a
 // sharded plan writes its unscaled double-double sum instead.
 __device__ __forceinline__ void finalize(const ExecArgs& a, const PermDesc& D, dd2 v, int exp2)
@@ -299,11 +308,8 @@ __device__ __forceinline__ void finalize(const ExecArgs& a, const PermDesc& D, d
         re = 1.0;
         im = 0.0;
     } else {
-        double h, e;
-        fast_two_sum(v.rh, v.rl, h, e);
-        re = scalbn(h + e, exp2 + 1 - D.n);
-        fast_two_sum(v.ih, v.il, h, e);
-        im = scalbn(h + e, exp2 + 1 - D.n);
+        re = scale_exp2(__dadd_rn(v.rh, v.rl), exp2 + 1 - D.n);
+        im = scale_exp2(__dadd_rn(v.ih, v.il), exp2 + 1 - D.n);
     }
     if (a.out_amp)
         a.out_amp[D.out] = make_double2(re, im);
@@ -447,6 +453,11 @@ __device__ __forceinline__ dd2 int_walk(const PermDesc& D, const MetaView& mv, c
         add_term(p, E, w, (s & 1u) != 0, acc);
         ++s;
         if (s == L || (s & 31u) == 0) {
+            if (L <= 32u) {  // the only fold of a short chunk
+                rh = acc.x;
+                ih = acc.y;
+                break;
+            }
             dd_acc(rh, rl, acc.x);
             dd_acc(ih, il, acc.y);
             acc = make_double2(0.0, 0.0);
@@ -459,7 +470,8 @@ __device__ __forceinline__ dd2 int_walk(const PermDesc& D, const MetaView& mv, c
             uint64_t wu;
             const int d = gray_step_at(lo, s + (uint32_t)lane, weighted, up, wu);
             steps = ((uint32_t)(sm.lowrow[d] * ld) << 1) | (up ? 0u : 1u);
-            step_w = (double)wu;
+            if (weighted)
+                step_w = (double)wu;
         }
         const uint32_t step = __shfl_sync(0xffffffffu, steps, q);
         if (weighted)

@@ -704,6 +704,11 @@ __device__ __forceinline__ dd2 haf_walk_int(const HafDesc& D, const HafMeta& mt,
         acc.y = __fma_rn(__ll2double_rn(pv.y), f, acc.y);
         ++s;
         if (s == L || (s & 15u) == 0) {
+            if (L <= 16u) {  // the only fold of a short chunk
+                rh = acc.x;
+                ih = acc.y;
+                break;
+            }
             dd_acc(rh, rl, acc.x);
             dd_acc(ih, il, acc.y);
             acc = make_double2(0.0, 0.0);
@@ -717,7 +722,8 @@ __device__ __forceinline__ dd2 haf_walk_int(const HafDesc& D, const HafMeta& mt,
             uint64_t wu;
             const int d = gray_step_at(lo, s + (uint32_t)lane, weighted, up, wu);
             steps = ((uint32_t)d << 1) | (up ? 0u : 1u);
-            step_w = (double)wu;
+            if (weighted)
+                step_w = (double)wu;
         }
         const uint32_t step = __shfl_sync(0xffffffffu, steps, sq);
         if (weighted)
