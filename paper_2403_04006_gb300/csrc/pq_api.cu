@@ -611,10 +611,9 @@ static void free_plan_device(pq_plan* P)
 // Raise the dynamic shared-memory limit of the plan's forward kernel.
 static cudaError_t forward_prepare(const pq_plan* P)
 {
-    if (P->fwd_nl > 0)
-        return fwd_reg_prepare(P->fwd_nl, P->wpb * fwd_reg_smem_per_warp(P->kmax, P->fwd_ld));
-    if (P->fwd_nl < 0)
-        return fwd_reg_mixed_prepare(P->wpb * fwd_reg_smem_per_warp(P->kmax, P->fwd_ld));
+    if (P->fwd_nl != 0)
+        return fwd_reg_prepare(std::max(P->fwd_nl, 0),
+                               P->wpb * fwd_reg_smem_per_warp(P->kmax, P->fwd_ld));
     return fwd_prepare(P->lmax, P->wpb * fwd_smem_per_warp(P->kmax, P->lmax));
 }
 
@@ -666,7 +665,9 @@ static int schedule_and_upload(pq_plan* P)
         }
         const bool want = P->opts.column_sums == PQ_SUMS_REGISTERS ||
                           (P->opts.column_sums == PQ_SUMS_AUTO && one);
-        P->fwd_nl = (want && P->lmax <= kFwdRegMaxLd) ? (one ? std::max(cls, 4) : -1) : 0;
+        P->fwd_nl = (want && P->lmax <= (one ? kFwdRegMaxLd : kFwdMixedMaxLd))
+                        ? (one ? std::max(cls, 4) : -1)
+                        : 0;
         P->fwd_ld = P->fwd_nl > 0   ? P->fwd_nl
                     : P->fwd_nl < 0 ? fwd_reg_class_of(P->lmax)
                                     : P->lmax;
@@ -677,11 +678,12 @@ static int schedule_and_upload(pq_plan* P)
     if (per_warp > 200 * 1024)
         return fail(PQ_ERR_UNSUPPORTED, "shared memory per warp %d too large", per_warp);
     int wpb = 0, bps = 0;
-    launch_geometry(P->fwd_nl > 0   ? fwd_reg_regs_per_thread(P->fwd_nl)
-                    : P->fwd_nl < 0 ? fwd_reg_mixed_regs_per_thread()
-                                    : fwd_regs_per_thread(P->lmax),
+    const int reg_class = std::max(P->fwd_nl, 0);
+    launch_geometry(P->fwd_nl != 0 ? fwd_reg_regs_per_thread(reg_class)
+                                   : fwd_regs_per_thread(P->lmax),
                     per_warp,
-                    P->opts.warps_per_block > 0 ? P->opts.warps_per_block : 8,
+                    std::min(P->opts.warps_per_block > 0 ? P->opts.warps_per_block : 8,
+                             P->fwd_nl != 0 ? fwd_reg_max_warps(reg_class) : 8),
                     P->opts.blocks_per_sm > 0 ? P->opts.blocks_per_sm : 8, wpb, bps);
     P->wpb = wpb;
     P->blocks = std::max(1, P->num_sms * bps);
@@ -1140,11 +1142,9 @@ static int run_forward_raw(pq_plan* P, const void* src, void* amps, double* prob
             const int64_t tb = P->plain_first[p], te = P->plain_first[p + 1];
             const unsigned grid = (unsigned)((te - tb + P->wpb - 1) / P->wpb);
             cudaError_t e =
-                P->fwd_nl > 0 ? fwd_reg_launch(P->fwd_nl, a, tb, te, P->kmax, P->fwd_ld, grid,
-                                               P->wpb, 0, st)
-                : P->fwd_nl < 0
-                    ? fwd_reg_mixed_launch(a, tb, te, P->kmax, P->fwd_ld, grid, P->wpb, 0, st)
-                    : fwd_launch_plain(P->lmax, a, tb, te, P->kmax, P->wpb, st);
+                P->fwd_nl != 0 ? fwd_reg_launch(std::max(P->fwd_nl, 0), a, tb, te, P->kmax,
+                                                P->fwd_ld, grid, P->wpb, 0, st)
+                               : fwd_launch_plain(P->lmax, a, tb, te, P->kmax, P->wpb, st);
             if (e != cudaSuccess)
                 return fail(PQ_ERR_CUDA, "plain launch failed: %s", cudaGetErrorString(e));
         }
@@ -1152,11 +1152,8 @@ static int run_forward_raw(pq_plan* P, const void* src, void* amps, double* prob
     }
     ExecArgs a = exec_args(P, src, amps, probs, true, partial);
     if (P->fwd_nl != 0) {
-        cudaError_t e =
-            P->fwd_nl > 0 ? fwd_reg_launch(P->fwd_nl, a, 0, a.ntasks, P->kmax, P->fwd_ld,
-                                           (unsigned)P->blocks, P->wpb, 1, st)
-                          : fwd_reg_mixed_launch(a, 0, a.ntasks, P->kmax, P->fwd_ld,
-                                                 (unsigned)P->blocks, P->wpb, 1, st);
+        cudaError_t e = fwd_reg_launch(std::max(P->fwd_nl, 0), a, 0, a.ntasks, P->kmax, P->fwd_ld,
+                                       (unsigned)P->blocks, P->wpb, 1, st);
         if (e != cudaSuccess)
             return fail(PQ_ERR_CUDA, "persistent launch failed: %s", cudaGetErrorString(e));
         return PQ_OK;
