@@ -246,38 +246,37 @@ static void order_digits(ItemPlan& it, const std::vector<int>& low_count)
     it.dtop = top;
 }
 
-// FP64 warp instructions of a cut, the quantity the batched cut minimises:
-// per task, L terms of per_term (plus per_weight times the rate at which the
-// low-digit weight changes), per_high per high digit for the chunk start,
-// per_task_low per low digit and per_task once; per_task_weighted more when
-// the low-digit weight is not constant (a low radix above 2) and
-// per_task_whigh more when a high digit can carry a weight above 1 (a high
-// radix above 2).
+// Warp instructions of a cut, the quantity the batched cut minimises: per task,
+// L terms of per_term, per_high per high digit for the chunk start,
+// per_task_low per low digit and per_task once.  (The backward counts FP64
+// instructions, the pipe that bounds it.)
 struct CutCost {
-    double per_term = 0.0, per_weight = 0.0, per_high = 0.0, per_task = 0.0, per_task_low = 0.0;
-    double per_task_weighted = 0.0, per_task_whigh = 0.0;
+    double per_term = 0.0, per_high = 0.0, per_task = 0.0, per_task_low = 0.0;
 };
 
-// The forward kernel's costs: Gray step 2l, the products 4 each, the fused
-// accumulation 4, the double-double fold 10 every 32 terms; 2 DFMA per weight
-// change; a chunk start 2l + 2 per high digit; per lane and task the chunk's
-// last fold (8), the weighted run's (4), the high-digit weight's double-double
-// product (14, when some high digit has radix > 2; the lane sum itself is
-// integer work) and the staging (2k).
+// The forward kernel's costs: 34 instructions per product, with the column's
+// update (45 for one of the prefix walk, which normalises more often), 45 per
+// term for its step, factor and accumulation; a chunk start's digit and its row
+// of 64-bit multiplies; per task the lane sum, the guard and the finish, and the
+// staging of the base matrix.
 static CutCost forward_cut_cost(const ItemPlan& it)
 {
     int cmax = 1;
     for (int c : it.cmul)
         cmax = std::max(cmax, c);
-    const double products = (cmax == 1) ? (it.l - 2) : (it.l + cmax - 3);
     CutCost cc;
-    cc.per_term = 2.0 * it.l + 4.0 * std::max(products, 0.0) + 4.0 + 10.0 / 32.0;
-    cc.per_weight = 2.0;
-    cc.per_high = 2.0 * it.l + 2.0;
-    cc.per_task = 8.0 + 2.0 * it.k;
-    cc.per_task_weighted = 4.0;
-    cc.per_task_whigh = 14.0;
+    cc.per_term = 45.0 + (cmax == 1 ? 34.0 * it.l : 45.0 * (it.l + cmax - 2));
+    cc.per_high = 30.0 + 12.0 * it.l;
+    cc.per_task = 4500.0 + 40.0 * it.k + 5.0 * it.k * it.l;
     return cc;
+}
+
+// One warp task of the item's cut.
+static double forward_task_cost(const ItemPlan& it)
+{
+    const CutCost cc = forward_cut_cost(it);
+    return (double)it.L * cc.per_term + (double)((int)it.drad.size() - it.J) * cc.per_high +
+           cc.per_task;
 }
 
 // Items that any cut treats alike: the same number of summed rows, column
@@ -368,24 +367,15 @@ static void choose_chunks(ItemPlan& it, int log2_cap, int jmax = kMaxLowDigits,
     }
     if (min_chunks == kWarp) {
         // Batched method: among the neighbouring cuts (one digit longer, up
-        // to two shorter) take the one with the fewest FP64 warp instructions:
+        // to two shorter) take the one with the fewest warp instructions:
         // every lane of a task executes L terms whether or not it has a chunk,
         // and every task pays its chunk start-up and reductions.
         const CutCost k = cc ? *cc : forward_cut_cost(it);
         const int nd = (int)it.drad.size();
-        auto cost_rate = [&](int j, int64_t lj, double wrate, bool whigh) {
-            const double ppt = k.per_term + k.per_weight * wrate;
-            const double ovh = (nd - j) * k.per_high + k.per_task + j * k.per_task_low +
-                               (wrate > 0.0 ? k.per_task_weighted : 0.0) +
-                               (whigh ? k.per_task_whigh : 0.0);
-            const int64_t tasks = (it.T / lj + kWarp - 1) / kWarp;
-            return tasks * ((double)lj * ppt + ovh);
-        };
         auto cost_of = [&](int j, int64_t lj) {
-            bool whigh = false;
-            for (int d = j; d < nd; ++d)
-                whigh = whigh || it.drad[d] > 2;
-            return cost_rate(j, lj, weight_change_rate(it.drad, j), whigh);
+            const double ovh = (nd - j) * k.per_high + k.per_task + j * k.per_task_low;
+            const int64_t tasks = (it.T / lj + kWarp - 1) / kWarp;
+            return tasks * ((double)lj * k.per_term + ovh);
         };
         int bestJ = J;
         int64_t bestL = L;
@@ -435,12 +425,7 @@ static void choose_chunks(ItemPlan& it, int log2_cap, int jmax = kMaxLowDigits,
                     return;
                 if (i == vals.size()) {
                     --budget;
-                    const int a2 = (!vals.empty() && vals[0] == 2) ? cur[0] : 0;
-                    const double wr = (a2 == j) ? 0.0 : std::ldexp(1.0, -a2);
-                    bool whigh = !it.drad.empty() && it.drad.back() > kMaxLowRadix;
-                    for (size_t q = 0; q < vals.size(); ++q)
-                        whigh = whigh || (vals[q] > 2 && cur[q] < cnt[q]);
-                    const double c = cost_rate(j, lj, wr, whigh);
+                    const double c = cost_of(j, lj);
                     if (c < best * 0.999) {
                         best = c;
                         bestc = cur;
@@ -546,12 +531,6 @@ static int explicit_log2_for(const pq_plan* P, const ItemPlan& it)
     return tune_get(it.n);
 }
 
-static int default_log2_for(const pq_plan* P, const ItemPlan& it)
-{
-    const int e = explicit_log2_for(P, it);
-    return e > 0 ? e : 10;
-}
-
 template <typename T>
 static int dev_upload(T** dst, const std::vector<T>& src)
 {
@@ -633,16 +612,6 @@ static int schedule_and_upload(pq_plan* P)
     }
     P->lmax = lmax_needed;
     P->kmax = kmax;
-    // The plain method runs one permanent per launch, so each permanent is cut
-    // finely enough to occupy the whole GPU: at least 4 warps per SM, and for
-    // a large permanent up to two waves of 16 resident warps per SM (chunks of
-    // at least 64 terms, so that each chunk's start stays cheap; eight waves
-    // measured slower at 2.9e7 terms).
-    // The batched method keeps a warp's worth of chunks per permanent and
-    // fills the GPU with many permanents at once.
-    const int64_t plain_min = (int64_t)P->num_sms * 4 * kWarp;
-    const int64_t plain_max = (int64_t)P->num_sms * 16 * 2 * kWarp;
-
     // Where the walk keeps its column sums.  Registers pay when every
     // permanent falls in one column class (m = 24 boson sampling, 4096
     // patterns of 12 photons: 0.92 ms against 1.08 ms in shared memory); a
@@ -688,49 +657,60 @@ static int schedule_and_upload(pq_plan* P)
     P->wpb = wpb;
     P->blocks = std::max(1, P->num_sms * bps);
 
-    if (P->opts.method == PQ_METHOD_PLAIN) {
-        for (ItemPlan& it : P->items) {
-            const int64_t plain_chunks = std::max(plain_min, std::min(plain_max, it.T / 64));
-            choose_chunks(it, default_log2_for(P, it), kMaxLowDigits,
-                          P->opts.chunk_log2 == 0 ? plain_chunks : kWarp);
-        }
-    } else {
-        // The batched method cuts each permanent into at least a warp's worth
-        // of chunks.  A small batch then has too few, too long tasks for the
-        // GPU: the last ones leave SMs idle (4096 permanents of the ragged
-        // recipe took 4.0 ms with chunks of up to 2^10 terms, 1.5 ms with 2^6).
-        // So the chunk cap is lowered, for the whole batch, until the longest
-        // warp task is at most half of a resident warp's average share of the
-        // work; large batches keep their caps (65536 permanents: the longest
-        // task is a quarter of a share).  Chunk lengths that the caller fixed
-        // are kept as they are.
-        const double warps = (double)P->blocks * P->wpb;
+    // Chunk cap.  Long chunks start less often and pay a task's staging and lane
+    // sum less often; short ones give the GPU enough tasks, and tasks of even
+    // size at the end.  So the cap is lowered from 2^10 to 2^0 terms and the
+    // one with the least estimated time is kept: the longest task or the work
+    // over the resident warps (0.85 of them: full speed is reached a little
+    // before all are there), whichever is more, and a quarter of a mean task
+    // for the tail.  Measured, in us, at the caps around the choice: 4096 patterns
+    // of 12 photons 2^5 230, 2^6 199 (chosen); 64 ragged permanents 2^4 73,
+    // 2^3 53, 2^2 44 (chosen); 4096 ragged 2^5 452, 2^6 428 (chosen), 2^7 446; a
+    // single (2, ..., 2) permanent, k = 14, 3691 tasks 185, 1846 tasks 187, 1231
+    // tasks 260, 11072 tasks 241.  The batched method runs the whole batch in one
+    // launch, so its cap is chosen for the batch; the plain method runs one
+    // permanent per launch and chooses it for each.  Chunk lengths that the
+    // caller fixed are kept as they are, and the shards of a permanent, which
+    // must all cut it alike, keep caps of 2^10.
+    {
+        const double warps = 0.85 * (double)P->blocks * P->wpb;
         for (ItemPlan& it : P->items)  // an earlier cut may have reordered the digits
             if (!it.trivial && !std::is_sorted(it.drad.begin(), it.drad.end()))
                 order_digits(it, {});
         ItemGroups groups(P->items);
-        auto cut_all = [&](int gcap) {
-            double total = 0.0, longest = 0.0;
-            for (size_t g = 0; g < groups.first.size(); ++g) {
+        const bool search = P->opts.chunk_log2 == 0 && P->opts.shard_count == 0;
+        // Cut the groups [g0, g1) with the given cap; the launch's estimated time.
+        auto cut = [&](size_t g0, size_t g1, int cap, bool whole_batch, std::vector<Cut>& out) {
+            double total = 0.0, longest = 0.0, tasks = 0.0;
+            for (size_t g = g0; g < g1; ++g) {
                 ItemPlan& it = groups.first[g];
                 const int e = explicit_log2_for(P, it);
-                choose_chunks(it, e > 0 ? e : std::min(10, gcap), kMaxLowDigits, kWarp, true,
-                              nullptr, &groups.cut[g]);
-                const double cost = (double)it.L * fwd_flops_per_term(it) +
-                                    2.0 * (double)((int)it.drow.size() - it.J) * it.l + 2.0 * it.l;
-                total += (double)groups.count[g] * cost *
-                         (double)((it.nchunks + kWarp - 1) / kWarp);
+                choose_chunks(it, e > 0 ? e : cap, kMaxLowDigits, kWarp, true, nullptr, &out[g]);
+                const double cost = forward_task_cost(it);
+                const double nt = (double)((it.nchunks + kWarp - 1) / kWarp) *
+                                  (whole_batch ? (double)groups.count[g] : 1.0);
+                total += nt * cost;
+                tasks += nt;
                 longest = std::max(longest, cost);
             }
-            return total > 0.0 ? longest / (total / warps) : 0.0;
+            return tasks > 0.0 ? std::max(total / warps, longest) + 0.25 * total / tasks : 0.0;
         };
-        int gcap = 30;
-        double ratio = cut_all(gcap);
-        if (P->opts.chunk_log2 == 0 && P->opts.shard_count == 0) {
-            for (int c = 12; c >= 4 && ratio > 0.5; --c) {
-                gcap = c;
-                ratio = cut_all(gcap);
+        auto choose = [&](size_t g0, size_t g1, bool whole_batch) {
+            double best = cut(g0, g1, 10, whole_batch, groups.cut);
+            std::vector<Cut> trial = groups.cut;
+            for (int cap = 9; search && cap >= 0; --cap) {
+                const double t = cut(g0, g1, cap, whole_batch, trial);
+                if (t < 0.99 * best) {
+                    best = t;
+                    std::copy(trial.begin() + g0, trial.begin() + g1, groups.cut.begin() + g0);
+                }
             }
+        };
+        if (P->opts.method == PQ_METHOD_PLAIN) {
+            for (size_t g = 0; g < groups.first.size(); ++g)
+                choose(g, g + 1, false);
+        } else {
+            choose(0, groups.first.size(), true);
         }
         for (int64_t p = 0; p < np; ++p) {
             ItemPlan& it = P->items[p];
