@@ -200,17 +200,13 @@ __device__ __forceinline__ BInt unit_product(const Cols& col, int l, int& E)
     return p;
 }
 
-// Column j of a term with repeated columns: pre, the product of the columns so
-// far, is normalised at odd j and before it is used as an extra factor; at the
-// first column with extras (jf) ex starts as that prefix, and every further
-// extra multiplies it in (n_extra = ecnt[j] of them at column j).
-__device__ __forceinline__ void prefix_column(BInt& pre, int& E, BInt& ex, int& Ex, int j, int jf,
+// The extra factors of a prefix (n_extra = ecnt[j] copies at column j, > 0): at
+// the first column with extras (jf) ex starts as that prefix, and every further
+// extra multiplies it in.
+__device__ __forceinline__ void extra_factors(BInt& pre, int& E, BInt& ex, int& Ex, int j, int jf,
                                               int n_extra)
 {
-    if ((j & 1) || n_extra > 0)
-        bnorm(pre, E);
-    if (n_extra == 0)
-        return;
+    bnorm(pre, E);
     const BLimbs lp = limbs(pre);
     int e = 0;
     if (j == jf) {
@@ -226,6 +222,30 @@ __device__ __forceinline__ void prefix_column(BInt& pre, int& E, BInt& ex, int& 
     }
 }
 
+// Columns j and j + 1 (j + 1 < l, or j alone) of a term with repeated columns:
+// as one pair, p (S_j S_{j+1}), where no extra factor falls between them.
+// has(j): column j has extras.
+template <class Cols, class Has>
+__device__ __forceinline__ void prefix_pair(const Cols& col, const Has& has, BInt& pre, int& E,
+                                            BInt& ex, int& Ex, int j, int l, int jf,
+                                            const int32_t* ecnt)
+{
+    bnorm(pre, E);
+    if (j + 1 < l && !has(j)) {
+        const BInt q = bmul(sum_limbs(col(j)), sum_limbs(col(j + 1)));
+        pre = bmul(limbs(pre), limbs(q));
+    } else {
+        pre = bmul(limbs(pre), sum_limbs(col(j)));
+        if (has(j))
+            extra_factors(pre, E, ex, Ex, j, jf, ecnt[j]);
+        if (j + 1 >= l)
+            return;
+        pre = bmul(limbs(pre), sum_limbs(col(j + 1)));
+    }
+    if (has(j + 1))
+        extra_factors(pre, E, ex, Ex, j + 1, jf, ecnt[j + 1]);
+}
+
 // prod_j S_j^{c_j}; UNIT: no repeated column, else from the prefixes.
 template <int NL, bool UNIT, class Cols>
 __device__ __forceinline__ BInt term_product(const Cols& col, int l, int jf, uint32_t emask,
@@ -237,21 +257,20 @@ __device__ __forceinline__ BInt term_product(const Cols& col, int l, int jf, uin
     BInt pre = bint_plain(col(0)), ex = pre;
     int Ex = 0;
     if constexpr (NL == 0) {
-        prefix_column(pre, E, ex, Ex, 0, jf, ecnt[0]);
+        auto has = [&](int j) { return ecnt[j] > 0; };
+        if (has(0))
+            extra_factors(pre, E, ex, Ex, 0, jf, ecnt[0]);
 #pragma unroll 1
-        for (int j = 1; j < l; ++j) {
-            pre = bmul(limbs(pre), sum_limbs(col(j)));
-            prefix_column(pre, E, ex, Ex, j, jf, ecnt[j]);
-        }
+        for (int j = 1; j < l; j += 2)
+            prefix_pair(col, has, pre, E, ex, Ex, j, l, jf, ecnt);
     } else {
+        auto has = [&](int j) { return ((emask >> j) & 1u) != 0; };
+        if (has(0))
+            extra_factors(pre, E, ex, Ex, 0, jf, ecnt[0]);
 #pragma unroll
-        for (int j = 0; j < NL; ++j) {
-            if (j < l) {
-                if (j > 0)
-                    pre = bmul(limbs(pre), sum_limbs(col(j)));
-                prefix_column(pre, E, ex, Ex, j, jf, ((emask >> j) & 1u) ? ecnt[j] : 0);
-            }
-        }
+        for (int j = 1; j < NL; j += 2)
+            if (j < l)
+                prefix_pair(col, has, pre, E, ex, Ex, j, j + 1 < NL ? l : j + 1, jf, ecnt);
     }
     E += Ex;
     return bmul(limbs(pre), limbs(ex));
