@@ -978,6 +978,7 @@ struct pq_haf_plan {
     int loop = 0;
     int64_t batch = 0, ntasks = 0, ngroups = 0;
     int kmax = 1, wpb = 1, blocks = 1, per_warp = 0;
+    unsigned char* arena = nullptr;  // one allocation: the arrays below
     pqi::HafDesc* desc_d = nullptr;
     int32_t* meta_d = nullptr;
     pqi::Task* tasks_d = nullptr;
@@ -992,12 +993,7 @@ static void haf_plan_free(pq_haf_plan* P)
 {
     if (!P)
         return;
-    dev_free(P->desc_d);
-    dev_free(P->meta_d);
-    dev_free(P->tasks_d);
-    dev_free(P->part_d);
-    dev_free(P->cnt_d);
-    dev_free(P->loopc_d);
+    dev_free(P->arena);
     delete P;
     host_object_freed();
 }
@@ -1218,26 +1214,37 @@ static int haf_plan_build(const int64_t* mat_off, const int32_t* k, const int32_
     P->ngroups = ngroups;
     P->kmax = kmax;
     int rc = PQ_OK;
-    if (dev_alloc((void**)&P->loopc_d, sizeof(double) * std::max<size_t>(loopc.size(), 1)) !=
-            cudaSuccess ||
-        dev_alloc((void**)&P->desc_d, sizeof(HafDesc) * batch) != cudaSuccess ||
-        dev_alloc((void**)&P->meta_d, sizeof(int32_t) * std::max<size_t>(meta.size(), 1)) !=
-            cudaSuccess ||
-        dev_alloc((void**)&P->tasks_d, sizeof(Task) * sorted.size()) != cudaSuccess ||
-        dev_alloc((void**)&P->part_d, sizeof(double) * 4 * std::max<int32_t>(slot, 1)) !=
-            cudaSuccess ||
-        dev_alloc((void**)&P->cnt_d, sizeof(int32_t) * (batch + 1 + ngroups)) != cudaSuccess)
+    // One allocation and one upload: six of the one and four of the other, with
+    // the frees, were most of a one-shot call (300 small hafnians: 400 us, the
+    // kernel 29 of them).  The counters come zeroed with the upload.
+    std::vector<unsigned char> image;
+    auto place = [&](const void* src, size_t bytes) {
+        const size_t at = (image.size() + 255) & ~size_t(255);
+        image.resize(at + std::max<size_t>(bytes, 1));
+        if (src && bytes)
+            std::memcpy(image.data() + at, src, bytes);
+        return at;
+    };
+    const size_t at_desc = place(desc.data(), sizeof(HafDesc) * batch);
+    const size_t at_tasks = place(sorted.data(), sizeof(Task) * sorted.size());
+    const size_t at_loopc = place(loopc.data(), sizeof(double) * loopc.size());
+    const size_t at_meta = place(meta.data(), sizeof(int32_t) * meta.size());
+    const size_t at_cnt = place(nullptr, sizeof(int32_t) * (size_t)(batch + 1 + ngroups));
+    const size_t at_part = (image.size() + 255) & ~size_t(255);
+    const size_t total = at_part + sizeof(double) * 4 * (size_t)std::max<int32_t>(slot, 1);
+    if (dev_alloc((void**)&P->arena, total) != cudaSuccess)
         rc = report(PQ_ERR_NOMEM, "hafnian workspace allocation failed");
     if (rc == PQ_OK &&
-        (cudaMemcpy(P->desc_d, desc.data(), sizeof(HafDesc) * batch, cudaMemcpyHostToDevice) !=
-             cudaSuccess ||
-         (!meta.empty() && cudaMemcpy(P->meta_d, meta.data(), sizeof(int32_t) * meta.size(),
-                                      cudaMemcpyHostToDevice) != cudaSuccess) ||
-         cudaMemcpy(P->tasks_d, sorted.data(), sizeof(Task) * sorted.size(),
-                    cudaMemcpyHostToDevice) != cudaSuccess ||
-         (!loopc.empty() && cudaMemcpy(P->loopc_d, loopc.data(), sizeof(double) * loopc.size(),
-                                       cudaMemcpyHostToDevice) != cudaSuccess)))
+        cudaMemcpy(P->arena, image.data(), image.size(), cudaMemcpyHostToDevice) != cudaSuccess)
         rc = report(PQ_ERR_CUDA, "hafnian upload failed");
+    if (rc == PQ_OK) {
+        P->desc_d = reinterpret_cast<HafDesc*>(P->arena + at_desc);
+        P->tasks_d = reinterpret_cast<Task*>(P->arena + at_tasks);
+        P->loopc_d = reinterpret_cast<double*>(P->arena + at_loopc);
+        P->meta_d = reinterpret_cast<int32_t*>(P->arena + at_meta);
+        P->cnt_d = reinterpret_cast<int32_t*>(P->arena + at_cnt);
+        P->part_d = reinterpret_cast<double*>(P->arena + at_part);
+    }
     if (rc == PQ_OK) {
         P->per_warp = haf_warp_smem_bytes(kmax);
         cudaFuncAttributes fa{};
@@ -1270,13 +1277,16 @@ static int haf_plan_build(const int64_t* mat_off, const int32_t* k, const int32_
     return PQ_OK;
 }
 
-// Execution: clear the counters and launch; allocates nothing, no sync.
+// Execution: clear the counters (unless they are as uploaded) and launch;
+// allocates nothing, no sync.
 static int haf_plan_launch(pq_haf_plan* P, const pq_c128* mats, const pq_c128* gamma,
-                           pq_c128* out, cudaStream_t st)
+                           pq_c128* out, cudaStream_t st, bool reset)
 {
     if (P->batch == 0)
         return PQ_OK;
-    if (cudaMemsetAsync(P->cnt_d, 0, sizeof(int32_t) * (P->batch + 1 + P->ngroups), st) != cudaSuccess)
+    if (reset &&
+        cudaMemsetAsync(P->cnt_d, 0, sizeof(int32_t) * (P->batch + 1 + P->ngroups), st) !=
+            cudaSuccess)
         return report(PQ_ERR_CUDA, "hafnian counter reset failed");
     HafArgs a;
     a.desc = P->desc_d;
@@ -1312,7 +1322,7 @@ static int run_hafnians(const pq_c128* mats, const int64_t* mat_off, const int32
     if (rc != PQ_OK)
         return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    rc = haf_plan_launch(P, mats, gamma, out, st);
+    rc = haf_plan_launch(P, mats, gamma, out, st, false);
     if (cudaStreamSynchronize(st) != cudaSuccess && rc == PQ_OK)
         rc = report(PQ_ERR_CUDA, "hafnian kernel failed");
     haf_plan_free(P);
@@ -1365,7 +1375,7 @@ extern "C" int pq_hafnian_plan_run(pq_haf_plan* plan, const pq_c128* mats, const
     if (plan->batch > 0 && (!mats || !out || (plan->loop && !gamma)))
         return pqi::report(PQ_ERR_ARG, "null argument");
     return pqi::haf_plan_launch(plan, mats, plan->loop ? gamma : nullptr, out,
-                                (cudaStream_t)stream);
+                                (cudaStream_t)stream, true);
 }
 
 extern "C" int pq_hafnian_plan_destroy(pq_haf_plan* plan)
