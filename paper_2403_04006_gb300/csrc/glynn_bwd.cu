@@ -76,7 +76,7 @@ struct BwdSmem {
     double* wh;       // 32
     int32_t* lowrow;  // 16
     int32_t* cm;      // ld
-    int32_t* rowdig;  // kmax: low digit of each row, or -1
+    int32_t* rowdig;  // kmax: low digit of each row, -1 (no digit) or -2 (a high digit)
     int ld;
     __device__ BwdSmem(unsigned char* raw, int kmax, int ld_, int jb, int n2)
     {
@@ -267,9 +267,9 @@ __device__ void bwd_stage(const BwdArgs& a, const PermDesc& D, const MetaView& m
         sm.cm[j] = mv.cmul[j];
     for (int i = lane; i < k; i += kWarp) {
         int dg = -1;
-        for (int d = 0; d < D.J; ++d)
+        for (int d = 0; d < D.ndig; ++d)
             if (mv.drow[d] == i)
-                dg = d;
+                dg = d < D.J ? d : -2;
         sm.rowdig[i] = dg;
     }
     __syncwarp();
@@ -495,8 +495,8 @@ __device__ void bwd_combine(const BwdArgs& a, const Task& t, const PermDesc& D, 
             gx += __ldcg(base_slot + 2 * ((int64_t)q * kl + e));
             gy += __ldcg(base_slot + 2 * ((int64_t)q * kl + e) + 1);
         }
-        gx = scalbn(gx, 1 - D.n);
-        gy = scalbn(gy, 1 - D.n);
+        gx = scale_exp2(gx, 1 - D.n);
+        gy = scale_exp2(gy, 1 - D.n);
         // grad_b = coef * conj(G)
         outg[e] = make_double2(coef.x * gx + coef.y * gy, coef.y * gx - coef.x * gy);
     }
@@ -551,7 +551,7 @@ __global__ void __launch_bounds__(256, 2) glynn_bwd_kernel(BwdArgs a, int64_t t_
     for (;;) {
         int q = 0;
         if (lane == 0)
-            q = atomicAdd(a.counters, 1);
+            q = atomicAdd(a.queue, 1);
         q = __shfl_sync(0xffffffffu, q, 0);
         const int64_t ti = t_begin + q;
         if (ti >= t_end)
@@ -592,8 +592,8 @@ __global__ void __launch_bounds__(256, 2) glynn_bwd_kernel(BwdArgs a, int64_t t_
 // a region that holds the correction rows C (jb x ld x kLS) during the walk
 // and, at the end of a task, the accumulators A' (ld x kLS; above kBwdRegAccLd
 // columns they have a place of their own) and the row multipliers X (kmax x kLS
-// doubles), then the correction sums V (jb x ld), the weights wh (32) and small
-// integer arrays.
+// doubles), then the correction sums V (jb x ld), the lanes' sums W (ld), the
+// weights wh (32) and small integer arrays.
 constexpr int kBwdRegAccLd = 10;
 
 __host__ __device__ inline long bwdr_region_bytes(int kmax, int ld, int jb)
@@ -606,7 +606,7 @@ __host__ __device__ inline long bwdr_region_bytes(int kmax, int ld, int jb)
 
 __host__ __device__ inline int bwdr_warp_smem_bytes(int kmax, int ld, int jb)
 {
-    const long bytes = 16L * (kmax * ld + ld) + bwdr_region_bytes(kmax, ld, jb) + 16L * jb * ld +
+    const long bytes = 16L * (kmax * ld + ld) + bwdr_region_bytes(kmax, ld, jb) + 16L * (jb + 1) * ld +
                        8L * 32 + 4L * (16 + 2 * ld + kmax);
     return (int)((bytes + 15) & ~15L);
 }
@@ -618,6 +618,7 @@ struct BwdRegSmem {
     double2* C;       // jb x ld x kLS    -- region: during the walk
     double* X;        // kmax x kLS       -- region: at the end of a task
     double2* V;       // jb x ld
+    double2* W;       // ld
     double* wh;       // 32
     int32_t* lowrow;  // 16
     int32_t* cm;      // ld
@@ -634,7 +635,8 @@ struct BwdRegSmem {
         X = reinterpret_cast<double*>(A + kLS * ld);
         V = reinterpret_cast<double2*>(reinterpret_cast<unsigned char*>(A) +
                                        bwdr_region_bytes(kmax, ld, jb));
-        wh = reinterpret_cast<double*>(V + jb * ld);
+        W = V + jb * ld;
+        wh = reinterpret_cast<double*>(W + ld);
         lowrow = reinterpret_cast<int32_t*>(wh + 32);
         cm = lowrow + 16;
         cexp = cm + ld;
@@ -994,29 +996,69 @@ __device__ void bwdr_task(const BwdArgs& a, const Task& t, BwdRegSmem& sm, BwdSt
                 if (j < l)
                     sm.A[j * kLS + lane] = A[j];
         }
+        // A row whose count x_i is the same on every lane (no digit, a low digit,
+        // or a high digit that stays put over the task's 32 chunks: most rows)
+        // takes x_i W_j with W_j = sum_q wh_q A_jq, formed once per column; the
+        // others take the sum over the lanes, 64 DFMA per 32 entries, which for
+        // every row was a quarter of a short task's FP64 work.
+        const int g0 = active ? 0 : -1;
+        uint64_t varies = 0;  // rows, at most PQ_MAX_DIM of them
         {
             const double whl = sm.wh[lane];
             double* X = sm.X + lane;
-            for (int i = 0; i < k; ++i)
-                X[i * kLS] = whl * (double)mv.rmul[i];
             int64_t cc = chunk;
             const bool narrow = D.nchunks <= 0x7fffffff;
             for (int d = J; d < ndig; ++d) {
                 const int g = next_digit(cc, mv.drad[d], narrow);
-                const int row = mv.drow[d];
-                X[row * kLS] = whl * (double)(mv.rmul[row] - 2 * g);
-            }
-            const uint64_t gv = gray_value_at(lo, (uint32_t)D.L - 1u);
-            for (int d = 0; d < J; ++d) {
-                const int g = (int)((gv >> (4 * d)) & 15u);
-                const int row = sm.lowrow[d];
-                X[row * kLS] = whl * (double)(mv.rmul[row] - 2 * g);
+                const int first = __shfl_sync(0xffffffffu, g, 0);  // lane 0 has a chunk
+                const int row = mv.drow[d], x = mv.rmul[row] - 2 * g;
+                if (__any_sync(0xffffffffu, g0 == 0 && g != first)) {
+                    varies |= uint64_t(1) << row;
+                    X[row * kLS] = whl * (double)x;
+                } else if (lane == 0) {
+                    X[row * kLS] = (double)x;
+                }
             }
         }
-        __syncwarp();
-        for (int e = lane; e < kl; e += kWarp) {
-            const int i = e / l, j = e - i * l;
+        const uint64_t gv = gray_value_at(lo, (uint32_t)D.L - 1u);
+        for (int i = lane; i < k; i += kWarp) {
             const int dg = sm.rowdig[i];
+            if (dg >= 0)  // rowdig: low digit, -1 none, -2 a high digit (above)
+                sm.X[i * kLS] = (double)(mv.rmul[i] - 2 * (int)((gv >> (4 * dg)) & 15u));
+            else if (dg == -1)
+                sm.X[i * kLS] = (double)mv.rmul[i];
+        }
+        __syncwarp();  // every lane's accumulators are in place
+        for (int j = lane; j < l; j += kWarp) {
+            const double2* Aq = sm.A + j * kLS;
+            double wx = 0.0, wy = 0.0;
+            for (int q = 0; q < 32; ++q) {
+                const double2 av = Aq[q];
+                wx = __fma_rn(sm.wh[q], av.x, wx);
+                wy = __fma_rn(sm.wh[q], av.y, wy);
+            }
+            sm.W[j] = make_double2(wx, wy);
+        }
+        __syncwarp();
+        auto put = [&](int i, int j, double gx, double gy) {
+            const int dg = sm.rowdig[i];
+            if (dg >= 0) {
+                const double2 v = sm.V[dg * NL + j];
+                gx = __dsub_rn(gx, v.x);
+                gy = __dsub_rn(gy, v.y);
+            }
+            const double cj = (double)sm.cm[j];
+            const int x = st.exp2 + sm.cexp[j], e = i * l + j;
+            slot[2 * e] = scale_exp2(cj * gx, x);
+            slot[2 * e + 1] = scale_exp2(cj * gy, x);
+        };
+        const int nv = __popcll(varies);
+        for (int e = lane; e < nv * l; e += kWarp) {
+            const int o = e / l, j = e - o * l;
+            uint64_t left = varies;  // the o-th varying row
+            for (int q = 0; q < o; ++q)
+                left &= left - 1;
+            const int i = __ffsll((long long)left) - 1;
             const double2* Aq = sm.A + j * kLS;
             const double* uq = sm.X + i * kLS;
             double gx = 0.0, gy = 0.0;
@@ -1025,15 +1067,15 @@ __device__ void bwdr_task(const BwdArgs& a, const Task& t, BwdRegSmem& sm, BwdSt
                 gx = __fma_rn(uq[q], av.x, gx);
                 gy = __fma_rn(uq[q], av.y, gy);
             }
-            if (dg >= 0) {
-                const double2 v = sm.V[dg * NL + j];
-                gx = __dsub_rn(gx, v.x);
-                gy = __dsub_rn(gy, v.y);
-            }
-            const double cj = (double)sm.cm[j];
-            const int x = st.exp2 + sm.cexp[j];
-            slot[2 * e] = scalbn(cj * gx, x);
-            slot[2 * e + 1] = scalbn(cj * gy, x);
+            put(i, j, gx, gy);
+        }
+        for (int e = lane; e < kl; e += kWarp) {
+            const int i = e / l, j = e - i * l;
+            if ((varies >> i) & 1u)
+                continue;
+            const double x = sm.X[i * kLS];
+            const double2 w = sm.W[j];
+            put(i, j, __dmul_rn(x, w.x), __dmul_rn(x, w.y));
         }
     }
     bwd_combine(a, t, D, kl, lane);
@@ -1051,6 +1093,12 @@ __global__ void __launch_bounds__(256, NL <= 4 ? 2 : 1) glynn_bwd_reg_kernel(Bwd
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     BwdRegSmem sm(smem_raw + warp * bwdr_warp_smem_bytes(kmax, NL, jb), kmax, NL, jb);
     BwdStaged st;
+    // A batch's classes are launched so that the next may start while this one's
+    // last warps run (programmatic dependent launch): its blocks fill the SMs
+    // as they fall idle.  Every kernel of the chain waits for the one before it
+    // at its own end, so the kernel after the chain follows all of them.
+    if (queue)
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (!queue) {
         const int64_t ti = t_begin + (int64_t)blockIdx.x * (blockDim.x >> 5) + warp;
         if (ti >= t_end)
@@ -1067,7 +1115,7 @@ __global__ void __launch_bounds__(256, NL <= 4 ? 2 : 1) glynn_bwd_reg_kernel(Bwd
     for (;;) {
         int q = 0;
         if (lane == 0)
-            q = atomicAdd(a.counters, 1);
+            q = atomicAdd(a.queue, 1);
         q = __shfl_sync(0xffffffffu, q, 0);
         const int64_t ti = t_begin + q;
         if (ti >= t_end)
@@ -1080,6 +1128,7 @@ __global__ void __launch_bounds__(256, NL <= 4 ? 2 : 1) glynn_bwd_reg_kernel(Bwd
         }
         bwdr_task<NL>(a, a.tasks[ti], sm, st, lane);
     }
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // ---------------------------------------------------------------- scatter
@@ -1249,35 +1298,31 @@ cudaError_t bwdr_prepare(int ld, int smem_bytes)
     return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
 }
 
-template <int NL>
-static void bwdr_launch_nl(const BwdArgs& a, int64_t t_begin, int64_t t_end, int kmax, int jb,
-                           unsigned grid, int wpb, int queue, cudaStream_t st)
+static cudaError_t bwdr_launch(int ld, BwdArgs a, int64_t t_begin, int64_t t_end, int kmax, int jb,
+                               unsigned grid, int wpb, int queue, bool chained, cudaStream_t st)
 {
-    glynn_bwd_reg_kernel<NL><<<grid, 32 * wpb, wpb * bwdr_warp_smem_bytes(kmax, NL, jb), st>>>(
-        a, t_begin, t_end, kmax, jb, queue);
-}
-
-static cudaError_t bwdr_launch(int ld, const BwdArgs& a, int64_t t_begin, int64_t t_end, int kmax,
-                               int jb, unsigned grid, int wpb, int queue, cudaStream_t st)
-{
-    switch (ld) {
-    case 2: bwdr_launch_nl<2>(a, t_begin, t_end, kmax, jb, grid, wpb, queue, st); break;
-    case 4: bwdr_launch_nl<4>(a, t_begin, t_end, kmax, jb, grid, wpb, queue, st); break;
-    case 6: bwdr_launch_nl<6>(a, t_begin, t_end, kmax, jb, grid, wpb, queue, st); break;
-    case 8: bwdr_launch_nl<8>(a, t_begin, t_end, kmax, jb, grid, wpb, queue, st); break;
-    case 10: bwdr_launch_nl<10>(a, t_begin, t_end, kmax, jb, grid, wpb, queue, st); break;
-    case 12: bwdr_launch_nl<12>(a, t_begin, t_end, kmax, jb, grid, wpb, queue, st); break;
-    case 14: bwdr_launch_nl<14>(a, t_begin, t_end, kmax, jb, grid, wpb, queue, st); break;
-    case 16: bwdr_launch_nl<16>(a, t_begin, t_end, kmax, jb, grid, wpb, queue, st); break;
-    default: return cudaErrorInvalidValue;
-    }
-    return cudaGetLastError();
+    const void* f = bwdr_kernel_for(ld);
+    if (!f)
+        return cudaErrorInvalidValue;
+    void* args[] = {&a, &t_begin, &t_end, &kmax, &jb, &queue};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(32 * wpb);
+    cfg.dynamicSmemBytes = (size_t)wpb * bwdr_warp_smem_bytes(kmax, ld, jb);
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelExC(&cfg, f, args);
 }
 
 cudaError_t bwdr_launch_persistent(int ld, const BwdArgs& a, int64_t t_begin, int64_t t_end,
-                                   int kmax, int jb, int blocks, int wpb, cudaStream_t st)
+                                   int kmax, int jb, int blocks, int wpb, bool chained,
+                                   cudaStream_t st)
 {
-    return bwdr_launch(ld, a, t_begin, t_end, kmax, jb, (unsigned)blocks, wpb, 1, st);
+    return bwdr_launch(ld, a, t_begin, t_end, kmax, jb, (unsigned)blocks, wpb, 1, chained, st);
 }
 
 cudaError_t bwdr_launch_plain(int ld, const BwdArgs& a, int64_t t_begin, int64_t t_end, int kmax,
@@ -1285,7 +1330,7 @@ cudaError_t bwdr_launch_plain(int ld, const BwdArgs& a, int64_t t_begin, int64_t
 {
     const int64_t nt = t_end - t_begin;
     return bwdr_launch(ld, a, t_begin, t_end, kmax, jb, (unsigned)((nt + wpb - 1) / wpb), wpb, 0,
-                       st);
+                       false, st);
 }
 
 cudaError_t scatter_grad_batch(const PermDesc* desc, const int32_t* meta, int64_t nperm,

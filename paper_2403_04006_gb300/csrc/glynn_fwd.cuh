@@ -297,15 +297,6 @@ __device__ __forceinline__ void reweight(const LowWalk& wk, int J, double& wlow,
     wlow = (double)low_weight(wk, J);
 }
 
-// x 2^e: integer work on the exponent where both are normal numbers.
-__device__ __forceinline__ double scale_exp2(double x, int e)
-{
-    const int h = __double2hiint(x), f = (h >> 20) & 0x7ff;
-    if (f == 0 || f == 0x7ff || f + e <= 0 || f + e >= 0x7ff)
-        return scalbn(x, e);
-    return __hiloint2double(h + (int)((uint32_t)e << 20), __double2loint(x));
-}
-
 // Write per = 2^{-(n-1)} * sum, and |per|^2 * norm, the sum being v 2^exp2; a
 // sharded plan writes its unscaled double-double sum instead.
 __device__ __forceinline__ void finalize(const ExecArgs& a, const PermDesc& D, dd2 v, int exp2)

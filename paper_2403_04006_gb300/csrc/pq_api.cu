@@ -586,6 +586,13 @@ static void free_plan_device(pq_plan* P)
     }
 }
 
+// The forward's queue head, the permanents' counters, the task groups' and the
+// queue heads of the backward's classes.
+static size_t counter_bytes(const pq_plan* P)
+{
+    return (size_t)(P->nperm + 1 + P->ngroups + kBwdMaxClasses) * sizeof(int32_t);
+}
+
 // Chunks, tasks, descriptors, device upload.
 // Raise the dynamic shared-memory limit of the plan's forward kernel.
 static cudaError_t forward_prepare(const pq_plan* P)
@@ -858,7 +865,7 @@ static int schedule_and_upload(pq_plan* P)
     PQ_ALLOC(&P->partials_d, std::max<size_t>(slot, 1) * 4 * sizeof(double));
     dev_free(P->counters_d);
     P->counters_d = nullptr;
-    PQ_ALLOC(&P->counters_d, (size_t)(np + 1 + P->ngroups) * sizeof(int32_t));
+    PQ_ALLOC(&P->counters_d, counter_bytes(P));
     if (!P->err_d) {
         PQ_ALLOC(&P->err_d, 2 * sizeof(int32_t));
         PQ_CUDA(cudaMemset(P->err_d, 0, 2 * sizeof(int32_t)));
@@ -1112,10 +1119,9 @@ static int run_forward_raw(pq_plan* P, const void* src, void* amps, double* prob
 {
     if (!P->uploaded)
         return fail(PQ_ERR_STATE, "the plan lost its device data in a failed re-planning");
-    PQ_CUDA(cudaMemsetAsync(P->counters_d, 0,
-                            (size_t)(P->nperm + 1 + P->ngroups) * sizeof(int32_t), st));
     if (P->nperm == 0)
         return PQ_OK;
+    PQ_CUDA(cudaMemsetAsync(P->counters_d, 0, counter_bytes(P), st));
     if (P->opts.method == PQ_METHOD_PLAIN) {
         ExecArgs a = exec_args(P, src, amps, probs, false, partial);
         for (int64_t p = 0; p < P->nperm; ++p) {
@@ -1132,8 +1138,9 @@ static int run_forward_raw(pq_plan* P, const void* src, void* amps, double* prob
     }
     ExecArgs a = exec_args(P, src, amps, probs, true, partial);
     if (P->fwd_nl != 0) {
-        cudaError_t e = fwd_reg_launch(std::max(P->fwd_nl, 0), a, 0, a.ntasks, P->kmax, P->fwd_ld,
-                                       (unsigned)P->blocks, P->wpb, 1, st);
+        cudaError_t e =
+            fwd_reg_launch(std::max(P->fwd_nl, 0), a, 0, a.ntasks, P->kmax, P->fwd_ld,
+                           (unsigned)P->blocks, P->wpb, 1, st);
         if (e != cudaSuccess)
             return fail(PQ_ERR_CUDA, "persistent launch failed: %s", cudaGetErrorString(e));
         return PQ_OK;
@@ -1418,6 +1425,8 @@ extern "C" int pq_probe_fp64_peak(int64_t iters, double* flops_per_s, double* ms
 // workspace (column sums, accumulators, prefixes, corrections) is sized for
 // permanents like it rather than for the largest in the batch.
 static const int kBwdClassLd[] = {2, 4, 6, 8, 10, 12, 14, 16, 20, 24, 28, 32, 40};
+static_assert(sizeof(kBwdClassLd) / sizeof(kBwdClassLd[0]) <= kBwdMaxClasses,
+              "a queue head for every class");
 
 static int ensure_backward(pq_plan* P)
 {
@@ -1507,7 +1516,10 @@ static int ensure_backward(pq_plan* P)
         bc.per_term = bwd_instr_per_term(it, C.reg != 0);
         // (in the register walk a high digit is integer work, about a quarter)
         bc.per_high = C.reg ? 0.5 * it.l + 1.0 : 2.0 * it.l;
-        bc.per_task = it.k + 66.0 * it.k * it.l / 32.0;
+        // (in the register walk the lane sums of the columns and of the about
+        // five rows whose digit varies over a task, and the staging)
+        bc.per_task = C.reg ? 130.0 + 10.0 * it.l + 0.2 * it.k * it.l
+                            : it.k + 66.0 * it.k * it.l / 32.0;
         bc.per_task_low = 2.0 * it.l;
         return bc;
     };
@@ -1718,7 +1730,7 @@ static int run_backward(pq_plan* P, const void* src, const pq_c128* grad_out, co
     int rc = ensure_backward(P);
     if (rc != PQ_OK)
         return rc;
-    PQ_CUDA(cudaMemsetAsync(P->counters_d, 0, (size_t)(P->nperm + 1) * sizeof(int32_t), st));
+    PQ_CUDA(cudaMemsetAsync(P->counters_d, 0, counter_bytes(P), st));
     if (P->nperm == 0)
         return PQ_OK;
     BwdArgs a;
@@ -1750,17 +1762,19 @@ static int run_backward(pq_plan* P, const void* src, const pq_c128* grad_out, co
                 return fail(PQ_ERR_CUDA, "plain backward launch failed: %s", cudaGetErrorString(e));
         }
     } else {
-        // one persistent launch per class; the task queue counter restarts at
-        // zero for each (the per-permanent counters were cleared above)
+        // one persistent launch per class, widest first (its tasks are the
+        // longest), each with a queue counter of its own; register kernels are
+        // chained, so that a class fills the SMs that the one before leaves idle
         a.tasks = P->tasks_bwd_batched_d;
-        for (size_t c = 0; c < P->bwd_classes.size(); ++c) {
+        bool chained = false;
+        for (size_t c = P->bwd_classes.size(); c-- > 0;) {
             const BwdClass& C = P->bwd_classes[c];
-            if (c > 0)
-                PQ_CUDA(cudaMemsetAsync(P->counters_d, 0, sizeof(int32_t), st));
+            a.queue = P->counters_d + P->nperm + 1 + P->ngroups + c;
             e = C.reg ? bwdr_launch_persistent(C.ld, a, C.t_begin, C.t_end, C.kmax, C.jb,
-                                               C.blocks, C.wpb, st)
+                                               C.blocks, C.wpb, chained, st)
                       : bwd_launch_persistent(C.ld, a, C.t_begin, C.t_end, C.kmax, C.jb, C.n2,
                                               C.blocks, C.wpb, st);
+            chained = C.reg != 0;
             if (e != cudaSuccess)
                 return fail(PQ_ERR_CUDA, "backward launch failed: %s", cudaGetErrorString(e));
         }

@@ -100,6 +100,15 @@ __device__ __forceinline__ void cfma_acc(double2& acc, double2 p, double2 s)
     }
 }
 
+// x 2^e: integer work on the exponent where both are normal numbers.
+__device__ __forceinline__ double scale_exp2(double x, int e)
+{
+    const int h = __double2hiint(x), f = (h >> 20) & 0x7ff;
+    if (f == 0 || f == 0x7ff || f + e <= 0 || f + e >= 0x7ff)
+        return scalbn(x, e);
+    return __hiloint2double(h + (int)((uint32_t)e << 20), __double2loint(x));
+}
+
 // ---------------------------------------------------------------- binomials
 // Exact C(top, g) for the small tops of low digits (top <= 14).
 __host__ __device__ __forceinline__ uint64_t binom_u64(int top, int g)

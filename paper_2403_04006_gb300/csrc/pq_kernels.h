@@ -99,7 +99,8 @@ struct BwdArgs {
     int64_t* gpart_off;        // per permanent: offset (in complex entries) of slot 0
     double2* grad_local;       // per permanent: oriented k x l gradient (complex)
     int64_t* grad_local_off;   // per permanent: offset of its block
-    int32_t* counters;
+    int32_t* counters;        // [1 + p] finished tasks of p
+    int32_t* queue;           // task queue head of this launch
     int32_t* err;             // device error record (pq_internal.h)
     int64_t nperm;            // permanents (bound of Task::perm)
     int64_t nmeta;            // entries of the metadata pool
@@ -115,12 +116,14 @@ cudaError_t bwd_launch_plain(int lmax, const BwdArgs& a, int64_t t_begin, int64_
 // The register-resident walk (column sums and prefixes in registers) for even
 // product-column bounds up to kBwdRegMaxLd.
 constexpr int kBwdRegMaxLd = 16;
+constexpr int kBwdMaxClasses = 16;  // launches of one batched backward, at most
 bool bwdr_supported(int ld);
 int bwdr_smem_bytes_for(int kmax, int ld, int jb);
 int bwdr_regs_per_thread(int ld);
 cudaError_t bwdr_prepare(int ld, int smem_bytes);
 cudaError_t bwdr_launch_persistent(int ld, const BwdArgs& a, int64_t t_begin, int64_t t_end,
-                                   int kmax, int jb, int blocks, int wpb, cudaStream_t st);
+                                   int kmax, int jb, int blocks, int wpb, bool chained,
+                                   cudaStream_t st);
 cudaError_t bwdr_launch_plain(int ld, const BwdArgs& a, int64_t t_begin, int64_t t_end, int kmax,
                               int jb, int wpb, cudaStream_t st);
 
