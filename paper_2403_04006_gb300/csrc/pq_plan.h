@@ -93,6 +93,7 @@ struct pq_plan {
     // (a row of class NL holds NL columns, at least 4, so it can be wider
     // than lmax)
     int fwd_ld = 0;
+    bool direct = false;    // every permanent is at most one task
     bool uploaded = false;  // device data matches the host schedule (a failed re-plan clears it)
     std::vector<pqi::PermDesc> desc_bwd_h;
     std::vector<pqi::Task> tasks_bwd_plain_h, tasks_bwd_batched_h;
