@@ -102,8 +102,9 @@ typedef struct {
 /* Where a lane keeps its column sums in the forward walk. */
 #define PQ_SUMS_AUTO 0      /* the planner's choice (default)                            */
 #define PQ_SUMS_SHARED 1    /* shared memory, lane-major: any product side               */
-#define PQ_SUMS_REGISTERS 2 /* registers: product sides of at most 20 columns (the plan
-                               falls back to shared memory for wider ones)              */
+#define PQ_SUMS_REGISTERS 2 /* registers: product sides of at most 32 columns in a batch of
+                               one column class, 20 in a mixed one (the plan falls back
+                               to shared memory for wider ones)                         */
 
 /* Plan options; zero-initialise and set what you need. */
 typedef struct {
@@ -146,7 +147,9 @@ int pq_plan_destroy(pq_plan* plan);
 
 /* Per(A_b) for every item of the batch (Eq. (per_def) with the multiplicities
  * of Sec. 4.2), evaluated by the multiplicity-extended BB/FG formula over a
- * mixed-radix Gray code in FP64 with double-double accumulation.
+ * mixed-radix Gray code, the products in 64-bit block integers (FP64 where an
+ * entry is not finite or a column's sums can overflow), accumulated in
+ * double-double.
  * b: device descriptor; out: device, batch entries.  plan: made by
  * pq_plan_create for the same sizes, or NULL, in which case the call copies
  * the sizes to the host, plans, runs the batched method and synchronises
@@ -436,22 +439,19 @@ int pq_plan_device_error(pq_plan* plan, int32_t* code, int64_t* task, int32_t cl
 /* Statistics of a plan, host memory: number of permanents, total Gray-code
  * terms, algorithmic FP64 flops of one forward execution (FMA = 2; the count
  * of a straightforward Glynn evaluation: 2l + 6(n-1) + 2 per term, +2 for a
- * non-unit weight), FP64 instructions the forward kernel needs for its terms
- * (Gray step, products, fused accumulation, weights, double-double fold;
- * each DADD, DMUL or DFMA counts one), number of warp tasks and of kernel
- * launches one execution makes.  flops_backward is the algorithmic count of
- * a backward that forms the k x l rank-1 update of every term (2l + 6(n-1)
- * + 2 + 18l + 8kl); the kernel's correction scheme avoids that update, so
- * fp64_instr_backward (per term: column and correction updates, prefix and
- * suffix products, accumulation; per chunk: the start from the high digits;
- * per task: the lane contraction) is the count to compare with the FP64
- * pipe.  fp64_instr_backward is filled in by the first backward call (zero
- * before it), which also settles launches_backward.
- * fp64_instr_forward_executed adds what the forward executes besides the
- * terms, counted per lane: the lanes of a task without a chunk (they walk
- * with the others), each chunk's start from its high digits, the fold and
- * scaling of each chunk's sum, the per-task lane reduction and the
- * per-permanent combination of task partials. */
+ * non-unit weight), number of warp tasks and of kernel launches one execution
+ * makes.  The kernels form column sums and products in integers, so the FP64
+ * instructions they issue are far fewer (each DADD, DMUL, DFMA or conversion
+ * counts one): fp64_instr_forward is 4 per term and the double-double folds;
+ * fp64_instr_forward_executed counts them per lane, the lanes of a task
+ * without a chunk included.  flops_backward is the algorithmic count of a
+ * backward that forms the k x l rank-1 update of every term (2l + 6(n-1) + 2 +
+ * 18l + 8kl); the kernel's correction scheme avoids that update, and
+ * fp64_instr_backward (per term the accumulations and corrections, per task the
+ * lane contraction; for product sides of more than 16 columns the products
+ * too) is the count to compare with the FP64 pipe.  It is filled in by the
+ * first backward call (zero before it), which also settles
+ * launches_backward. */
 typedef struct {
     int64_t permanents;
     int64_t terms;

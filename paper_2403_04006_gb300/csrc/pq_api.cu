@@ -201,18 +201,6 @@ static int build_item(const int32_t* r, const int32_t* c, int k0, int l0, int64_
     return PQ_OK;
 }
 
-// Share of the Gray steps of a chunk (the lowest j digits, ascending radix)
-// after which the low-digit weight prod_d C(top_d, g_d) changes: only digits
-// of radix > 2 change it, and the a leading radix-2 digits take all but
-// 2^-a of the steps.  Zero when every low digit has radix 2.
-static double weight_change_rate(const std::vector<int32_t>& drad, int j)
-{
-    int a = 0;
-    while (a < j && drad[a] == 2)
-        ++a;
-    return a == j ? 0.0 : std::ldexp(1.0, -a);
-}
-
 // Put the digits of the given low multiset first (ascending radix, ties in
 // row order), then the others in the same order.  low_count[v]: how many
 // digits of radix v go low.  The walk takes any digits as its low ones: the
@@ -477,37 +465,29 @@ static double fwd_flops_per_term(const ItemPlan& it)
     return 2.0 * it.l + 6.0 * (it.n - 1) + 2.0 + (it.weighted ? 2.0 : 0.0);
 }
 
-// FP64 instructions of one term in glynn_fwd.cu: Gray step 2l; products of
-// P(l) and the extra prefixes, 4 each; fused accumulation 4; 2 DFMA per
-// change of the low-digit weight; the double-double fold, 10 every 32 terms.
-static double fwd_instr_per_term(const ItemPlan& it)
-{
-    if (it.n == 1)
-        return 2.0;
-    int cmax = 1;
-    for (int c : it.cmul)
-        cmax = std::max(cmax, c);
-    const double products = (cmax == 1) ? (it.l - 2) : (it.l + cmax - 3);
-    return 2.0 * it.l + 4.0 * products + 4.0 + 2.0 * weight_change_rate(it.drad, it.J) +
-           10.0 / 32.0;
-}
+// FP64 instructions of one forward term: two conversions and two fused adds
+// (the column sums and products are integers), and the double-double fold, 12
+// every 32 terms.
+constexpr double kFwdInstrPerTerm = 4.0 + 12.0 / 32.0;
 
 static double bwd_flops_per_term(const ItemPlan& it)
 {
     return fwd_flops_per_term(it) + 18.0 * it.l + 8.0 * it.k * it.l;
 }
 
-// FP64 instructions of one backward term in glynn_bwd.cu: column-sum and
-// correction updates 4l; prefixes 4(l - 2); per middle column the fused
-// accumulation of prefix times weighted suffix and the suffix update, 8; the
-// end columns and the weighted suffix's start 6; per repeated column its
-// powers, the scaled derivative and one more product, 4(c - 1) + 6.
+// FP64 instructions of one backward term in glynn_bwd.cu.  Register walk (at
+// most 16 columns): products in integers, the accumulations 4l and the
+// corrections 2l.  Shared-memory walk: column-sum and correction updates 4l;
+// prefixes 4(l - 2); per middle column the fused accumulation of prefix times
+// weighted suffix and the suffix update, 8; the end columns and the weighted
+// suffix's start 6; per repeated column its powers, the scaled derivative and
+// one more product, 4(c - 1) + 6.
 static double bwd_instr_per_term(const ItemPlan& it, bool reg)
 {
     if (it.n == 1)
         return 2.0;
     const int l = it.l;
-    if (reg)  // products in integers: the accumulations 4l, the corrections 2l
+    if (reg)
         return 6.0 * l;
     double rep = 0.0;
     for (int c : it.cmul)
@@ -620,13 +600,12 @@ static int schedule_and_upload(pq_plan* P)
     P->lmax = lmax_needed;
     P->kmax = kmax;
     // Where the walk keeps its column sums.  Registers pay when every
-    // permanent falls in one column class (m = 24 boson sampling, 4096
-    // patterns of 12 photons: 0.92 ms against 1.08 ms in shared memory); a
-    // batch that mixes classes runs one instantiation per class in one kernel,
-    // whose register count is that of the widest (226: 8 warps per SM), and
-    // was slower than shared memory (ragged batch: 24.6 ms against 22.7 ms),
-    // so the planner takes registers for a single class only, and a caller
-    // may ask for them (PQ_SUMS_REGISTERS) or for shared memory.
+    // permanent falls in one column class (4096 patterns of 12 photons in
+    // m = 24: 194 us; one n = 30 permanent: 35.2 ms, 49.1 ms in shared
+    // memory).  A batch that mixes classes would run one instantiation per
+    // class in one kernel, with the registers of the widest and different code
+    // on the warps of one SM, so the planner takes shared memory there, and a
+    // caller may ask for either (PQ_SUMS_REGISTERS, PQ_SUMS_SHARED).
     {
         int cls = 0;
         bool one = true;
@@ -807,22 +786,11 @@ static int schedule_and_upload(pq_plan* P)
             const int64_t tt = (c1 - q0 * kWarp) * it.L;
             terms += tt;
             flops_f += (double)tt * fpt;
-            instr_f += (double)tt * fwd_instr_per_term(it);
+            instr_f += (double)tt * kFwdInstrPerTerm;
             flops_b += (double)tt * bwd_flops_per_term(it);
-            // per task, every lane: L terms, the chunk start ((ndig - J) row
-            // updates of 2l), the chunk's last folds (8, 12 when weighted) and
-            // the high-digit weight's product (14, when a high radix is above
-            // 2); the lane sum is integer work.  Per permanent with several
-            // tasks, the partials' double-double sum (14 per 32 tasks and lane)
-            bool whigh = false;
-            for (size_t d = it.J; d < it.drad.size(); ++d)
-                whigh = whigh || it.drad[d] > 2;
-            const double lane = (double)it.L * fwd_instr_per_term(it) +
-                                2.0 * it.l * (double)((int)it.drow.size() - it.J) +
-                                (it.weighted ? 12.0 : 8.0) + (whigh ? 14.0 : 0.0);
-            instr_fx += (double)nt * 32.0 * lane;
-            if (nt > 1)
-                instr_fx += 32.0 * 14.0 * (double)((nt + kWarp - 1) / kWarp);
+            // per task every lane walks L terms, with a chunk or without, and adds
+            // its folds; the lane sum and the partials' sums are integer work
+            instr_fx += (double)nt * 32.0 * ((double)it.L * kFwdInstrPerTerm + 4.0);
         }
         if (slot < 0)
             return fail(PQ_ERR_UNSUPPORTED, "too many tasks");
@@ -2054,11 +2022,9 @@ extern "C" int pq_autotune(pq_plan* P, const pq_batch* b, const pq_c128* U, void
         }
     }
     // Where the walk keeps its column sums.  For a batch of one column class
-    // the planner takes registers, which measured from 10% slower (4096
-    // collision-free permanents of n = 16) to 11% faster (m = 24 boson
-    // sampling, 4096 patterns) than shared memory, with its chunking: time
-    // the whole plan both ways and keep shared memory only if it is at least
-    // 1% faster.  The choice is the plan's (its options), not the process's.
+    // the planner takes registers; time the whole plan both ways, with its
+    // chunking, and keep shared memory only if it is at least 1% faster.  The
+    // choice is the plan's (its options), not the process's.
     const int32_t saved_sums = P->opts.column_sums;
     if (rc == PQ_OK && P->opts.column_sums == PQ_SUMS_AUTO && P->fwd_nl > 0) {
         float t_reg = 0.0f, t_sh = 0.0f;
