@@ -38,7 +38,8 @@
 // takes one conversion and one fused add per term and component.  All sums are
 // taken modulo 2^64: only q and l themselves have to stay in range.  In FP64
 // the walk was bound by the FP64 pipe (85 to 90% active): (2, ..., 2) at
-// N = 36 took 19.1 ms (hafnian), N = 28 with loops 1.68 ms.  A matrix
+// N = 36 took 19.1 ms (hafnian), N = 28 with loops 1.68 ms; in integers, bound
+// by the wide multiplies and their adds, 4.87 ms and 0.34 ms.  A matrix
 // without a scale (non-finite or subnormal entries, a bound beyond FP64) is
 // walked in FP64.
 #include <cuda_runtime.h>
@@ -505,8 +506,7 @@ __device__ __forceinline__ BInt haf_power(longlong2 q, int n, int& E)
     E = Ex;
 #pragma unroll 1
     for (int bit = 30 - __clz(n); bit >= 0; --bit) {
-        const BLimbs lh = limbs(h);
-        h = bmul(lh, lh);
+        h = bsqr(limbs(h));
         E *= 2;
         bnorm(h, E);
         if ((n >> bit) & 1) {
@@ -555,7 +555,7 @@ __device__ __forceinline__ BInt haf_loop_poly(longlong2 q, longlong2 l, int P, b
         int Eq = 0;
         bnorm(qw, Eq);
         const BLimbs ll = limbs(lw);
-        BInt sw = bmul(ll, ll);
+        BInt sw = bsqr(ll);
         int Es = 0;
         bnorm(sw, Es);
         constexpr int kNone = -(1 << 18), kLeast = -(1 << 17);  // exponent of an exact zero
@@ -564,7 +564,7 @@ __device__ __forceinline__ BInt haf_loop_poly(longlong2 q, longlong2 l, int P, b
         const BLimbs lq = limbs(qw), ls = limbs(sw);
         if (P > 0) {
             int n0 = 0, n1 = 0, n2 = 0;
-            BInt v0 = bmul(lq, lq), v1 = bmul(lq, ls), v2 = bmul(ls, ls);
+            BInt v0 = bsqr(lq), v1 = bmul(lq, ls), v2 = bsqr(ls);
             bnorm(v0, n0);
             bnorm(v1, n1);
             bnorm(v2, n2);

@@ -176,6 +176,22 @@ __device__ __forceinline__ BInt bmul(const BLimbs& p, const BLimbs& s)
     return r;
 }
 
+// (p p) >> 64: the bits of bmul(p, p), from 7 wide multiplies instead of 12.
+__device__ __forceinline__ BInt bsqr(const BLimbs& p)
+{
+    const int64_t mr = mulw(p.a, p.b) - mulw(p.c, p.d);
+    const int64_t mi = mulw(p.a, p.d) + mulw(p.b, p.c);
+    const int64_t m = mulw(p.a, p.c);
+    const int64_t hr = mulw(p.a, p.a) - mulw(p.c, p.c) + (int64_t)(int)(mr >> 31);
+    const int64_t hi = m + m + (int64_t)(int)(mi >> 31);
+    BInt r;
+    r.rh = (int)(hr >> 32);
+    r.rl = (uint32_t)hr;
+    r.ih = (int)(hi >> 32);
+    r.il = (uint32_t)hi;
+    return r;
+}
+
 // Shift left until the larger high word has its top bit at position 29; the
 // shift (at most 30) is added to E.
 __device__ __forceinline__ void bnorm(BInt& p, int& E)
