@@ -1015,6 +1015,7 @@ struct pq_haf_plan {
     int64_t batch = 0, ntasks = 0, ngroups = 0;
     int kmax = 1, wpb = 1, blocks = 1, per_warp = 0;
     unsigned char* arena = nullptr;  // one allocation: the arrays below
+    std::vector<unsigned char> image;  // its host copy, until the upload has been waited for
     pqi::HafDesc* desc_d = nullptr;
     int32_t* meta_d = nullptr;
     pqi::Task* tasks_d = nullptr;
@@ -1034,10 +1035,12 @@ static void haf_plan_free(pq_haf_plan* P)
     host_object_freed();
 }
 
-// Plan: digits, chunks, tasks (longest first), loop-polynomial factors;
-// uploads them and raises the kernel's shared-memory limit.
+// Plan: digits, chunks, tasks (longest first), loop-polynomial factors; uploads
+// them on the stream (the caller waits for it before it drops P->image) and
+// raises the kernel's shared-memory limit.
 static int haf_plan_build(const int64_t* mat_off, const int32_t* k, const int32_t* rep,
-                          const int64_t* rep_off, int64_t batch, bool loop, pq_haf_plan** out)
+                          const int64_t* rep_off, int64_t batch, bool loop, cudaStream_t st,
+                          pq_haf_plan** out)
 {
     *out = nullptr;
     if (batch < 0 || (batch > 0 && (!mat_off || !k || !rep || !rep_off)))
@@ -1252,8 +1255,11 @@ static int haf_plan_build(const int64_t* mat_off, const int32_t* k, const int32_
     int rc = PQ_OK;
     // One allocation and one upload: six of the one and four of the other, with
     // the frees, were most of a one-shot call (300 small hafnians: 400 us, the
-    // kernel 29 of them).  The counters come zeroed with the upload.
-    std::vector<unsigned char> image;
+    // kernel 29 of them).  The counters come zeroed with the upload.  It is made
+    // on the stream that the kernel runs on: a plain cudaMemcpy from pageable
+    // memory may return before the data has arrived, and streams that do not wait
+    // for the default one would read what the memory held before.
+    std::vector<unsigned char>& image = P->image;
     auto place = [&](const void* src, size_t bytes) {
         const size_t at = (image.size() + 255) & ~size_t(255);
         image.resize(at + std::max<size_t>(bytes, 1));
@@ -1271,7 +1277,8 @@ static int haf_plan_build(const int64_t* mat_off, const int32_t* k, const int32_
     if (dev_alloc((void**)&P->arena, total) != cudaSuccess)
         rc = report(PQ_ERR_NOMEM, "hafnian workspace allocation failed");
     if (rc == PQ_OK &&
-        cudaMemcpy(P->arena, image.data(), image.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+        cudaMemcpyAsync(P->arena, image.data(), image.size(), cudaMemcpyHostToDevice, st) !=
+            cudaSuccess)
         rc = report(PQ_ERR_CUDA, "hafnian upload failed");
     if (rc == PQ_OK) {
         P->desc_d = reinterpret_cast<HafDesc*>(P->arena + at_desc);
@@ -1306,6 +1313,7 @@ static int haf_plan_build(const int64_t* mat_off, const int32_t* k, const int32_
             rc = report(PQ_ERR_CUDA, "hafnian kernel attribute setup failed");
     }
     if (rc != PQ_OK) {
+        cudaStreamSynchronize(st);  // the upload may be in flight
         haf_plan_free(P);
         return rc;
     }
@@ -1353,11 +1361,11 @@ static int run_hafnians(const pq_c128* mats, const int64_t* mat_off, const int32
 {
     if (batch > 0 && (!mats || !out))
         return report(PQ_ERR_ARG, "null argument");
+    cudaStream_t st = (cudaStream_t)stream;
     pq_haf_plan* P = nullptr;
-    int rc = haf_plan_build(mat_off, k, rep, rep_off, batch, gamma != nullptr, &P);
+    int rc = haf_plan_build(mat_off, k, rep, rep_off, batch, gamma != nullptr, st, &P);
     if (rc != PQ_OK)
         return rc;
-    cudaStream_t st = (cudaStream_t)stream;
     rc = haf_plan_launch(P, mats, gamma, out, st, false);
     if (cudaStreamSynchronize(st) != cudaSuccess && rc == PQ_OK)
         rc = report(PQ_ERR_CUDA, "hafnian kernel failed");
@@ -1400,7 +1408,17 @@ extern "C" int pq_hafnian_plan_create(const int64_t* mat_off, const int32_t* k, 
 {
     if (!out)
         return pqi::report(PQ_ERR_ARG, "null output");
-    return pqi::haf_plan_build(mat_off, k, rep, rep_off, batch, loop != 0, out);
+    int rc = pqi::haf_plan_build(mat_off, k, rep, rep_off, batch, loop != 0, nullptr, out);
+    // a run may come on any stream: the upload is complete when the plan exists
+    if (rc == PQ_OK && (*out)->arena) {
+        if (cudaStreamSynchronize(nullptr) != cudaSuccess) {
+            pqi::haf_plan_free(*out);
+            *out = nullptr;
+            return pqi::report(PQ_ERR_CUDA, "hafnian upload failed");
+        }
+        std::vector<unsigned char>().swap((*out)->image);
+    }
+    return rc;
 }
 
 extern "C" int pq_hafnian_plan_run(pq_haf_plan* plan, const pq_c128* mats, const pq_c128* gamma,
