@@ -181,8 +181,11 @@ static int lossy_plan_build(int32_t m, const int32_t* input_occ, const int32_t* 
          dev_alloc((void**)&L->pbig, sizeof(double) * L->NB) != cudaSuccess ||
          dev_alloc((void**)&L->first_d, sizeof(int64_t) * (B + 1)) != cudaSuccess))
         rc = report(PQ_ERR_NOMEM, "lossy workspace allocation failed");
-    if (rc == PQ_OK && cudaMemcpy(L->first_d, first.data(), sizeof(int64_t) * (B + 1),
-                                  cudaMemcpyHostToDevice) != cudaSuccess)
+    // (a copy from pageable memory may return before the device holds the data,
+    // and a run may come on any stream)
+    if (rc == PQ_OK && (cudaMemcpy(L->first_d, first.data(), sizeof(int64_t) * (B + 1),
+                                   cudaMemcpyHostToDevice) != cudaSuccess ||
+                        cudaStreamSynchronize(nullptr) != cudaSuccess))
         rc = report(PQ_ERR_CUDA, "pattern offsets upload failed");
     if (rc != PQ_OK) {
         lossy_plan_free(L);

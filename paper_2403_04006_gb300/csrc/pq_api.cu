@@ -511,6 +511,7 @@ static int explicit_log2_for(const pq_plan* P, const ItemPlan& it)
     return tune_get(it.n);
 }
 
+// Copies on the default stream (the caller waits for them once, uploads_done).
 template <typename T>
 static int dev_upload(T** dst, const std::vector<T>& src)
 {
@@ -528,6 +529,15 @@ static int dev_upload(T** dst, const std::vector<T>& src)
         if (e != cudaSuccess)
             return fail(PQ_ERR_CUDA, "cudaMemcpy failed: %s", cudaGetErrorString(e));
     }
+    return PQ_OK;
+}
+
+// A copy from pageable memory may return, and a memset does, before the device
+// holds the data, and streams that do not wait for the default one would read
+// what was there before: a plan is ready for any stream after this.
+static int uploads_done()
+{
+    PQ_CUDA(cudaStreamSynchronize(nullptr));
     return PQ_OK;
 }
 
@@ -844,6 +854,8 @@ static int schedule_and_upload(pq_plan* P)
     cudaError_t e = forward_prepare(P);
     if (e != cudaSuccess)
         return fail(PQ_ERR_CUDA, "kernel attribute setup failed: %s", cudaGetErrorString(e));
+    if ((rc = uploads_done()) != PQ_OK)
+        return rc;
     P->uploaded = true;
     return PQ_OK;
 }
@@ -1186,6 +1198,11 @@ static int read_device_error(pq_plan* P, int32_t* code, int64_t* task, bool clea
     PQ_CUDA(cudaMemcpy(rec, P->err_d, sizeof(rec), cudaMemcpyDeviceToHost));
     if (clear && (rec[0] || rec[1]))
         PQ_CUDA(cudaMemset(P->err_d, 0, sizeof(rec)));
+    if (clear) {
+        const int rc = uploads_done();
+        if (rc != PQ_OK)
+            return rc;
+    }
     *code = rec[0];
     *task = rec[1];
     return PQ_OK;
@@ -1695,6 +1712,8 @@ static int ensure_backward(pq_plan* P)
     cudaError_t e = bwd_prepare(P->lmax, max_smem);
     if (e != cudaSuccess)
         return fail(PQ_ERR_CUDA, "backward attribute setup failed: %s", cudaGetErrorString(e));
+    if ((rc = uploads_done()) != PQ_OK)
+        return rc;
     P->stats.launches_backward = (P->opts.method == PQ_METHOD_PLAIN)
                                      ? np + 1
                                      : (int64_t)P->bwd_classes.size() + 1;

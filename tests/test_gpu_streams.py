@@ -60,3 +60,41 @@ def test_hafnian_plan_run_at_once(dev, loop):
         return plan.run(x[0][0], x[1] if loop else None)
 
     both(dev, call, [hafnians(s, dev) for s in range(ROUNDS)])
+
+
+def batch(seed, dev):
+    rng = np.random.default_rng(seed)
+    items = []
+    for _ in range(int(rng.integers(1, 40))):
+        n = int(rng.integers(2, 10))
+        A = rng.standard_normal((n, n)) + 1j * rng.standard_normal((n, n))
+        items.append((A, [1] * n, [1] * n) if n % 2 else
+                     (A[:n // 2, :n // 2], [2] * (n // 2), [2] * (n // 2)))
+    pb = W.pack_batch(items)
+    go = rng.standard_normal(len(items)) + 1j * rng.standard_normal(len(items))
+    return pb, api.DeviceBatch(pb, dev), torch.from_numpy(go).to(dev)
+
+
+@pytest.mark.parametrize("method", ["batched", "plain"])
+def test_permanents_planned_and_run_at_once(dev, method):
+    """The forward, and the first backward call, which plans the backward."""
+    def call(x):
+        pb, db, go = x
+        plan = api.Plan.for_batch(pb, method=method)
+        per = api.permanent_batched(db, plan)
+        return torch.cat([per, api.permanent_backward(db, go, plan)])
+
+    both(dev, call, [batch(s, dev) for s in range(ROUNDS)])
+
+
+def test_lossy_planned_and_run_at_once(dev):
+    def inputs(seed):
+        rng = np.random.default_rng(seed)
+        m = 3 + seed % 4
+        s = np.array([1, 1, 1] + [0] * (m - 3), dtype=np.int32)
+        t = np.concatenate([W.compositions(q, m) for q in range(4)])
+        dev_of = lambda x: torch.from_numpy(np.ascontiguousarray(x)).to(dev)
+        return (m, s, t), [dev_of(x) for x in (W.haar_unitary(m, rng), rng.uniform(0.5, 0.9, m),
+                                               W.haar_unitary(m, rng))]
+
+    both(dev, lambda x: api.LossyPlan(*x[0]).run(*x[1]), [inputs(s) for s in range(ROUNDS)])
