@@ -66,7 +66,10 @@ __host__ __device__ __forceinline__ uint64_t bint_bits(double x)
 // column whose units (times multiplicity) add up to u is scaled by
 // 2^bint_scale(hmax, u), which keeps its sums below 2^kSumBits (1 - 2^-21).
 // A column of subnormal entries (hmax < 2^20) is added up exactly, in units of
-// 2^-1074, so that it loses no bits (bint_scale_subnormal).
+// 2^-1074, so that it loses no bits (bint_scale_subnormal: at most 58 bits, and
+// one to spare, since a sum that is exactly the bound would reach 2^kSumBits
+// less a few units, where the high word of a negative number is -2^30 already
+// and bnorm's shift would be negative).
 __host__ __device__ __forceinline__ uint32_t bint_mag(double re, double im)
 {
     const uint32_t x = (uint32_t)(bint_bits(re) >> 32) & 0x7fffffffu;
@@ -106,7 +109,7 @@ __host__ __device__ __forceinline__ uint64_t bint_mag_subnormal(double re, doubl
 
 __host__ __device__ __forceinline__ int bint_scale_subnormal(uint64_t sum)
 {
-    return kSumBits + 1074 - bint_width(sum);
+    return kSumBits + 1073 - bint_width(sum);
 }
 
 // round(x 2^e) as an integer, ties away from zero; |x| 2^e < 2^63.
