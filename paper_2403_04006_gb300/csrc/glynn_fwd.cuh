@@ -24,7 +24,10 @@
 //     accumulator with TwoSum.
 // A base matrix with a non-finite entry, or a column whose bound overflows, has
 // no such scale: its tasks walk in FP64 (fp64_walk), so that infinities and
-// NaNs propagate as FP64 arithmetic gives them.
+// NaNs propagate as FP64 arithmetic gives them.  Matrices whose columns all lie
+// near the real or imaginary axis have a unit for each part (other_walk), so that
+// the small part keeps its bits: 16384 ragged permanents 2.03 ms (1.52 with parts
+// of like size, 5.34 for the FP64 walk), one n = 24 permanent 0.91 (0.60, 2.64).
 // A warp task is up to 32 chunks of one permanent (one per lane).  The lanes'
 // sums are added exactly, in 128-bit integers (pq_fixsum.cuh), and the tasks
 // of one permanent in task order by the warp that finishes last, so results
@@ -81,14 +84,20 @@ struct WarpSmem {
         ecnt = lowrow + 16;
         cexp = ecnt + ld;
     }
+    // of a walk with its column sums elsewhere
+    __device__ WarpSmem(longlong2* M_, longlong2* base_, int32_t* lowrow_, int ld_)
+        : M(M_), base(base_), S(nullptr), lowrow(lowrow_), ecnt(lowrow_ + 16),
+          cexp(lowrow_ + 16 + ld_), ld(ld_)
+    {
+    }
 };
 
 // What a warp keeps about the permanent it has staged.
 struct Staged {
     int perm = -1;
+    int mode = kStagedInt;
     int exp2 = 0;       // the terms' sum times 2^exp2 is the sum of prod_j S_j^{c_j}
     uint32_t emask = 0; // bit j: column j < 32 has extra prefixes
-    bool fp64 = false;  // staged as doubles, for fp64_walk
 };
 
 // Copy the oriented base matrix of permanent D into shared memory as scaled
@@ -113,8 +122,8 @@ static __device__ void stage_perm(const ExecArgs& a, const PermDesc& D, const Me
     __syncwarp();
     int esum = 0;
     st.perm = -1;
-    st.fp64 = !bint_stage(Md, sm.ld, k, l, mv.rmul, mv.cmul, sm.cexp, bad, lane, esum);
-    if (st.fp64) {
+    st.mode = bint_stage(Md, sm.ld, k, l, mv.rmul, mv.cmul, sm.cexp, bad, lane, esum, false);
+    if (st.mode == kStagedFp64) {
         double2* base = reinterpret_cast<double2*>(sm.base);
         for (int j = lane; j < l; j += kWarp) {
             double2 s = make_double2(0.0, 0.0);
@@ -145,18 +154,18 @@ static __device__ void stage_perm(const ExecArgs& a, const PermDesc& D, const Me
 // The column sums of one term, after its Gray step.  Shared memory: column j is
 // read, moved by the changed row's 2 b_j (STEP 1: the digit went up, 2: down,
 // 0: the chunk's first term) and written back as the term needs it.
-template <int STEP>
+template <int STEP, int STRIDE>
 struct SharedCols {
-    longlong2* S;        // this lane's, stride 32
+    longlong2* S;        // this lane's
     const longlong2* b;  // the changed row
     __device__ __forceinline__ longlong2 operator()(int j) const
     {
-        longlong2 s = S[j * 32];
+        longlong2 s = S[j * STRIDE];
         if (STEP != 0) {
             const longlong2 d = b[j];
             s.x = STEP == 1 ? s.x - d.x : s.x + d.x;
             s.y = STEP == 1 ? s.y - d.y : s.y + d.y;
-            S[j * 32] = s;
+            S[j * STRIDE] = s;
         }
         return s;
     }
@@ -171,36 +180,36 @@ struct RegCols {
 // prod_j S_j without repeated columns, 2^E times the integers returned: S_0 S_1,
 // then the columns in pairs, p (S_j S_{j+1}).  NL > 0: registers, unrolled,
 // l <= NL; NL = 0: shared memory.
-template <int NL, class Cols>
-__device__ __forceinline__ BInt unit_product(const Cols& col, int l, int& E)
+template <int NL, class Mul, class Cols>
+__device__ __forceinline__ BInt unit_product(const Mul& mul, const Cols& col, int l, int& E)
 {
     const longlong2 s0 = col(0);
     if (l == 1)
         return bint_plain(s0);
-    BInt p = bmul(sum_limbs(s0), sum_limbs(col(1)));
+    BInt p = mul(sum_limbs(s0), sum_limbs(col(1)));
     if constexpr (NL == 0) {
         int j = 2;
 #pragma unroll 1
         for (; j + 1 < l; j += 2) {
             const BLimbs x = sum_limbs(col(j)), y = sum_limbs(col(j + 1));
-            const BInt q = bmul(x, y);
+            const BInt q = mul(x, y);
             bnorm(p, E);
-            p = bmul(limbs(p), limbs(q));
+            p = mul(limbs(p), limbs(q));
         }
         if (j < l) {
             bnorm(p, E);
-            p = bmul(limbs(p), sum_limbs(col(j)));
+            p = mul(limbs(p), sum_limbs(col(j)));
         }
     } else {
 #pragma unroll
         for (int j = 2; j < NL; j += 2) {  // NL is even
             if (j + 1 < l) {
-                const BInt q = bmul(sum_limbs(col(j)), sum_limbs(col(j + 1)));
+                const BInt q = mul(sum_limbs(col(j)), sum_limbs(col(j + 1)));
                 bnorm(p, E);
-                p = bmul(limbs(p), limbs(q));
+                p = mul(limbs(p), limbs(q));
             } else if (j < l) {
                 bnorm(p, E);
-                p = bmul(limbs(p), sum_limbs(col(j)));
+                p = mul(limbs(p), sum_limbs(col(j)));
             }
         }
     }
@@ -210,8 +219,9 @@ __device__ __forceinline__ BInt unit_product(const Cols& col, int l, int& E)
 // The extra factors of a prefix (n_extra = ecnt[j] copies at column j, > 0): at
 // the first column with extras (jf) ex starts as that prefix, and every further
 // extra multiplies it in.
-__device__ __forceinline__ void extra_factors(BInt& pre, int& E, BInt& ex, int& Ex, int j, int jf,
-                                              int n_extra)
+template <class Mul>
+__device__ __forceinline__ void extra_factors(const Mul& mul, BInt& pre, int& E, BInt& ex, int& Ex,
+                                              int j, int jf, int n_extra)
 {
     bnorm(pre, E);
     const BLimbs lp = limbs(pre);
@@ -223,7 +233,7 @@ __device__ __forceinline__ void extra_factors(BInt& pre, int& E, BInt& ex, int& 
     }
 #pragma unroll 1
     for (; e < n_extra; ++e) {
-        ex = bmul(limbs(ex), lp);
+        ex = mul(limbs(ex), lp);
         Ex += E;
         bnorm(ex, Ex);
     }
@@ -232,55 +242,55 @@ __device__ __forceinline__ void extra_factors(BInt& pre, int& E, BInt& ex, int& 
 // Columns j and j + 1 (j + 1 < l, or j alone) of a term with repeated columns:
 // as one pair, p (S_j S_{j+1}), where no extra factor falls between them.
 // has(j): column j has extras.
-template <class Cols, class Has>
-__device__ __forceinline__ void prefix_pair(const Cols& col, const Has& has, BInt& pre, int& E,
-                                            BInt& ex, int& Ex, int j, int l, int jf,
-                                            const int32_t* ecnt)
+template <class Mul, class Cols, class Has>
+__device__ __forceinline__ void prefix_pair(const Mul& mul, const Cols& col, const Has& has,
+                                            BInt& pre, int& E, BInt& ex, int& Ex, int j, int l,
+                                            int jf, const int32_t* ecnt)
 {
     bnorm(pre, E);
     if (j + 1 < l && !has(j)) {
-        const BInt q = bmul(sum_limbs(col(j)), sum_limbs(col(j + 1)));
-        pre = bmul(limbs(pre), limbs(q));
+        const BInt q = mul(sum_limbs(col(j)), sum_limbs(col(j + 1)));
+        pre = mul(limbs(pre), limbs(q));
     } else {
-        pre = bmul(limbs(pre), sum_limbs(col(j)));
+        pre = mul(limbs(pre), sum_limbs(col(j)));
         if (has(j))
-            extra_factors(pre, E, ex, Ex, j, jf, ecnt[j]);
+            extra_factors(mul, pre, E, ex, Ex, j, jf, ecnt[j]);
         if (j + 1 >= l)
             return;
-        pre = bmul(limbs(pre), sum_limbs(col(j + 1)));
+        pre = mul(limbs(pre), sum_limbs(col(j + 1)));
     }
     if (has(j + 1))
-        extra_factors(pre, E, ex, Ex, j + 1, jf, ecnt[j + 1]);
+        extra_factors(mul, pre, E, ex, Ex, j + 1, jf, ecnt[j + 1]);
 }
 
 // prod_j S_j^{c_j}; UNIT: no repeated column, else from the prefixes.
-template <int NL, bool UNIT, class Cols>
-__device__ __forceinline__ BInt term_product(const Cols& col, int l, int jf, uint32_t emask,
-                                             const int32_t* ecnt, int& E)
+template <int NL, bool UNIT, class Mul, class Cols>
+__device__ __forceinline__ BInt term_product(const Mul& mul, const Cols& col, int l, int jf,
+                                             uint32_t emask, const int32_t* ecnt, int& E)
 {
     E = 0;
     if constexpr (UNIT)
-        return unit_product<NL>(col, l, E);
+        return unit_product<NL>(mul, col, l, E);
     BInt pre = bint_plain(col(0)), ex = pre;
     int Ex = 0;
     if constexpr (NL == 0) {
         auto has = [&](int j) { return ecnt[j] > 0; };
         if (has(0))
-            extra_factors(pre, E, ex, Ex, 0, jf, ecnt[0]);
+            extra_factors(mul, pre, E, ex, Ex, 0, jf, ecnt[0]);
 #pragma unroll 1
         for (int j = 1; j < l; j += 2)
-            prefix_pair(col, has, pre, E, ex, Ex, j, l, jf, ecnt);
+            prefix_pair(mul, col, has, pre, E, ex, Ex, j, l, jf, ecnt);
     } else {
         auto has = [&](int j) { return ((emask >> j) & 1u) != 0; };
         if (has(0))
-            extra_factors(pre, E, ex, Ex, 0, jf, ecnt[0]);
+            extra_factors(mul, pre, E, ex, Ex, 0, jf, ecnt[0]);
 #pragma unroll
         for (int j = 1; j < NL; j += 2)
             if (j < l)
-                prefix_pair(col, has, pre, E, ex, Ex, j, j + 1 < NL ? l : j + 1, jf, ecnt);
+                prefix_pair(mul, col, has, pre, E, ex, Ex, j, j + 1 < NL ? l : j + 1, jf, ecnt);
     }
     E += Ex;
-    return bmul(limbs(pre), limbs(ex));
+    return mul(limbs(pre), limbs(ex));
 }
 
 // acc +-= w 2^(-kSumBits - E) p
@@ -304,9 +314,11 @@ __device__ __forceinline__ void reweight(const LowWalk& wk, int J, double& wlow,
     wlow = (double)low_weight(wk, J);
 }
 
-// Write per = 2^{-(n-1)} * sum, and |per|^2 * norm, the sum being v 2^exp2; a
-// sharded plan writes its unscaled double-double sum instead.
-__device__ __forceinline__ void finalize(const ExecArgs& a, const PermDesc& D, dd2 v, int exp2)
+// Write per = 2^{-(n-1)} * sum, and |per|^2 * norm, the sum being v with the powers
+// of two and of i of its staging; a sharded plan writes its unscaled
+// double-double sum instead.
+__device__ __forceinline__ void finalize(const ExecArgs& a, const PermDesc& D, dd2 v,
+                                         int exp2, int f, int turns)
 {
     if (a.out_partial) {
         double* o = a.out_partial + 4 * (int64_t)D.out;
@@ -314,27 +326,24 @@ __device__ __forceinline__ void finalize(const ExecArgs& a, const PermDesc& D, d
             o[0] = 1.0;
             o[1] = o[2] = o[3] = 0.0;
         } else {
-            o[0] = scalbn(v.rh, exp2);
-            o[1] = scalbn(v.rl, exp2);
-            o[2] = scalbn(v.ih, exp2);
-            o[3] = scalbn(v.il, exp2);
+            const double2 h = turn(scalbn(v.rh, exp2), scalbn(v.ih, exp2 - f), turns);
+            const double2 e = turn(scalbn(v.rl, exp2), scalbn(v.il, exp2 - f), turns);
+            o[0] = h.x;
+            o[1] = e.x;
+            o[2] = h.y;
+            o[3] = e.y;
         }
         return;
     }
-    double re, im;
-    if (D.trivial) {
-        re = 1.0;
-        im = 0.0;
-    } else {
-        re = scale_exp2(__dadd_rn(v.rh, v.rl), exp2 + 1 - D.n);
-        im = scale_exp2(__dadd_rn(v.ih, v.il), exp2 + 1 - D.n);
-    }
+    double2 per = make_double2(1.0, 0.0);
+    if (!D.trivial)
+        per = turn(scale_exp2(__dadd_rn(v.rh, v.rl), exp2 + 1 - D.n),
+                   scale_exp2(__dadd_rn(v.ih, v.il), exp2 - f + 1 - D.n), turns);
     if (a.out_amp)
-        a.out_amp[D.out] = make_double2(re, im);
+        a.out_amp[D.out] = per;
     if (a.out_prob)
-        a.out_prob[D.out] = (re * re + im * im) * D.norm;
+        a.out_prob[D.out] = (per.x * per.x + per.y * per.y) * D.norm;
 }
-
 
 // The task's sum: every lane's chunk sum (rh + rl, ih + il) times its
 // high-digit weight (-1)^neg whigh_u (zero for a lane without a chunk), added
@@ -370,14 +379,14 @@ __device__ __forceinline__ dd2 task_sum(double rh, double rl, double ih, double 
 // The task's sum res (the same on every lane) goes to the permanent's output
 // if the permanent has one task; otherwise to its slot, and the warps that
 // finish last add the slots (gather_partials).
-static __device__ void combine_task(const ExecArgs& a, const Task& t, const PermDesc& D, dd2 res, int exp2,
-                             int lane)
+static __device__ void combine_task(const ExecArgs& a, const Task& t, const PermDesc& D, dd2 res,
+                                    int exp2, int f, int turns, int lane)
 {
     if (gather_partials(a.partials + 4 * (int64_t)D.slot0, a.counters + 1 + t.perm,
                         a.groups + D.gslot0, t.part - D.part0, D.ntasks, res.rh, res.rl, res.ih,
                         res.il, lane) &&
         lane == 0)
-        finalize(a, D, res, exp2);
+        finalize(a, D, res, exp2, f, turns);
 }
 
 // ---------------------------------------------------------------- the walk
@@ -398,14 +407,15 @@ __device__ __forceinline__ void start_walk(LowWalk& wk, const MetaView& mv, int 
 // (task_sum).  NL = 0: column sums in shared memory; NL > 0: in registers.
 // With and without repeated columns are walks of their own: one loop holding
 // both bodies took half as many instructions again per column.
-template <int NL, bool UNIT>
-__device__ __forceinline__ dd2 int_walk(const PermDesc& D, const MetaView& mv, const WarpSmem& sm,
-                                        uint32_t emask, int64_t chunk, bool active, int lane)
+// S: this lane's column sums with the given stride (NL = 0).
+template <int NL, bool UNIT, int STRIDE = 32, class Mul>
+__device__ __forceinline__ dd2 int_walk(const Mul& mul, longlong2* S, const PermDesc& D,
+                                        const MetaView& mv, const WarpSmem& sm, uint32_t emask,
+                                        int64_t chunk, bool active, int lane)
 {
     const int l = D.l, J = D.J, ndig = D.ndig, ld = NL > 0 ? NL : sm.ld;
     constexpr int kRegs = NL > 0 ? NL : 1;
     longlong2 R[kRegs];
-    longlong2* S = sm.S + lane;
     if constexpr (NL > 0) {
 #pragma unroll
         for (int j = 0; j < NL; ++j)
@@ -413,7 +423,7 @@ __device__ __forceinline__ dd2 int_walk(const PermDesc& D, const MetaView& mv, c
     } else {
 #pragma unroll 1
         for (int j = 0; j < l; ++j)
-            S[j * 32] = sm.base[j];
+            S[j * STRIDE] = sm.base[j];
     }
     const bool narrow = D.nchunks <= 0x7fffffff;
     uint64_t whigh_u = 1;
@@ -437,10 +447,10 @@ __device__ __forceinline__ dd2 int_walk(const PermDesc& D, const MetaView& mv, c
 #pragma unroll 1
             for (int j = 0; j < l; ++j) {
                 const longlong2 b = Mr[j];
-                longlong2 s = S[j * 32];
+                longlong2 s = S[j * STRIDE];
                 s.x -= g * b.x;
                 s.y -= g * b.y;
-                S[j * 32] = s;
+                S[j * STRIDE] = s;
             }
         }
         whigh_u *= high_binom(mv.dtop[d], g);
@@ -464,9 +474,9 @@ __device__ __forceinline__ dd2 int_walk(const PermDesc& D, const MetaView& mv, c
     int E;
     BInt p;
     if constexpr (NL > 0)
-        p = term_product<NL, UNIT>(RegCols<kRegs>{R}, l, jf, emask, sm.ecnt, E);
+        p = term_product<NL, UNIT>(mul, RegCols<kRegs>{R}, l, jf, emask, sm.ecnt, E);
     else
-        p = term_product<0, UNIT>(SharedCols<0>{S, sm.M}, l, jf, emask, sm.ecnt, E);
+        p = term_product<0, UNIT>(mul, SharedCols<0, STRIDE>{S, sm.M}, l, jf, emask, sm.ecnt, E);
     uint32_t s = 0;
 #pragma unroll 1
     for (;;) {
@@ -513,11 +523,11 @@ __device__ __forceinline__ dd2 int_walk(const PermDesc& D, const MetaView& mv, c
                     R[j].y -= b.y;
                 }
             }
-            p = term_product<NL, UNIT>(RegCols<kRegs>{R}, l, jf, emask, sm.ecnt, E);
+            p = term_product<NL, UNIT>(mul, RegCols<kRegs>{R}, l, jf, emask, sm.ecnt, E);
         } else if (step & 1u) {
-            p = term_product<0, UNIT>(SharedCols<2>{S, Mr}, l, jf, emask, sm.ecnt, E);
+            p = term_product<0, UNIT>(mul, SharedCols<2, STRIDE>{S, Mr}, l, jf, emask, sm.ecnt, E);
         } else {
-            p = term_product<0, UNIT>(SharedCols<1>{S, Mr}, l, jf, emask, sm.ecnt, E);
+            p = term_product<0, UNIT>(mul, SharedCols<1, STRIDE>{S, Mr}, l, jf, emask, sm.ecnt, E);
         }
     }
     return task_sum(rh, rl, ih, il, whigh_u, (gpar & 1) != 0, active);
@@ -556,7 +566,7 @@ static __device__ void fp64_term(const double2* S, int l, int jf, const int32_t*
         cfma_acc<false>(acc, pre, ex);
 }
 
-static __device__ __noinline__ dd2 fp64_walk(const PermDesc& D, const MetaView& mv, const WarpSmem& sm,
+static __device__ dd2 fp64_walk(const PermDesc& D, const MetaView& mv, const WarpSmem& sm,
                                       int64_t chunk, bool active)
 {
     const int l = D.l, J = D.J, ndig = D.ndig;
@@ -608,6 +618,41 @@ static __device__ __noinline__ dd2 fp64_walk(const PermDesc& D, const MetaView& 
     return task_sum(rh, rl, ih, il, whigh_u, (gpar & 1) != 0, active);
 }
 
+// The sum of a walk off the main path; the imaginary part is to be taken times 2^-f,
+// and the whole times i^turns.
+struct WalkSum {
+    dd2 v;
+    int f, turns;
+};
+
+// The walks of matrices that are not staged as integers of one unit.  Not inlined,
+// and called with what it cannot read again, so that the main path keeps no object
+// in memory for it.
+static __device__ __noinline__ WalkSum other_walk(const PermDesc* desc, const int32_t* meta,
+                                                  longlong2* M, longlong2* base, int32_t* lowrow,
+                                                  int ld, int mode, uint32_t emask, int64_t chunk,
+                                                  bool active, int lane)
+{
+    const PermDesc D = *desc;
+    const MetaView mv = meta_view(meta, D);
+    const WarpSmem sm(M, base, lowrow, ld);
+    WalkSum r;
+    r.f = r.turns = 0;
+    if (mode == kStagedFp64) {
+        r.v = fp64_walk(D, mv, sm, chunk, active);
+        return r;
+    }
+    // column sums in local memory
+    longlong2 S[PQ_MAX_PRODUCT_COLS];
+    r.f = sscale_of(sm.cexp[0]).f;
+    for (int j = 0; j < D.l; ++j)
+        r.turns += sscale_of(sm.cexp[j]).turned ? mv.cmul[j] : 0;
+    const PartUnits mul{min(63, 2 * r.f)};
+    r.v = D.jf < 0 ? int_walk<0, true, 1>(mul, S, D, mv, sm, emask, chunk, active, lane)
+                   : int_walk<0, false, 1>(mul, S, D, mv, sm, emask, chunk, active, lane);
+    return r;
+}
+
 template <int NL>
 __device__ __forceinline__ void process_task(const ExecArgs& a, const Task& t, WarpSmem& sm,
                                              Staged& st, int lane)
@@ -615,6 +660,7 @@ __device__ __forceinline__ void process_task(const ExecArgs& a, const Task& t, W
     const PermDesc D = a.desc[t.perm];
     const MetaView mv = meta_view(a.meta, D);
     dd2 res = {0.0, 0.0, 0.0, 0.0};
+    int f = 0, turns = 0;
     if (!D.trivial) {
         if (st.perm != t.perm) {
             __syncwarp();
@@ -624,14 +670,19 @@ __device__ __forceinline__ void process_task(const ExecArgs& a, const Task& t, W
         const int64_t chunk0 = (int64_t)t.part * kWarp;
         const bool active = chunk0 + lane < D.nchunks;
         const int64_t chunk = active ? (chunk0 + lane) : 0;
-        if (st.fp64)
-            res = fp64_walk(D, mv, sm, chunk, active);
-        else if (D.jf < 0)
-            res = int_walk<NL, true>(D, mv, sm, st.emask, chunk, active, lane);
-        else
-            res = int_walk<NL, false>(D, mv, sm, st.emask, chunk, active, lane);
+        if (st.mode != kStagedInt) {
+            const WalkSum r = other_walk(a.desc + t.perm, a.meta, sm.M, sm.base, sm.lowrow, sm.ld,
+                                         st.mode, st.emask, chunk, active, lane);
+            res = r.v;
+            f = r.f;
+            turns = r.turns;
+        } else if (D.jf < 0) {
+            res = int_walk<NL, true>(OneUnit(), sm.S + lane, D, mv, sm, st.emask, chunk, active, lane);
+        } else {
+            res = int_walk<NL, false>(OneUnit(), sm.S + lane, D, mv, sm, st.emask, chunk, active, lane);
+        }
     }
-    combine_task(a, t, D, res, st.exp2, lane);
+    combine_task(a, t, D, res, st.exp2, f, turns, lane);
 }
 
 // Task ti of the list, once its guards pass (a failing task is skipped and

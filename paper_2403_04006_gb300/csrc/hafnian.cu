@@ -41,7 +41,10 @@
 // N = 36 took 19.1 ms (hafnian), N = 28 with loops 1.68 ms; in integers, bound
 // by the wide multiplies and their adds, 4.67 ms and 0.34 ms.  A matrix
 // without a scale (non-finite or subnormal entries, a bound beyond FP64) is
-// walked in FP64.
+// walked in FP64.  Where the terms lie near the real or imaginary axis, one unit
+// for both parts would round the small one (pq_blockint.cuh): a hafnian then has a
+// unit for each part, a loop hafnian, whose factors add two terms of any ratio,
+// keeps the FP64 walk.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -205,8 +208,9 @@ struct HafMeta {
 // What a warp keeps about the item it has staged.
 struct HafStaged {
     int item = -1;
-    bool fp64 = false;  // staged as doubles
+    int mode = kStagedInt;
     int exp2 = 0;       // the terms' sum times 2^exp2 is the sum of s(g) times the polynomial
+                        // (in integers: without its leading factor)
     int eq = 0, el = 0; // q and l times 2^eq, 2^el are the integers
     int ref2 = 0, ref1 = 0;  // loop hafnian: upper bounds of a factor's exponent (pair, odd root)
 };
@@ -394,17 +398,128 @@ __device__ __noinline__ dd2 haf_walk_fp64(const HafDesc& D, const HafMeta& mt, c
     return res;
 }
 
-// Stage item D as scaled integers: M = 2 b, y0 = B r, gam.  Returns false (nothing converted) if the item has no scale.
+// Whether the terms of an item can lie near an axis (pq_blockint.cuh): b the parts
+// of the entries that q takes, g those of the loop weights, root the exponent of
+// the loop polynomial's largest root (its first factor is q + 2^root l^2 or so).
+// q^n is near an axis where q is; a factor of the loop polynomial where the larger
+// of its two terms' parts are far apart, and N = 1 leaves l alone.
+template <bool LOOP>
+__device__ __forceinline__ bool haf_near_axis(const BParts& b, const BParts& g, int N, int root)
+{
+    if (!LOOP)
+        return bint_near_axis(b);
+    if (N == 1)
+        return bint_near_axis(g);
+    constexpr int kNone = -(1 << 20);
+    int re = b.no_re() ? kNone : bint_exponent(b.re) - 1023;
+    int im = b.no_im() ? kNone : bint_exponent(b.im) - 1023;
+    const int x = g.no_re() ? kNone : bint_exponent(g.re) - 1023;
+    const int y = g.no_im() ? kNone : bint_exponent(g.im) - 1023;
+    re = max(re, 2 * max(x, y) + root);
+    im = max(im, x + y + 1 + root);
+    return min(re, im) > kNone / 2 && abs(re - im) >= kAxisBits;
+}
+
+// The power of two that brings the largest part near 1, leaving at most 900
+// binades below it to the smaller one.
+__device__ __forceinline__ int unit_scale(const BParts& m)
+{
+    const int x = bint_exponent(m.re), y = bint_exponent(m.im);
+    const int hi = max(x, y), lo = m.no_re() || m.no_im() ? hi : min(x, y);
+    return 1023 - hi + max(0, hi - lo - 900);
+}
+
+// A loop hafnian near an axis, for the FP64 walk: entries times 2^(2 t) and loop
+// weights times 2^t, which multiplies every term by 2^(t N) and keeps the powers in
+// range.  Returns t.
+__device__ __noinline__ int haf_scale(const HafSmem& sm, int k, const BParts& b, const BParts& g,
+                                      uint32_t hmax, int lane)
+{
+    int t = b.no_re() && b.no_im() ? 1 << 20 : unit_scale(b) >> 1;
+    if (!g.no_re() || !g.no_im())
+        t = min(t, unit_scale(g));
+    t = min(t, (1023 + 900 - bint_exponent(hmax)) >> 1);  // all entries stay finite
+    for (int e = lane; e < k * k; e += kWarp)
+        sm.M[e] = make_double2(scalbn(sm.M[e].x, 2 * t), scalbn(sm.M[e].y, 2 * t));
+    for (int i = lane; i < k; i += kWarp)
+        sm.gam[i] = make_double2(scalbn(sm.gam[i].x, t), scalbn(sm.gam[i].y, t));
+    __syncwarp();
+    return t;
+}
+
+// The scale of the sums of one part (im or re) of q, hmax its entries' largest
+// high word.
+__device__ __forceinline__ int haf_part_scale(const HafMeta& mt, const HafSmem& sm, int k, bool im,
+                                              uint32_t hmax, int lane)
+{
+    uint64_t units = 0;
+    for (int i = lane; i < k; i += kWarp) {
+        uint32_t row = 0;
+        for (int j = 0; j < k; ++j) {
+            const double2 v = sm.M[i * k + j];
+            row += (uint32_t)(mt.rmul[j] + (j == i ? 1 : 0)) *
+                   bint_units(bint_mag(im ? v.y : v.x, 0.0), hmax);
+        }
+        units += (uint64_t)mt.rmul[i] * row;
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1)
+        units += __shfl_xor_sync(0xffffffffu, units, off);
+    units += (units >> 20) + 1;  // the rounding of the entries stays inside the bound
+    return kSumBits + 1044 - (int)(hmax >> 20) - bint_width(units);
+}
+
+// A hafnian near an axis: M = 2 b with a unit for each part, divided by i where the
+// imaginary part is the larger.  False if a part has no scale (subnormal).
+__device__ __noinline__ bool haf_stage_parts(const HafMeta& mt, const HafSmem& sm, int k,
+                                             const BParts& all, SScale& s, int lane)
+{
+    if (min(all.re, all.im) < 0x100000u)
+        return false;
+    s.turned = bint_exponent(all.im) > bint_exponent(all.re);
+    const int big = haf_part_scale(mt, sm, k, s.turned, max(all.re, all.im), lane);
+    const int small = haf_part_scale(mt, sm, k, !s.turned, min(all.re, all.im), lane);
+    s.e = min(big, small);
+    s.f = small - s.e;
+    longlong2* M = reinterpret_cast<longlong2*>(sm.M);
+    for (int e = lane; e < k * k; e += kWarp) {
+        const double2 b = sm.M[e];
+        M[e] = make_longlong2(2 * bint_of(s.turned ? b.y : b.x, s.e),
+                              2 * bint_of(s.turned ? -b.x : b.y, s.e + s.f));
+    }
+    __syncwarp();
+    return true;
+}
+
+__device__ __forceinline__ void warp_parts(BParts& m)
+{
+    m.re = __reduce_max_sync(0xffffffffu, m.re);
+    m.im = __reduce_max_sync(0xffffffffu, m.im);
+    m.re_low = __reduce_or_sync(0xffffffffu, m.re_low);
+    m.im_low = __reduce_or_sync(0xffffffffu, m.im_low);
+}
+
+// Stage item D as scaled integers: M = 2 b, y0 = B r, gam; a hafnian near an axis
+// with a unit for each part (ci[0]: its SScale).  Returns false if it stays in
+// doubles: an item without a scale as it came, a loop hafnian near an axis scaled.
 template <bool LOOP>
 __device__ bool haf_stage_int(const HafDesc& D, const HafMeta& mt, const HafSmem& sm, HafStaged& st,
                               int lane)
 {
     const int k = D.k;
+    st.mode = kStagedInt;
+    st.exp2 = 0;
     bool bad = false;
-    uint32_t hmax = 0, gmax = 0;
-    for (int e = lane; e < k * k; e += kWarp)
-        hmax = max(hmax, bint_mag(sm.M[e].x, sm.M[e].y));
-    hmax = __reduce_max_sync(0xffffffffu, hmax);
+    BParts all, b, g;  // b: without the diagonal entries of single indices, which q cancels
+    for (int e = lane; e < k * k; e += kWarp) {
+        const int i = e / k;
+        all.add(sm.M[e].x, sm.M[e].y);
+        if (e != i * k + i || mt.rmul[i] > 1)
+            b.add(sm.M[e].x, sm.M[e].y);
+    }
+    warp_parts(b);
+    const uint32_t hmax = __reduce_max_sync(0xffffffffu, max(all.re, all.im));
+    uint32_t gmax = 0;
     // |q| <= 1/2 (sum_ij r_i r_j |b_ij| + sum_i r_i |b_ii|)
     uint64_t units = 0;
     for (int i = lane; i < k; i += kWarp) {
@@ -422,29 +537,43 @@ __device__ bool haf_stage_int(const HafDesc& D, const HafMeta& mt, const HafSmem
     bad = hmax < 0x100000u || hmax >= 0x7ff00000u || eq < kSumBits - 1023;
     int el = 0;
     if (LOOP) {
-        bool nonzero = false;
-        for (int i = lane; i < k; i += kWarp) {
-            gmax = max(gmax, bint_mag(sm.gam[i].x, sm.gam[i].y));
-            nonzero = nonzero || sm.gam[i].x != 0.0 || sm.gam[i].y != 0.0;
-        }
-        gmax = __reduce_max_sync(0xffffffffu, gmax);
+        for (int i = lane; i < k; i += kWarp)
+            g.add(sm.gam[i].x, sm.gam[i].y);
+        warp_parts(g);
+        gmax = max(g.re, g.im);
         uint32_t gu = 0;
         for (int i = lane; i < k; i += kWarp)
             gu += (uint32_t)mt.rmul[i] * bint_units(bint_mag(sm.gam[i].x, sm.gam[i].y), gmax);
         gu = __reduce_add_sync(0xffffffffu, gu);
-        if (__any_sync(0xffffffffu, nonzero)) {
+        if (!g.no_re() || !g.no_im()) {
             el = bint_scale(gmax, gu);
             bad = bad || gmax < 0x100000u || gmax >= 0x7ff00000u || el < kSumBits - 1023;
         }
     }
     if (bad)
         return false;
+    const int root = LOOP && D.N > 1 ? (int)sm.ci[0] : 0;
+    SScale ps{eq, 0, false};
+    if (haf_near_axis<LOOP>(b, g, D.N, root)) {
+        if (LOOP) {
+            st.exp2 = -haf_scale(sm, k, b, g, hmax, lane) * D.N;
+            return false;
+        }
+        warp_parts(all);
+        if (!haf_stage_parts(mt, sm, k, all, ps, lane))
+            return false;
+        st.mode = kStagedParts;
+        if (lane == 0)
+            sm.ci[0] = ps.pack();
+    }
     longlong2* M = reinterpret_cast<longlong2*>(sm.M);
     longlong2* y0 = reinterpret_cast<longlong2*>(sm.y0);
     longlong2* gam = reinterpret_cast<longlong2*>(sm.gam);
-    for (int e = lane; e < k * k; e += kWarp) {
-        const double2 b = sm.M[e];
-        M[e] = make_longlong2(2 * bint_of(b.x, eq), 2 * bint_of(b.y, eq));
+    if (st.mode == kStagedInt) {
+        for (int e = lane; e < k * k; e += kWarp) {
+            const double2 v = sm.M[e];
+            M[e] = make_longlong2(2 * bint_of(v.x, eq), 2 * bint_of(v.y, eq));
+        }
     }
     if (LOOP) {
         for (int i = lane; i < k; i += kWarp) {
@@ -473,19 +602,9 @@ __device__ bool haf_stage_int(const HafDesc& D, const HafMeta& mt, const HafSmem
         st.ref1 = jo == 0 ? 0 : 2 + max(xq, xs + (int)sm.ci[4 * P] + 2);
         st.exp2 = kSumBits + 64 * (P + jo + no - 1) + P * st.ref2 + jo * st.ref1 - no * el;
     } else {
-        st.exp2 = kSumBits + 64 * (D.n - 1) - D.n * eq;
+        st.exp2 = kSumBits + 64 * (D.n - 1) - D.n * ps.e;
     }
     return true;
-}
-
-__device__ __forceinline__ BInt bint_words(longlong2 s)
-{
-    BInt p;
-    p.rh = (int)(s.x >> 32);
-    p.rl = (uint32_t)s.x;
-    p.ih = (int)(s.y >> 32);
-    p.il = (uint32_t)s.y;
-    return p;
 }
 
 __device__ __forceinline__ longlong2 bint_pair(const BInt& p)
@@ -498,8 +617,9 @@ __device__ __forceinline__ longlong2 bint_pair(const BInt& p)
 // integers, normalised, and their exponents E.  M = 2 interleaves two terms,
 // whose dependent chains of products then hide each other (N = 36: 4.87 -> 4.67
 // ms; 14 warps fit on an SM by shared memory, which leaves 128 registers).
-template <int M>
-__device__ __forceinline__ void haf_power(const longlong2 (&q)[M], int n, BInt (&h)[M], int (&E)[M])
+template <int M, class Mul>
+__device__ __forceinline__ void haf_power(const longlong2 (&q)[M], int n, BInt (&h)[M], int (&E)[M],
+                                          const Mul& mul)
 {
     BLimbs lx[M];
     int Ex[M];
@@ -515,14 +635,14 @@ __device__ __forceinline__ void haf_power(const longlong2 (&q)[M], int n, BInt (
     for (int bit = 30 - __clz(n); bit >= 0; --bit) {
 #pragma unroll
         for (int i = 0; i < M; ++i) {
-            h[i] = bsqr(limbs(h[i]));
+            h[i] = mul.sqr(limbs(h[i]));
             E[i] *= 2;
             bnorm(h[i], E[i]);
         }
         if ((n >> bit) & 1) {
 #pragma unroll
             for (int i = 0; i < M; ++i) {
-                h[i] = bmul(limbs(h[i]), lx[i]);
+                h[i] = mul(limbs(h[i]), lx[i]);
                 E[i] += Ex[i];
                 bnorm(h[i], E[i]);
             }
@@ -620,9 +740,10 @@ __device__ __forceinline__ BInt haf_loop_poly(longlong2 q, longlong2 l, int P, b
 // The walk of this lane's chunk in block integers; returns the task's sum.
 // All sums are taken modulo 2^64 (unsigned): y may leave the range of 64 bits,
 // q and l do not.
-template <bool LOOP>
+template <bool LOOP, class Mul>
 __device__ __forceinline__ dd2 haf_walk_int(const HafDesc& D, const HafMeta& mt, const HafSmem& sm,
-                                            const HafStaged& st, int64_t c, bool active, int lane)
+                                            const HafStaged& st, int64_t c, bool active, int lane,
+                                            const Mul& mul)
 {
     const int k = D.k, J = D.J, nd = D.ndig;
     const ulonglong2* M = reinterpret_cast<const ulonglong2*>(sm.M);
@@ -776,14 +897,14 @@ __device__ __forceinline__ dd2 haf_walk_int(const HafDesc& D, const HafMeta& mt,
             const longlong2 q2[2] = {q0, make_longlong2((long long)q.x, (long long)q.y)};
             BInt p[2];
             int E[2];
-            haf_power<2>(q2, n, p, E);
+            haf_power(q2, n, p, E, mul);
             add_term(p[0], E[0], s - 1, w0);
             add_term(p[1], E[1], s, w);
         } else {
             const longlong2 q1[1] = {q0};
             BInt p[1];
             int E[1];
-            haf_power<1>(q1, n, p, E);
+            haf_power(q1, n, p, E, mul);
             add_term(p[0], E[0], s, w);
         }
         ++s;
@@ -815,6 +936,13 @@ __device__ __forceinline__ dd2 haf_walk_int(const HafDesc& D, const HafMeta& mt,
     return res;
 }
 
+__device__ __noinline__ dd2 haf_walk_parts(const HafDesc& D, const HafMeta& mt, const HafSmem& sm,
+                                           const HafStaged& st, int64_t c, bool active, int lane)
+{
+    const PartUnits mul{min(63, 2 * sscale_of((int32_t)sm.ci[0]).f)};
+    return haf_walk_int<false>(D, mt, sm, st, c, active, lane, mul);
+}
+
 template <bool LOOP>
 __device__ void haf_task(const HafArgs& a, const Task& t, const HafSmem& sm, HafStaged& st, int lane)
 {
@@ -840,8 +968,8 @@ __device__ void haf_task(const HafArgs& a, const Task& t, const HafSmem& sm, Haf
                     sm.ci[j] = __double_as_longlong(a.loopc[D.coef_off + nf + j]);
             }
             __syncwarp();
-            st.fp64 = !haf_stage_int<LOOP>(D, mt, sm, st, lane);
-            if (st.fp64) {
+            if (!haf_stage_int<LOOP>(D, mt, sm, st, lane)) {
+                st.mode = kStagedFp64;
                 for (int j = lane; j < k; j += kWarp) {  // y0 = B r
                     double2 s = make_double2(0.0, 0.0);
                     for (int i = 0; i < k; ++i) {
@@ -858,8 +986,12 @@ __device__ void haf_task(const HafArgs& a, const Task& t, const HafSmem& sm, Haf
         const int64_t chunk0 = (int64_t)t.part * kWarp;
         const bool active = chunk0 + lane < D.nchunks;
         const int64_t c = active ? (chunk0 + lane) : 0;
-        res = st.fp64 ? haf_walk_fp64<LOOP>(D, mt, sm, c, active, lane)
-                      : haf_walk_int<LOOP>(D, mt, sm, st, c, active, lane);
+        if (st.mode == kStagedFp64)
+            res = haf_walk_fp64<LOOP>(D, mt, sm, c, active, lane);
+        else if (LOOP || st.mode == kStagedInt)
+            res = haf_walk_int<LOOP>(D, mt, sm, st, c, active, lane, OneUnit());
+        else
+            res = haf_walk_parts(D, mt, sm, st, c, active, lane);
     }
 
     auto finish = [&](dd2 v) {
@@ -868,13 +1000,18 @@ __device__ void haf_task(const HafArgs& a, const Task& t, const HafSmem& sm, Haf
             o = make_double2(D.value, 0.0);
         } else {
             // the FP64 walk's terms hold the loop polynomial's leading factor
-            const double f = LOOP && !st.fp64 ? D.value * sm.cj[0] : D.value;
-            const int x = (st.fp64 ? 0 : st.exp2) + 1 - D.N;
+            const double f = LOOP && st.mode == kStagedInt ? D.value * sm.cj[0] : D.value;
+            const int x = st.exp2 + 1 - D.N;
             double h, e;
             fast_two_sum(v.rh, v.rl, h, e);
             o.x = scalbn((h + e) * f, x);
             fast_two_sum(v.ih, v.il, h, e);
-            o.y = scalbn((h + e) * f, x);
+            if (!LOOP && st.mode == kStagedParts) {
+                const SScale ps = sscale_of((int32_t)sm.ci[0]);
+                o = turn(o.x, scalbn((h + e) * f, x - ps.f), ps.turned ? D.n : 0);
+            } else {
+                o.y = scalbn((h + e) * f, x);
+            }
         }
         a.out[t.perm] = o;
     };
