@@ -691,9 +691,9 @@ static int schedule_and_upload(pq_plan* P)
             }
             return tasks > 0.0 ? std::max(total / warps, longest) + 0.25 * total / tasks : 0.0;
         };
+        std::vector<Cut> trial(groups.cut.size());
         auto choose = [&](size_t g0, size_t g1, bool whole_batch) {
             double best = cut(g0, g1, 10, whole_batch, groups.cut);
-            std::vector<Cut> trial = groups.cut;
             for (int cap = 9; search && cap >= 0; --cap) {
                 const double t = cut(g0, g1, cap, whole_batch, trial);
                 if (t < 0.99 * best) {
