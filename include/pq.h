@@ -579,6 +579,13 @@ int pq_fixsum_device(const double* hi, const double* lo, int32_t n, double* out,
  * its direction (+1 / -1) to host arrays digit[steps], dir[steps]. */
 int pq_gray_walk(const int32_t* radix, int32_t ndig, int64_t steps, int32_t* digit, int32_t* dir);
 
+/* The same steps as the integer walks work them out, each from its number alone:
+ * digit and dir as above, weight[s] the product of the binomials C(top[d], value
+ * of digit d) after step s (radix[d] - 1 <= top[d] <= 15), and value[s * ndig + d] the
+ * digits after it.  Host arrays; no GPU.  Errors: PQ_ERR_ARG. */
+int pq_gray_steps(const int32_t* radix, const int32_t* top, int32_t ndig, int64_t steps,
+                  int32_t* digit, int32_t* dir, int64_t* weight, int32_t* value);
+
 /* The factors the loop-hafnian kernel evaluates its degree-N polynomial
  * sum_{j <= N/2} q^j l^{N-2j} / (j! (N-2j)!) with (host only; no GPU needed):
  * out[0] = 1 / J!, J = floor(N/2); then for each pair of the real roots

@@ -35,6 +35,40 @@ extern "C" int pq_gray_walk(const int32_t* radix, int32_t ndig, int64_t steps, i
     return PQ_OK;
 }
 
+extern "C" int pq_gray_steps(const int32_t* radix, const int32_t* top, int32_t ndig, int64_t steps,
+                             int32_t* digit, int32_t* dir, int64_t* weight, int32_t* value)
+{
+    if (ndig < 0 || ndig > pqi::kMaxLowDigits || steps < 0 || (ndig > 0 && (!radix || !top)) ||
+        (steps > 0 && (!digit || !dir || !weight || !value)))
+        return PQ_ERR_ARG;
+    pqi::LowDigits lo;
+    lo.radm1 = lo.topp = 0;
+    lo.J = ndig;
+    int64_t total = 1;
+    for (int d = 0; d < ndig; ++d) {
+        if (radix[d] < 2 || radix[d] > pqi::kMaxLowRadix || top[d] < radix[d] - 1 || top[d] > 15)
+            return PQ_ERR_ARG;
+        lo.radm1 |= uint64_t(radix[d] - 1) << (4 * d);
+        lo.topp |= uint64_t(top[d]) << (4 * d);
+        total *= radix[d];
+        if (total > (int64_t(1) << 30))  // the longest chunk
+            return PQ_ERR_ARG;
+    }
+    if (steps > total - 1)
+        return PQ_ERR_ARG;
+    for (int64_t s = 0; s < steps; ++s) {
+        bool up;
+        uint64_t w;
+        digit[s] = pqi::gray_step_at(lo, (uint32_t)(s + 1), true, up, w);
+        dir[s] = up ? 1 : -1;
+        weight[s] = (int64_t)w;
+        const uint64_t g = pqi::gray_value_at(lo, (uint32_t)(s + 1));
+        for (int d = 0; d < ndig; ++d)
+            value[s * ndig + d] = (int32_t)((g >> (4 * d)) & 15u);
+    }
+    return PQ_OK;
+}
+
 // The forward kernels' exact warp sum, run on the host: the same conversion,
 // the same 26-bit limbs added as 32-bit words (as redux.sync adds them) and
 // the same conversion back, over n <= 32 lanes.
