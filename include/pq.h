@@ -149,7 +149,11 @@ int pq_plan_destroy(pq_plan* plan);
  * of Sec. 4.2), evaluated by the multiplicity-extended BB/FG formula over a
  * mixed-radix Gray code, the products in 64-bit block integers (FP64 where an
  * entry is not finite or a column's sums can overflow), accumulated in
- * double-double.
+ * double-double.  The error is bounded against the size of the terms: the real
+ * and imaginary parts share a unit, except where all columns lie near an axis
+ * (one part below 1/16 of the other in size), where each part keeps the
+ * precision that its own size gives it in FP64.  The same holds for gradients
+ * and hafnians.
  * b: device descriptor; out: device, batch entries.  plan: made by
  * pq_plan_create for the same sizes, or NULL, in which case the call copies
  * the sizes to the host, plans, runs the batched method and synchronises

@@ -894,7 +894,7 @@ __device__ __forceinline__ void bwdr_walk_int(const PermDesc& D, const MetaView&
 // entries, a column bound beyond FP64), with the lane's arrays in local memory.
 __device__ __noinline__ void bwdr_walk_fp64(const PermDesc& D, const MetaView& mv,
                                             const BwdRegSmem& sm, const LowDigits& lo,
-                                            int64_t chunk, int n2, double2* A, uint64_t& whigh_u,
+                                            int64_t chunk, double2* A, uint64_t& whigh_u,
                                             int& gpar, int lane)
 {
     const int l = D.l, ld = sm.ld;
@@ -1067,7 +1067,7 @@ __device__ void bwdr_task(const BwdArgs& a, const Task& t, BwdRegSmem& sm, BwdSt
         if (st.mode != kStagedInt) {
             double2 Af[kBwdRegMaxLd];
             if (st.mode == kStagedFp64)
-                bwdr_walk_fp64(D, mv, sm, lo, chunk, n2, Af, whigh_u, gpar, lane);
+                bwdr_walk_fp64(D, mv, sm, lo, chunk, Af, whigh_u, gpar, lane);
             else
                 bwdr_walk_parts(D, mv, sm, lo, chunk, Af, whigh_u, gpar, lane);
 #pragma unroll
@@ -1332,14 +1332,14 @@ int bwd_smem_bytes_for(int kmax, int ld, int jb, int n2)
     return bwd_warp_smem_bytes(kmax, ld, jb, n2);
 }
 
-int bwd_regs_per_thread(int)
+int bwd_regs_per_thread()
 {
     cudaFuncAttributes at{};
     return cudaFuncGetAttributes(&at, glynn_bwd_kernel) == cudaSuccess ? at.numRegs : 255;
 }
 
 // Raise (never lower) the kernel's dynamic shared-memory limit.
-cudaError_t bwd_prepare(int, int smem_bytes)
+cudaError_t bwd_prepare(int smem_bytes)
 {
     cudaFuncAttributes at{};
     cudaError_t e = cudaFuncGetAttributes(&at, glynn_bwd_kernel);

@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(256, 2) glynn_fwd_kernel(ExecArgs a, int64_t t
 // ---------------------------------------------------------------- host side
 int fwd_smem_per_warp(int kmax, int ld) { return warp_smem_bytes(kmax, ld); }
 
-int fwd_regs_per_thread(int)
+int fwd_regs_per_thread()
 {
     cudaFuncAttributes at{};
     return cudaFuncGetAttributes(&at, glynn_fwd_kernel) == cudaSuccess ? at.numRegs : 255;
@@ -47,7 +47,7 @@ int fwd_regs_per_thread(int)
 
 // Raise (never lower) the kernel's dynamic shared-memory limit: plans made
 // earlier with larger workspaces must keep launching.
-cudaError_t fwd_prepare(int, int smem_bytes)
+cudaError_t fwd_prepare(int smem_bytes)
 {
     cudaFuncAttributes at{};
     cudaError_t e = cudaFuncGetAttributes(&at, glynn_fwd_kernel);

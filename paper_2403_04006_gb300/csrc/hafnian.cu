@@ -20,7 +20,7 @@
 // the summand is even under flipping every sign).  A Gray step changes one
 // x_r by D = -+2:  q += D y_r + 2 B_rr with y = B x, then y_j += D B_jr and
 // l += D gamma_r.  Inside a chunk only the J low digits move, so the walk
-// reads y at the J low rows alone and keeps only those (2J DFMA a step
+// reads y at the J low rows alone and keeps only those (2J adds a step
 // instead of 2k); y is formed in full once per chunk for the start value of
 // q.  q^n is taken by repeated squaring.  The loop polynomial is homogeneous
 // of degree N/2 in (q, l^2): sum_j q^j s^{J-j} / (j! (N-2j)!) with s = l^2,
@@ -29,8 +29,7 @@
 // polynomial He_N (substituting z = -1/(2x^2) turns the sum into
 // x^{-N} He_N(x) / N!).  The roots are real, found once per N on the host by
 // Sturm-count bisection on the Jacobi matrix of He_N, and the kernel
-// multiplies the factors in pairs: 2 FP64 operations per unit of N instead
-// of Horner's 5.
+// multiplies the factors in pairs.
 //
 // The walk runs in 64-bit block integers (pq_blockint.cuh) on the integer
 // pipes, as the permanent's does: q, y and l are scaled integers (every update
@@ -1142,7 +1141,6 @@ static double factorial_h(int n)
     return r;
 }
 
-// Plan, upload, run and synchronise; gamma == nullptr selects the hafnian.
 }  // namespace pqi
 
 // A planned batch of (loop) hafnians: host schedule uploaded once, device
@@ -1295,9 +1293,13 @@ static int haf_plan_build(const int64_t* mat_off, const int32_t* k, const int32_
             D.coef_off = coef_at[N];
         }
         // Chunk length L = product of the J low radices, at most 4096 terms,
-        // at most T / (32 x the item's task share), and J minimising the FP64
-        // work per term: 2J + 8 for the walk plus 2k(ndig - J) + 4k + 64 per
-        // chunk for the start value.
+        // at most T / (32 x the item's task share), and J minimising the work per
+        // term, 2J + 8 for the walk plus 2k(ndig - J) + 4k + 64 per chunk for the
+        // start value: the FP64 walk's counts, which leave out a task's staging
+        // and lane sums.  With J - 1, J and J + 1, in ms: hafnian (2, ..., 2), k =
+        // 18, 4.76, 4.65, 4.97; k = 14 0.60, 0.25, 0.14; (3, ..., 3), k = 10 0.234,
+        // 0.235, 0.101; loop hafnian (2, ..., 2), k = 14 0.71, 0.35, 0.23.  So the
+        // share of 64 tasks per SM is the larger part of the smaller items' time.
         const double share = std::max(1.0, std::ceil(want_tasks * (double)T / t_total));
         const int64_t cap = std::max<int64_t>(
             1, std::min<int64_t>(4096, (int64_t)((double)T / (kWarp * share))));
@@ -1358,6 +1360,7 @@ static int haf_plan_build(const int64_t* mat_off, const int32_t* k, const int32_
             meta.push_back(d.rad);
         for (const Dg& d : it.dg)
             meta.push_back(d.top);
+        // relative cost of a term, for the tasks' order
         const double per_term = loop ? (2.0 * J + 10.0 * (N / 2) + 12.0) : (2.0 * J + 24.0);
         for (int64_t q = 0; q < nt; ++q) {
             tasks.push_back(Task{(int32_t)b, (int32_t)q});

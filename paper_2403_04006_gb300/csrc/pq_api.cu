@@ -590,7 +590,7 @@ static cudaError_t forward_prepare(const pq_plan* P)
     if (P->fwd_nl != 0)
         return fwd_reg_prepare(std::max(P->fwd_nl, 0),
                                P->wpb * fwd_reg_smem_per_warp(P->kmax, P->fwd_ld));
-    return fwd_prepare(P->lmax, P->wpb * fwd_smem_per_warp(P->kmax, P->lmax));
+    return fwd_prepare(P->wpb * fwd_smem_per_warp(P->kmax, P->lmax));
 }
 
 static int schedule_and_upload(pq_plan* P)
@@ -612,10 +612,12 @@ static int schedule_and_upload(pq_plan* P)
     // Where the walk keeps its column sums.  Registers pay when every
     // permanent falls in one column class (4096 patterns of 12 photons in
     // m = 24: 194 us; one n = 30 permanent: 35.2 ms, 49.1 ms in shared
-    // memory).  A batch that mixes classes would run one instantiation per
-    // class in one kernel, with the registers of the widest and different code
-    // on the warps of one SM, so the planner takes shared memory there, and a
-    // caller may ask for either (PQ_SUMS_REGISTERS, PQ_SUMS_SHARED).
+    // memory).  A batch that mixes classes runs one instantiation per class in
+    // one kernel, with the registers of the widest and different code on the
+    // warps of one SM (65536 ragged permanents, n = 4..20: 11.6 ms against 5.77
+    // in shared memory; n = 4..10: 0.374 against 0.288), so the planner takes
+    // shared memory there, and a caller may ask for either (PQ_SUMS_REGISTERS,
+    // PQ_SUMS_SHARED).
     {
         int cls = 0;
         bool one = true;
@@ -645,7 +647,7 @@ static int schedule_and_upload(pq_plan* P)
     int wpb = 0, bps = 0;
     const int reg_class = std::max(P->fwd_nl, 0);
     launch_geometry(P->fwd_nl != 0 ? fwd_reg_regs_per_thread(reg_class)
-                                   : fwd_regs_per_thread(P->lmax),
+                                   : fwd_regs_per_thread(),
                     per_warp,
                     std::min(P->opts.warps_per_block > 0 ? P->opts.warps_per_block : 8,
                              P->fwd_nl != 0 ? fwd_reg_max_warps(reg_class) : 8),
@@ -1107,7 +1109,7 @@ static int run_forward_raw(pq_plan* P, const void* src, void* amps, double* prob
     // Where every permanent is one task and all of them are resident at once
     // there is nothing to count and no queue to keep: one warp per task, and no
     // reset of the counters before the kernel (330 patterns of 4 photons: 19.4 ->
-    // 18.1 us a call).  With more tasks than warps the queue is the faster of the
+    // 17.4 us a call).  With more tasks than warps the queue is the faster of the
     // two (42504 permanents of up to 5 photons: 162 us against 169).
     const bool direct = P->direct && P->opts.method == PQ_METHOD_BATCHED &&
                         (int64_t)P->tasks_plain_h.size() <= (int64_t)P->blocks * P->wpb;
@@ -1474,7 +1476,7 @@ static int ensure_backward(pq_plan* P)
             continue;
         BwdClass& C = cls[c];
         C.reg = bwdr_supported(C.ld) ? 1 : 0;
-        const int regs = C.reg ? bwdr_regs_per_thread(C.ld) : bwd_regs_per_thread(C.ld);
+        const int regs = C.reg ? bwdr_regs_per_thread(C.ld) : bwd_regs_per_thread();
         const double nbar = cls_terms[c] > 0 ? cls_nterms[c] / cls_terms[c] : 1.0;
         double best = -1.0;
         for (int J = kBwdMaxLowDigits; J >= 1; --J) {
@@ -1709,7 +1711,7 @@ static int ensure_backward(pq_plan* P)
     }
     P->bwd_jb = jb;
     P->bwd_n2 = n2;
-    cudaError_t e = bwd_prepare(P->lmax, max_smem);
+    cudaError_t e = bwd_prepare(max_smem);
     if (e != cudaSuccess)
         return fail(PQ_ERR_CUDA, "backward attribute setup failed: %s", cudaGetErrorString(e));
     if ((rc = uploads_done()) != PQ_OK)

@@ -167,15 +167,6 @@ __device__ __forceinline__ uint64_t high_binom(int top, int g)
     return binom_u64(top, g);
 }
 
-// C(top, g) in double (exact while it stays below 2^53).
-__device__ __forceinline__ double binom_f64(int top, int g)
-{
-    double r = 1.0;
-    for (int i = 1; i <= g; ++i)
-        r = r * (double)(top - g + i) / (double)i;
-    return r;
-}
-
 // ---------------------------------------------------------------- metadata views
 struct MetaView {
     const int32_t* ridx;

@@ -8,8 +8,8 @@ namespace pqi {
 
 // ---- forward (glynn_fwd.cu)
 int fwd_smem_per_warp(int kmax, int lmax);
-int fwd_regs_per_thread(int lmax);
-int bwd_regs_per_thread(int lmax);
+int fwd_regs_per_thread();
+int bwd_regs_per_thread();
 
 // Warps per block and resident blocks per SM that registers and shared
 // memory allow (65536 registers per SM, allocated per warp in units of 256;
@@ -58,7 +58,7 @@ inline void launch_geometry_max(int regs_per_thread, int smem_per_warp, int want
         }
     }
 }
-cudaError_t fwd_prepare(int lmax, int smem_bytes);
+cudaError_t fwd_prepare(int smem_bytes);
 cudaError_t fwd_launch_persistent(int lmax, const ExecArgs& a, int kmax, int blocks, int wpb,
                                   cudaStream_t st);
 cudaError_t fwd_launch_plain(int lmax, const ExecArgs& a, int64_t t_begin, int64_t t_end,
@@ -108,7 +108,7 @@ struct BwdArgs {
 int bwd_smem_bytes_for(int kmax, int lmax, int jb, int n2);
 constexpr int kBwdMaxLowDigits = 4;  // low digits the backward workspace holds
 constexpr int kBwdChunkLog2 = 7;     // backward chunks of at most 2^7 terms
-cudaError_t bwd_prepare(int lmax, int smem_bytes);
+cudaError_t bwd_prepare(int smem_bytes);
 cudaError_t bwd_launch_persistent(int ld, const BwdArgs& a, int64_t t_begin, int64_t t_end,
                                   int kmax, int jb, int n2, int blocks, int wpb, cudaStream_t st);
 cudaError_t bwd_launch_plain(int lmax, const BwdArgs& a, int64_t t_begin, int64_t t_end,

@@ -304,9 +304,9 @@ extern "C" int pq_permanent_noalloc(const pq_c128* B, int32_t k, int32_t l,
     const int kmax = h.desc.k > 0 ? h.desc.k : 1;
     const int per_warp = fwd_smem_per_warp(kmax, ld);
     int wpb = 0, bps = 0, sms = 0;
-    launch_geometry(fwd_regs_per_thread(ld), per_warp, 8, 8, wpb, bps);
+    launch_geometry(fwd_regs_per_thread(), per_warp, 8, 8, wpb, bps);
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        fwd_prepare(ld, wpb * per_warp) != cudaSuccess)
+        fwd_prepare(wpb * per_warp) != cudaSuccess)
         return noalloc_fail(PQ_ERR_CUDA, "kernel set-up failed");
     ExecArgs a;
     a.desc = desc_d;
