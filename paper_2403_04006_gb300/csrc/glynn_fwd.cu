@@ -10,7 +10,7 @@ namespace pqi {
 // the global counter until the range is exhausted (persistent launch of a
 // whole batch); queue == 0: warp w of block b takes task t_begin + b * wpb + w
 // (one launch per permanent, the plain method).
-__global__ void __launch_bounds__(256, 2) glynn_fwd_kernel(ExecArgs a, int64_t t_begin,
+__global__ void __launch_bounds__(256, 2) glynn_fwd_kernel(const __grid_constant__ ExecArgs a, int64_t t_begin,
                                                          int64_t t_end, int kmax, int ld,
                                                          int queue)
 {

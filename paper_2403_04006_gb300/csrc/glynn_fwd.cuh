@@ -25,7 +25,7 @@
 // A base matrix with a non-finite entry, or a column whose bound overflows, has
 // no such scale: its tasks walk in FP64 (fp64_walk), so that infinities and
 // NaNs propagate as FP64 arithmetic gives them.  Matrices whose columns all lie
-// near the real or imaginary axis have a unit for each part (other_walk), so that
+// near the real or imaginary axis have a unit for each part (other_task), so that
 // the small part keeps its bits: 16384 ragged permanents 2.03 ms (1.52 with parts
 // of like size, 5.34 for the FP64 walk), one n = 24 permanent 0.91 (0.60, 2.64).
 // A warp task is up to 32 chunks of one permanent (one per lane).  The lanes'
@@ -314,20 +314,25 @@ __device__ __forceinline__ void reweight(const LowWalk& wk, int J, double& wlow,
     wlow = (double)low_weight(wk, J);
 }
 
-// Write per = 2^{-(n-1)} * sum, and |per|^2 * norm, the sum being v with the powers
-// of two and of i of its staging; a sharded plan writes its unscaled
-// double-double sum instead.
-__device__ __forceinline__ void finalize(const ExecArgs& a, const PermDesc& D, dd2 v,
-                                         int exp2, int f, int turns)
+// Write per = 2^{-(n-1)} * sum, and |per|^2 * norm, the sum being v times 2^exp2, with
+// PARTS its imaginary part times 2^-f more and the whole times i^turns; a sharded plan
+// writes its unscaled double-double sum instead.
+template <bool PARTS>
+__device__ __forceinline__ void finalize(const ExecArgs& a, const PermDesc& D, dd2 v, int exp2,
+                                         int f, int turns)
 {
+    const int exp2_im = PARTS ? exp2 - f : exp2;
+    auto turned = [&](double re, double im) {
+        return PARTS ? turn(re, im, turns) : make_double2(re, im);
+    };
     if (a.out_partial) {
         double* o = a.out_partial + 4 * (int64_t)D.out;
         if (D.trivial) {
             o[0] = 1.0;
             o[1] = o[2] = o[3] = 0.0;
         } else {
-            const double2 h = turn(scalbn(v.rh, exp2), scalbn(v.ih, exp2 - f), turns);
-            const double2 e = turn(scalbn(v.rl, exp2), scalbn(v.il, exp2 - f), turns);
+            const double2 h = turned(scalbn(v.rh, exp2), scalbn(v.ih, exp2_im));
+            const double2 e = turned(scalbn(v.rl, exp2), scalbn(v.il, exp2_im));
             o[0] = h.x;
             o[1] = e.x;
             o[2] = h.y;
@@ -337,8 +342,8 @@ __device__ __forceinline__ void finalize(const ExecArgs& a, const PermDesc& D, d
     }
     double2 per = make_double2(1.0, 0.0);
     if (!D.trivial)
-        per = turn(scale_exp2(__dadd_rn(v.rh, v.rl), exp2 + 1 - D.n),
-                   scale_exp2(__dadd_rn(v.ih, v.il), exp2 - f + 1 - D.n), turns);
+        per = turned(scale_exp2(__dadd_rn(v.rh, v.rl), exp2 + 1 - D.n),
+                     scale_exp2(__dadd_rn(v.ih, v.il), exp2_im + 1 - D.n));
     if (a.out_amp)
         a.out_amp[D.out] = per;
     if (a.out_prob)
@@ -379,6 +384,7 @@ __device__ __forceinline__ dd2 task_sum(double rh, double rl, double ih, double 
 // The task's sum res (the same on every lane) goes to the permanent's output
 // if the permanent has one task; otherwise to its slot, and the warps that
 // finish last add the slots (gather_partials).
+template <bool PARTS>
 static __device__ void combine_task(const ExecArgs& a, const Task& t, const PermDesc& D, dd2 res,
                                     int exp2, int f, int turns, int lane)
 {
@@ -386,7 +392,7 @@ static __device__ void combine_task(const ExecArgs& a, const Task& t, const Perm
                         a.groups + D.gslot0, t.part - D.part0, D.ntasks, res.rh, res.rl, res.ih,
                         res.il, lane) &&
         lane == 0)
-        finalize(a, D, res, exp2, f, turns);
+        finalize<PARTS>(a, D, res, exp2, f, turns);
 }
 
 // ---------------------------------------------------------------- the walk
@@ -618,40 +624,43 @@ static __device__ dd2 fp64_walk(const PermDesc& D, const MetaView& mv, const War
     return task_sum(rh, rl, ih, il, whigh_u, (gpar & 1) != 0, active);
 }
 
-// The sum of a walk off the main path; the imaginary part is to be taken times 2^-f,
-// and the whole times i^turns.
-struct WalkSum {
-    dd2 v;
-    int f, turns;
-};
-
-// The walks of matrices that are not staged as integers of one unit.  Not inlined,
-// and called with what it cannot read again, so that the main path keeps no object
-// in memory for it.
-static __device__ __noinline__ WalkSum other_walk(const PermDesc* desc, const int32_t* meta,
-                                                  longlong2* M, longlong2* base, int32_t* lowrow,
-                                                  int ld, int mode, uint32_t emask, int64_t chunk,
-                                                  bool active, int lane)
+// The tasks of a permanent that is not staged as integers of one unit: the whole
+// rest of the task, so that the main path keeps nothing for it (with the walks
+// alone called and their sum combined on the main path, a class at its register
+// limit spilled more: one n = 26 permanent 1.98 -> 2.26 ms).
+static __device__ __noinline__ void other_task(const ExecArgs& a, Task t, longlong2* M,
+                                               longlong2* base, int32_t* lowrow, int ld, int mode,
+                                               int exp2, uint32_t emask, int lane)
 {
-    const PermDesc D = *desc;
-    const MetaView mv = meta_view(meta, D);
+    const PermDesc D = a.desc[t.perm];
+    const MetaView mv = meta_view(a.meta, D);
     const WarpSmem sm(M, base, lowrow, ld);
-    WalkSum r;
-    r.f = r.turns = 0;
+    const int64_t chunk0 = (int64_t)t.part * kWarp;
+    const bool active = chunk0 + lane < D.nchunks;
+    const int64_t chunk = active ? (chunk0 + lane) : 0;
     if (mode == kStagedFp64) {
-        r.v = fp64_walk(D, mv, sm, chunk, active);
-        return r;
+        const dd2 res = fp64_walk(D, mv, sm, chunk, active);
+        combine_task<false>(a, t, D, res, exp2, 0, 0, lane);
+        return;
     }
-    // column sums in local memory
+    // a unit for each part; column sums in local memory
     longlong2 S[PQ_MAX_PRODUCT_COLS];
-    r.f = sscale_of(sm.cexp[0]).f;
+    const int f = sscale_of(sm.cexp[0]).f;
+    int turns = 0;
     for (int j = 0; j < D.l; ++j)
-        r.turns += sscale_of(sm.cexp[j]).turned ? mv.cmul[j] : 0;
-    const PartUnits mul{min(63, 2 * r.f)};
-    r.v = D.jf < 0 ? int_walk<0, true, 1>(mul, S, D, mv, sm, emask, chunk, active, lane)
-                   : int_walk<0, false, 1>(mul, S, D, mv, sm, emask, chunk, active, lane);
-    return r;
+        turns += sscale_of(sm.cexp[j]).turned ? mv.cmul[j] : 0;
+    const PartUnits mul{min(63, 2 * f)};
+    const dd2 res = D.jf < 0 ? int_walk<0, true, 1>(mul, S, D, mv, sm, emask, chunk, active, lane)
+                             : int_walk<0, false, 1>(mul, S, D, mv, sm, emask, chunk, active, lane);
+    combine_task<true>(a, t, D, res, exp2, f, turns, lane);
 }
+
+// Whether the end of a task reads the descriptor again, so that the walk does not
+// hold it in registers: in the classes whose registers are short.  Held / read again:
+// n = 26 permanent 2.20 / 1.94 ms, 28 8.78 / 8.58, 30 35.7 / 35.4, 4096 patterns of 12
+// photons 195.5 / 193.7 us; but class 24 0.593 / 0.608 ms and, in shared memory, 65536
+// ragged permanents 5.74 / 5.80.
+constexpr bool fwd_reads_again(int nl) { return nl > 0 && nl != 24; }
 
 template <int NL>
 __device__ __forceinline__ void process_task(const ExecArgs& a, const Task& t, WarpSmem& sm,
@@ -660,29 +669,31 @@ __device__ __forceinline__ void process_task(const ExecArgs& a, const Task& t, W
     const PermDesc D = a.desc[t.perm];
     const MetaView mv = meta_view(a.meta, D);
     dd2 res = {0.0, 0.0, 0.0, 0.0};
-    int f = 0, turns = 0;
     if (!D.trivial) {
         if (st.perm != t.perm) {
             __syncwarp();
             stage_perm(a, D, mv, sm, st, lane);
             st.perm = t.perm;
         }
+        if (st.mode != kStagedInt) {
+            other_task(a, t, sm.M, sm.base, sm.lowrow, sm.ld, st.mode, st.exp2, st.emask, lane);
+            return;
+        }
         const int64_t chunk0 = (int64_t)t.part * kWarp;
         const bool active = chunk0 + lane < D.nchunks;
         const int64_t chunk = active ? (chunk0 + lane) : 0;
-        if (st.mode != kStagedInt) {
-            const WalkSum r = other_walk(a.desc + t.perm, a.meta, sm.M, sm.base, sm.lowrow, sm.ld,
-                                         st.mode, st.emask, chunk, active, lane);
-            res = r.v;
-            f = r.f;
-            turns = r.turns;
-        } else if (D.jf < 0) {
+        if (D.jf < 0)
             res = int_walk<NL, true>(OneUnit(), sm.S + lane, D, mv, sm, st.emask, chunk, active, lane);
-        } else {
+        else
             res = int_walk<NL, false>(OneUnit(), sm.S + lane, D, mv, sm, st.emask, chunk, active, lane);
-        }
     }
-    combine_task(a, t, D, res, st.exp2, f, turns, lane);
+    if (fwd_reads_again(NL)) {
+        asm volatile("" ::: "memory");
+        const PermDesc E = a.desc[t.perm];
+        combine_task<false>(a, t, E, res, st.exp2, 0, 0, lane);
+    } else {
+        combine_task<false>(a, t, D, res, st.exp2, 0, 0, lane);
+    }
 }
 
 // Task ti of the list, once its guards pass (a failing task is skipped and
@@ -717,7 +728,8 @@ __device__ __forceinline__ void run_task(const ExecArgs& a, int64_t ti, WarpSmem
 constexpr int fwd_reg_blocks(int nl) { return nl <= 6 ? 5 : nl <= 14 ? 4 : nl <= 26 ? 3 : 2; }
 
 template <int NL>
-__global__ void __launch_bounds__(128, fwd_reg_blocks(NL)) glynn_fwd_reg_kernel(ExecArgs a, int64_t t_begin,
+__global__ void __launch_bounds__(128, fwd_reg_blocks(NL)) glynn_fwd_reg_kernel(const __grid_constant__ ExecArgs a,
+                                                             int64_t t_begin,
                                                              int64_t t_end, int kmax, int ld,
                                                              int queue)
 {

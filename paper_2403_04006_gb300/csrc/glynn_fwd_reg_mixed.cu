@@ -6,7 +6,8 @@ namespace pqi {
 
 // All column classes in one persistent launch: each task runs the
 // instantiation of its own class.
-__global__ void __launch_bounds__(256, 2) glynn_fwd_reg_mixed_kernel(ExecArgs a, int64_t t_begin,
+__global__ void __launch_bounds__(256, 2) glynn_fwd_reg_mixed_kernel(const __grid_constant__ ExecArgs a,
+                                                                     int64_t t_begin,
                                                                      int64_t t_end, int kmax,
                                                                      int ld, int queue)
 {
