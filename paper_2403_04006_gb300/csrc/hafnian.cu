@@ -398,7 +398,7 @@ __device__ __noinline__ dd2 haf_walk_fp64(const HafDesc& D, const HafMeta& mt, c
 }
 
 // Whether the terms of an item can lie near an axis (pq_blockint.cuh): b the parts
-// of the entries that q takes, g those of the loop weights, root the exponent of
+// of the entries, g those of the loop weights, root the exponent of
 // the loop polynomial's largest root (its first factor is q + 2^root l^2 or so).
 // q^n is near an axis where q is; a factor of the loop polynomial where the larger
 // of its two terms' parts are far apart, and N = 1 leaves l alone.
@@ -432,12 +432,11 @@ __device__ __forceinline__ int unit_scale(const BParts& m)
 // weights times 2^t, which multiplies every term by 2^(t N) and keeps the powers in
 // range.  Returns t.
 __device__ __noinline__ int haf_scale(const HafSmem& sm, int k, const BParts& b, const BParts& g,
-                                      uint32_t hmax, int lane)
+                                      int lane)
 {
     int t = b.no_re() && b.no_im() ? 1 << 20 : unit_scale(b) >> 1;
     if (!g.no_re() || !g.no_im())
         t = min(t, unit_scale(g));
-    t = min(t, (1023 + 900 - bint_exponent(hmax)) >> 1);  // all entries stay finite
     for (int e = lane; e < k * k; e += kWarp)
         sm.M[e] = make_double2(scalbn(sm.M[e].x, 2 * t), scalbn(sm.M[e].y, 2 * t));
     for (int i = lane; i < k; i += kWarp)
@@ -471,20 +470,20 @@ __device__ __forceinline__ int haf_part_scale(const HafMeta& mt, const HafSmem& 
 // A hafnian near an axis: M = 2 b with a unit for each part, divided by i where the
 // imaginary part is the larger.  False if a part has no scale (subnormal).
 __device__ __noinline__ bool haf_stage_parts(const HafMeta& mt, const HafSmem& sm, int k,
-                                             const BParts& all, SScale& s, int lane)
+                                             const BParts& b, SScale& s, int lane)
 {
-    if (min(all.re, all.im) < 0x100000u)
+    if (min(b.re, b.im) < 0x100000u)
         return false;
-    s.turned = bint_exponent(all.im) > bint_exponent(all.re);
-    const int big = haf_part_scale(mt, sm, k, s.turned, max(all.re, all.im), lane);
-    const int small = haf_part_scale(mt, sm, k, !s.turned, min(all.re, all.im), lane);
+    s.turned = bint_exponent(b.im) > bint_exponent(b.re);
+    const int big = haf_part_scale(mt, sm, k, s.turned, max(b.re, b.im), lane);
+    const int small = haf_part_scale(mt, sm, k, !s.turned, min(b.re, b.im), lane);
     s.e = min(big, small);
     s.f = small - s.e;
     longlong2* M = reinterpret_cast<longlong2*>(sm.M);
     for (int e = lane; e < k * k; e += kWarp) {
-        const double2 b = sm.M[e];
-        M[e] = make_longlong2(2 * bint_of(s.turned ? b.y : b.x, s.e),
-                              2 * bint_of(s.turned ? -b.x : b.y, s.e + s.f));
+        const double2 v = sm.M[e];
+        M[e] = make_longlong2(2 * bint_of(s.turned ? v.y : v.x, s.e),
+                              2 * bint_of(s.turned ? -v.x : v.y, s.e + s.f));
     }
     __syncwarp();
     return true;
@@ -509,15 +508,11 @@ __device__ bool haf_stage_int(const HafDesc& D, const HafMeta& mt, const HafSmem
     st.mode = kStagedInt;
     st.exp2 = 0;
     bool bad = false;
-    BParts all, b, g;  // b: without the diagonal entries of single indices, which q cancels
-    for (int e = lane; e < k * k; e += kWarp) {
-        const int i = e / k;
-        all.add(sm.M[e].x, sm.M[e].y);
-        if (e != i * k + i || mt.rmul[i] > 1)
-            b.add(sm.M[e].x, sm.M[e].y);
-    }
+    BParts b, g;
+    for (int e = lane; e < k * k; e += kWarp)
+        b.add(sm.M[e].x, sm.M[e].y);
     warp_parts(b);
-    const uint32_t hmax = __reduce_max_sync(0xffffffffu, max(all.re, all.im));
+    const uint32_t hmax = max(b.re, b.im);
     uint32_t gmax = 0;
     // |q| <= 1/2 (sum_ij r_i r_j |b_ij| + sum_i r_i |b_ii|)
     uint64_t units = 0;
@@ -555,11 +550,10 @@ __device__ bool haf_stage_int(const HafDesc& D, const HafMeta& mt, const HafSmem
     SScale ps{eq, 0, false};
     if (haf_near_axis<LOOP>(b, g, D.N, root)) {
         if (LOOP) {
-            st.exp2 = -haf_scale(sm, k, b, g, hmax, lane) * D.N;
+            st.exp2 = -haf_scale(sm, k, b, g, lane) * D.N;
             return false;
         }
-        warp_parts(all);
-        if (!haf_stage_parts(mt, sm, k, all, ps, lane))
+        if (!haf_stage_parts(mt, sm, k, b, ps, lane))
             return false;
         st.mode = kStagedParts;
         if (lane == 0)
@@ -955,7 +949,12 @@ __device__ void haf_task(const HafArgs& a, const Task& t, const HafSmem& sm, Haf
             __syncwarp();
             for (int e = lane; e < k * k; e += kWarp) {
                 const int i = e / k, j = e - i * k;
-                sm.M[e] = a.src[D.src_off + (int64_t)mt.ridx[i] * D.ld + mt.ridx[j]];
+                double2 b = a.src[D.src_off + (int64_t)mt.ridx[i] * D.ld + mt.ridx[j]];
+                // q cancels the diagonal entry of a single index (x_i^2 = r_i = 1): left
+                // out, so that a large one takes no bits from the others
+                if (i == j && mt.rmul[i] == 1 && !not_finite(b.x) && !not_finite(b.y))
+                    b = make_double2(0.0, 0.0);
+                sm.M[e] = b;
             }
             if (LOOP) {
                 const int nf = D.N / 2 + 1;

@@ -213,6 +213,38 @@ def haf_items(seed):
 
 
 @pytest.mark.parametrize("loop", [False, True])
+def test_diagonal_of_single_indices(dev, loop):
+    """An index that occurs once has no pair with itself: its diagonal entry, however
+    large, takes nothing from the result (32 N 2^-53 of the majorants of the matrix
+    without these entries), unless it is not finite."""
+    rng = np.random.default_rng(18)
+    items = []
+    for size in (1e6, 1e6j, 1e40, -1e40j, 1e300 + 1e300j):
+        for k, r in ((2, [1, 1]), (4, [1, 1, 1, 1]), (3, [1, 2, 1]), (4, [2, 1, 1, 2])):
+            B = rng.standard_normal((k, k)) + 1j * rng.standard_normal((k, k))
+            B = (B + B.T) / 2
+            free = B.copy()
+            for i in range(k):
+                if r[i] == 1:
+                    B[i, i], free[i, i] = size * (1.0 + i), 0
+            items.append((B, free, r, rng.standard_normal(k) + 1j * rng.standard_normal(k)))
+    ks = np.array([B.shape[0] for B, _, _, _ in items], dtype=np.int32)
+    mo = np.concatenate([[0], np.cumsum(ks.astype(np.int64) ** 2)[:-1]])
+    ro = np.concatenate([[0], np.cumsum(ks, dtype=np.int64)[:-1]])
+    mats = torch.from_numpy(np.concatenate([B.reshape(-1) for B, _, _, _ in items])).to(dev)
+    gam = torch.from_numpy(np.concatenate([g for _, _, _, g in items])).to(dev)
+    rep = np.concatenate([r for _, _, r, _ in items]).astype(np.int32)
+    got = api.hafnian_repeated(mats, mo, ks, rep, ro, gamma=gam if loop else None).cpu().numpy()
+    for q, ((_, B, r, g), v) in enumerate(zip(items, got)):
+        g = g if loop else None
+        idx = [i for i, x in enumerate(r) for _ in range(x)]
+        assert parts_ok(v, exact_haf(B, g, idx), haf_majorant(B, g, r), 32 * sum(r) * 2.0 ** -53), (q, v)
+    mats[0] = float("inf")
+    got = api.hafnian_repeated(mats, mo, ks, rep, ro, gamma=gam if loop else None).cpu().numpy()
+    assert not np.isfinite(got[0])
+
+
+@pytest.mark.parametrize("loop", [False, True])
 def test_hafnians(dev, loop):
     """32 N 2^-53 of the majorants: N products, the updates of q and l, and the
     accumulation."""
